@@ -259,7 +259,9 @@ ka_status ka_layered_graph(int32_t d, int32_t L, int32_t M, uint64_t graph_seed,
 /* Kernel timing for roofline reports.  When enabled, ka_sweep brackets
  * every sweep-kernel launch with CUDA events on the context stream (the
  * events sit between launches that would otherwise overlap their prologues,
- * so the times are those of launches run one after the other).
+ * so the times are those of launches run one after the other; small
+ * topologies, whose sweeps otherwise run in one launch per call on chip, take
+ * a launch per group or class meanwhile).
  * ka_profile_read synchronises and returns the summed kernel time (ms) and
  * the number of launches since the last read; ka_profile_read_dirs returns
  * the same split by bond direction: host arrays kernel_ms[4] and

@@ -21,7 +21,7 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
   size_t n, n0, p, stage, counts, hist, pre_key, pre_idx, krem, unresolved, err, nbr, bu, bv, bid,
-      perm, inv, total;
+      perm, inv, rec, coff, total;
 };
 
 struct Shape {
@@ -113,6 +113,10 @@ Layout layout_of(const Shape& s) {
   if (s.topo != KA_CUBIC) {
     l.perm = take((size_t)s.N * sizeof(int32_t));
     l.inv = take((size_t)s.N * sizeof(int32_t));
+    if (ka::resident::graph_fits(s.N)) {
+      l.rec = take((size_t)s.E * ka::resident::graph_record_bytes(s.z));
+      l.coff = take((ka::resident::kMaxClasses + 1) * sizeof(int32_t));
+    }
   }
   l.total = off;
   return l;
@@ -176,6 +180,7 @@ ka_status create_common(const ka_params* params, void* buf, size_t bytes, bool o
   c->is.krem = (int64_t*)(base + l.krem);
   c->is.unresolved = (int32_t*)(base + l.unresolved);
   c->is.cand = c->stage ? (uint32_t*)c->stage : nullptr;  // idle during init
+  cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, params->device);
   c->is.cand_bytes = c->stage ? (size_t)s.N * s.W * sizeof(uint64_t) : 0;
 
   {
@@ -218,11 +223,22 @@ ka_status create_common(const ka_params* params, void* buf, size_t bytes, bool o
     // index order.
     std::vector<int32_t> perm, inv, nbr_d, bu_d, bv_d;
     std::vector<uint32_t> bid_d;
+    std::vector<uint16_t> rec;
+    std::vector<int32_t> coff;
     if (s.topo != KA_CUBIC) {
       ka::bfs_order(s.N, s.z, c->host.nbr.data(), perm, inv);
       ka::relabel_tables(c->host, s.z, perm, nbr_d, bu_d, bv_d, bid_d);
       c->g.perm = (const int32_t*)(base + l.perm);
       c->pl.inv = (const int32_t*)(base + l.inv);
+      if (ka::resident::graph_fits(s.N) && c->nclass <= ka::resident::kMaxClasses) {
+        rec.resize((size_t)s.E * ka::resident::graph_record_bytes(s.z) / sizeof(uint16_t));
+        ka::resident::graph_records(s.N, s.z, nbr_d.data(), bu_d.data(), bv_d.data(), s.E, rec.data());
+        coff.assign(c->host.class_off.begin(), c->host.class_off.end());
+        for (int64_t k = 0; k < c->nclass; ++k)
+          c->class_max = std::max(c->class_max, c->host.class_off[k + 1] - c->host.class_off[k]);
+        c->rec = (const uint4*)(base + l.rec);
+        c->coff = (const int32_t*)(base + l.coff);
+      }
     } else {
       nbr_d = c->host.nbr;
       bu_d = c->host.bu;
@@ -243,6 +259,12 @@ ka_status create_common(const ka_params* params, void* buf, size_t bytes, bool o
     if (!e && c->pl.inv)
       e = cudaMemcpyAsync((void*)c->pl.inv, inv.data(), inv.size() * 4, cudaMemcpyHostToDevice,
                           c->stream);
+    if (!e && c->rec)
+      e = cudaMemcpyAsync((void*)c->rec, rec.data(), rec.size() * sizeof(uint16_t),
+                          cudaMemcpyHostToDevice, c->stream);
+    if (!e && c->rec)
+      e = cudaMemcpyAsync((void*)c->coff, coff.data(), coff.size() * sizeof(int32_t),
+                          cudaMemcpyHostToDevice, c->stream);
     if (!e) e = cudaStreamSynchronize(c->stream);
     if (e) {
       if (owns) cudaFree(buf);
@@ -314,6 +336,31 @@ ka_status check_device_error(ka_ctx* c) {
 }  // namespace
 
 namespace ka {
+int resident_cluster(const ka_ctx* c, int64_t words) {
+  if (c->topo == KA_CUBIC)
+    return c->pencil && c->pl.V == 1 ? resident::cubic_cluster(c->d, c->L, words, c->sms) : 0;
+  return c->rec ? resident::graph_cluster(c->N, c->nbonds, c->class_max, words, c->sms) : 0;
+}
+
+resident::Unit resident_unit(const ka_ctx* c, int w, uint32_t t0, uint32_t count) {
+  resident::Unit u{};
+  const size_t at = (size_t)(w / c->pl.V) * c->pl.plane_elems() + (size_t)(w % c->pl.V);
+  u.n = c->pl.n + at;
+  u.p = c->pl.p + at;
+  u.rec = c->rec;
+  u.bid = c->g.bid;
+  u.coff = c->coff;
+  u.err = c->err_dev;
+  u.N = (int32_t)c->N;
+  u.nclass = (int32_t)c->nclass;
+  u.stride = c->pl.V;
+  u.t_base = t0;
+  u.count = count;
+  u.word = (uint32_t)w;
+  u.rk = c->rk;
+  return u;
+}
+
 ka_status create_context(const ka_params* params, void* buf, size_t bytes, bool owns, ka_ctx** out) {
   return create_common(params, buf, bytes, owns, out);
 }
@@ -397,7 +444,22 @@ ka_status ka_sweep(ka_ctx* c, int64_t n) {
   if (n == 0) return KA_OK;
   DeviceGuard dg(c->device);
   cudaError_t e = cudaSuccess;
-  if (c->pencil && ka::stream_preferred(c->d, c->L, c->pl.P)) {
+  // profiling times one group or class per launch
+  const int C = c->prof ? 0 : ka::resident_cluster(c, c->pl.W);
+  if (C) {
+    ka::resident::Args a{};
+    a.plane_elems = c->pl.plane_elems();
+    a.words_per_plane = c->pl.V;
+    a.most = (uint32_t)ka::resident::kMaxSweeps;
+    for (int64_t s = 0; s < n && !e; s += ka::resident::kMaxSweeps) {
+      a.one = ka::resident_unit(c, 0, (uint32_t)(c->sweep + s),
+                                (uint32_t)std::min(ka::resident::kMaxSweeps, n - s));
+      e = c->topo == KA_CUBIC
+              ? ka::resident::launch_cubic(a, c->d, c->L, c->m, (unsigned)c->pl.W, C, c->stream)
+              : ka::resident::launch_graph(a, c->N, c->nbonds, c->class_max, c->z, c->m,
+                                           (unsigned)c->pl.W, C, c->stream);
+    }
+  } else if (c->pencil && ka::stream_preferred(c->d, c->L, c->pl.P)) {
     // plane-outer order keeps the planes of one launch resident in the L2
     // across sweeps
     const int nq = ka::stream_planes_per_launch(c->L, c->pl.P);

@@ -5,6 +5,7 @@
 #include <vector>
 
 #include "ka_internal.cuh"
+#include "ka_resident.cuh"
 
 struct ka_ctx {
   ka_params prm;
@@ -22,6 +23,10 @@ struct ka_ctx {
   int* err_dev = nullptr;  // device error word of bounded device waits (0 = none)
   uint64_t* stage = nullptr;
   ka::GraphDev g{};
+  const uint4* rec = nullptr;       // small graphs: packed bonds and class offsets (ka_resident.cuh)
+  const int32_t* coff = nullptr;
+  int64_t class_max = 0;            // bonds of the largest class
+  int sms = 0;
   ka::Topology host;  // class offsets (graphs) and tables for inspection
   bool initialized = false;
   int64_t sweep = 0, K = -1;
@@ -40,6 +45,11 @@ struct ka_ctx {
 namespace ka {
 // Creates a context in a caller-provided (or owned) device buffer; defined in ka_api.cu.
 ka_status create_context(const ka_params* params, void* buf, size_t bytes, bool owns, ka_ctx** out);
+// Whether the sweeps of a context stay on chip (ka_resident.cuh), with `words`
+// words in the launch: the CTAs per word, or 0; and word w's unit for the
+// sweeps t0 .. t0 + count - 1.  Defined in ka_api.cu.
+int resident_cluster(const ka_ctx* c, int64_t words);
+resident::Unit resident_unit(const ka_ctx* c, int w, uint32_t t0, uint32_t count);
 // Device bytes a context needs; defined in ka_api.cu.
 ka_status context_bytes(const ka_params* params, size_t* bytes);
 }  // namespace ka

@@ -1,0 +1,8 @@
+// ka_resident_cubic_d3.cu -- on-chip cubic sweeps of dimension 3.
+#include "ka_resident_cubic.cuh"
+
+namespace ka {
+namespace resident {
+template cudaError_t launch_cubic_d<3>(const Args&, int, int, unsigned, int, cudaStream_t);
+}  // namespace resident
+}  // namespace ka

@@ -1,0 +1,301 @@
+// ka_resident_graph.cu -- on-chip sweeps of small graphs (ka_resident.cuh):
+// one cluster per word, one launch for all sweeps of a call.
+//
+// A bond's packed record holds the 16-bit positions of u, v and of their
+// other neighbours (missing ones point at a word that stays 0), so a class
+// needs one coalesced 16- or 32-byte load and the bond id per bond.  A thread
+// takes one bond of a class; its record is loaded two classes ahead and its
+// gate word computed one class ahead, while the group end is waited for.  The
+// gathers of a bond are shared-memory reads.
+//
+// The CTAs of a cluster send a bond's swap word as one entry of a buffer in
+// class order, and the receiver applies it to its copy: sent to their scattered
+// sites, the new words cost about two cycles each at the receiver (N = 2^14,
+// four CTAs: 3.0 us a class).
+#include <algorithm>
+
+#define KA_RESIDENT_DEVICE
+#include "ka_resident.cuh"
+
+namespace ka {
+namespace resident {
+namespace {
+
+// (c2 c1 c0) += x, bit-sliced; the count stays below 8 (at most 7 inputs)
+__device__ __forceinline__ void add3(uint64_t& c2, uint64_t& c1, uint64_t& c0, uint64_t x) {
+  const uint64_t k0 = c0 & x;
+  c0 ^= x;
+  const uint64_t k1 = c1 & k0;
+  c1 ^= k0;
+  c2 |= k1;
+}
+
+// [count <= M] of Z - 1 words at the given positions
+template <int Z, int M>
+__device__ __forceinline__ uint64_t at_most(const uint64_t* n, const uint32_t (&r)[Z], int from) {
+  uint64_t c2 = 0, c1 = 0, c0 = 0;
+#pragma unroll
+  for (int k = 0; k < Z - 1; ++k) {
+    const int e = from + k;
+    add3(c2, c1, c0, n[(r[e >> 1] >> (16 * (e & 1))) & 0xFFFFu]);
+  }
+  if constexpr (M >= Z - 1) {
+    return ~0ull;
+  } else {
+    const uint64_t g0 = (M & 1) ? 0ull : c0;
+    const uint64_t g1 = (M & 2) ? (c1 & g0) : (c1 | g0);
+    return ~((M & 4) ? (c2 & g1) : (c2 | g1));
+  }
+}
+
+// Z = 4 (records of 16 bytes, z <= 4) or 8 (32 bytes)
+template <int Z, int M, int C, bool B>
+__global__ void __launch_bounds__(1024) k_resident_graph(const __grid_constant__ Args a) {
+  constexpr int RW = Z / 4;  // 16-byte pieces of a record
+  extern __shared__ __align__(16) unsigned char dsm[];
+  __shared__ Unit su;
+  // class c: bonds [coff[c], coff[c + 1]), share[c] of them per CTA at most; the
+  // swapped bits of this CTA's are kept from slot[c] on
+  __shared__ int32_t coff[kMaxClasses + 1], share[kMaxClasses], slot[kMaxClasses];
+  __shared__ __align__(8) uint64_t bars[2];
+  const uint32_t rank = cluster_rank();
+  unit_of<B>(a, blockIdx.x / C, su);
+  uint32_t t = su.t_base + a.from, left_to_run = su.count > a.from ? min(su.count - a.from, a.most) : 0u;
+  if (left_to_run == 0) return;  // the whole cluster: one unit
+  const int N = su.N, nclass = su.nclass, tid = threadIdx.x;
+  // two entry buffers (C > 1), n, the swapped bits of this CTA's bonds (if fsmem)
+  uint64_t* buf = reinterpret_cast<uint64_t*>(dsm);
+  uint64_t* n = buf + 2 * a.entries;
+  uint64_t* f = n + N + 2;
+  const bool fsmem = a.fsmem != 0;
+  const Peers<C> peers(smem_addr(dsm), rank);
+  GroupEnd ge{smem_addr(bars), 0u, false};
+  if (tid < 2) bar_init(ge.bars + 8 * tid, blockDim.x / 32);
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  for (int c = tid; c <= nclass; c += blockDim.x) {
+    coff[c] = su.coff[c];
+    if (c < nclass) share[c] = (su.coff[c + 1] - su.coff[c] + C - 1) / C;
+  }
+  load_plane(su, n, N);
+  if (tid == 0) n[N] = 0;  // the word of missing neighbours
+  __syncthreads();
+  if (tid == 0) {
+    int at = 0;
+    for (int c = 0; c < nclass; ++c) {
+      slot[c] = at;
+      at += share[c];
+    }
+  }
+  if (fsmem)
+    for (int i = tid; i < a.fslots; i += blockDim.x) f[i] = 0;
+  // how many bonds of class c CTA r has, and their first
+  auto first = [&](int c, int r) { return coff[c] + r * share[c]; };
+  auto mine = [&](int c, int r) {
+    return max(0, min(share[c], coff[c + 1] - first(c, r)));
+  };
+
+  const uint32_t word = su.word;
+  uint32_t r[Z], rn[Z], id = 0;  // the records of this class and the next, the next one's id
+  uint32_t uv[C > 1 ? C - 1 : 1];  // the ends of the bonds whose entries this thread puts in place
+  uint64_t g = 0;
+  bool live = false, live_n = false;
+  auto fetch = [&](int c) {  // the record and id of this thread's bond of class c
+    live_n = tid < mine(c, (int)rank);
+    if (live_n) {
+      const int k = first(c, (int)rank) + tid;
+      const uint4* src = su.rec + (size_t)RW * k;
+#pragma unroll
+      for (int h = 0; h < RW; ++h) {
+        const uint4 x = __ldg(src + h);
+        rn[4 * h] = x.x;
+        rn[4 * h + 1] = x.y;
+        rn[4 * h + 2] = x.z;
+        rn[4 * h + 3] = x.w;
+      }
+      id = __ldg(su.bid + k);
+    }
+  };
+  auto ends = [&](int c) {  // entry tid of every other CTA's share of class c
+#pragma unroll
+    for (int d = 0; d < C - 1; ++d) {
+      const int o = (int)((rank + 1 + d) % C);
+      if (tid < mine(c, o))
+        uv[d] = __ldg(reinterpret_cast<const uint32_t*>(su.rec + (size_t)RW * (first(c, o) + tid)));
+    }
+  };
+  // the fetched class c becomes the current one: its gate words; the next is fetched
+  auto turn = [&](uint32_t tt, int c) {
+    live = live_n;
+#pragma unroll
+    for (int h = 0; h < Z; ++h) r[h] = rn[h];
+    const uint32_t e = id;
+    fetch(c + 1 < nclass ? c + 1 : 0);
+    const uint4 b = philox(make_uint4(tt, (uint32_t)c, e, word >> 1), unit_keys<B>(a, su));
+    g = (word & 1u) ? hi64(b) : lo64(b);
+  };
+  cluster_arrive();
+  fetch(0);
+  turn(t, 0);
+  ends(0);
+  cluster_wait();
+  for (; left_to_run; --left_to_run, ++t) {
+#pragma unroll 1
+    for (int c = 0; c < nclass; ++c) {
+      uint64_t sw = 0;
+      const int u = (int)(r[0] & 0xFFFFu), v = (int)(r[0] >> 16);
+      uint64_t* in = buf + (ge.phase & 1u) * a.entries;
+      const bool act = live;
+      if (act) {
+        const uint64_t nu = n[u], nv = n[v];
+        sw = (nu ^ nv) & g & at_most<Z, M>(n, r, 2) & at_most<Z, M>(n, r, 2 + Z - 1);
+        n[u] = nu ^ sw;
+        n[v] = nv ^ sw;
+        if constexpr (C > 1)
+          peers.st(smem_addr(in + first(c, (int)rank) - coff[c] + tid), sw, ge.bar());
+      }
+      ge.arrive((uint32_t)(coff[c + 1] - coff[c] - mine(c, (int)rank)) * 8u);
+      if (act) {
+        if (fsmem) {
+          f[slot[c] + tid] |= sw;
+        } else {
+          clear_bits(su.p + (size_t)u * su.stride, sw);
+          clear_bits(su.p + (size_t)v * su.stride, sw);
+        }
+      }
+      const int cn = c + 1 < nclass ? c + 1 : 0;
+      turn(cn ? t : t + 1, cn);
+      ge.wait(su.err);
+      if constexpr (C > 1) {
+#pragma unroll
+        for (int d = 0; d < C - 1; ++d) {
+          const int o = (int)((rank + 1 + d) % C);
+          if (tid < mine(c, o)) {
+            const uint64_t e = in[o * share[c] + tid];
+            n[uv[d] & 0xFFFFu] ^= e;
+            n[uv[d] >> 16] ^= e;
+          }
+        }
+        ends(cn);
+        __syncthreads();
+      }
+    }
+  }
+  store_plane(su, n, N, rank, C);
+  if (fsmem) {
+    for (int c = 0; c < nclass; ++c) {
+      if (tid >= mine(c, (int)rank)) continue;
+      const uint32_t e =
+          *reinterpret_cast<const uint32_t*>(su.rec + (size_t)RW * (first(c, (int)rank) + tid));
+      const uint64_t sw = f[slot[c] + tid];
+      clear_bits(su.p + (size_t)(e & 0xFFFFu) * su.stride, sw);
+      clear_bits(su.p + (size_t)(e >> 16) * su.stride, sw);
+    }
+  }
+  cluster_arrive();  // a CTA stays until the others have sent it all
+  cluster_wait();
+}
+
+template <int Z, int M>
+cudaError_t launch_m(const Args& a, unsigned words, int C, int threads, size_t smem, cudaStream_t st) {
+  const bool b = a.units != nullptr;
+  switch (C) {
+#define KA_C(CC)                                                                              \
+  case CC:                                                                                    \
+    return b ? launch_cluster(k_resident_graph<Z, M, CC, true>, a, words, CC, threads, smem, st) \
+             : launch_cluster(k_resident_graph<Z, M, CC, false>, a, words, CC, threads, smem, st);
+    KA_C(1)
+    KA_C(4)
+    KA_C(8)
+#undef KA_C
+    default:
+      return cudaErrorInvalidValue;
+  }
+}
+
+template <int Z>
+cudaError_t launch_z(const Args& a, int m, unsigned words, int C, int threads, size_t smem,
+                     cudaStream_t st) {
+  switch (m < Z - 1 ? m : Z - 1) {  // m >= z - 1: no constraint
+#define KA_CASE(MM) \
+  case MM:          \
+    return launch_m<Z, (MM < Z ? MM : 0)>(a, words, C, threads, smem, st);
+    KA_CASE(0)
+    KA_CASE(1)
+    KA_CASE(2)
+    KA_CASE(3)
+    KA_CASE(4)
+    KA_CASE(5)
+    KA_CASE(6)
+    KA_CASE(7)
+#undef KA_CASE
+    default:
+      return cudaErrorInvalidValue;
+  }
+}
+
+// shared memory: entry buffers, n of N sites, the swapped bits of a share of the bonds
+int64_t fslots_for(int64_t nbonds, int C) { return (nbonds + C - 1) / C + kMaxClasses; }
+size_t smem_for(int64_t N, int64_t class_max, int64_t nbonds, int C, bool f) {
+  return (C > 1 ? 2 * (size_t)((class_max + 1) & ~1LL) * 8 : 0) + (size_t)(N + 2) * 8 +
+         (f ? (size_t)fslots_for(nbonds, C) * 8 : 0);
+}
+
+constexpr size_t kGraphSmem = kSmemMax - 2048;  // beside the unit and the class tables
+
+}  // namespace
+
+bool graph_fits(int64_t N) { return N >= 2 && N < 65535 && (size_t)(N + 2) * 8 <= kGraphSmem; }
+
+int graph_record_bytes(int z) { return z <= 4 ? 16 : 32; }
+
+void graph_records(int64_t N, int z, const int32_t* nbr, const int32_t* bu, const int32_t* bv,
+                   int64_t nbonds, uint16_t* rec) {
+  const int Z = z <= 4 ? 4 : 8;
+  for (int64_t e = 0; e < nbonds; ++e) {
+    uint16_t* o = rec + e * 2 * Z;
+    const int32_t end[2] = {bu[e], bv[e]};
+    o[0] = (uint16_t)end[0];
+    o[1] = (uint16_t)end[1];
+    for (int s = 0; s < 2; ++s) {
+      uint16_t* q = o + 2 + s * (Z - 1);
+      int at = 0;
+      for (int k = 0; k < z; ++k) {
+        const int32_t x = nbr[(int64_t)end[s] * z + k];
+        if (x != end[s ^ 1]) q[at++] = (uint16_t)x;
+      }
+      while (at < Z - 1) q[at++] = (uint16_t)N;
+    }
+  }
+}
+
+int graph_cluster(int64_t N, int64_t nbonds, int64_t class_max, int64_t words, int sms) {
+  // a thread per bond of a class and all tables in shared memory; the fewest
+  // CTAs that do.  us a sweep (z = 4, one word) with 1, 4, 8 CTAs, and with one
+  // launch per class: N = 2^12 15.5, 17.4, 20.5; 37.  2^13: -, 21.7, 22.2; 40.
+  // 2^14: -, 45 (no room for the swapped bits), 31.5; 44.  With 32 words 2^14
+  // takes 48 with four CTAs and 94 with eight (they no longer run at once); 113.
+  auto fits = [&](int C, bool f) {
+    return class_max <= 1024 * C && smem_for(N, class_max, nbonds, C, f) <= kGraphSmem;
+  };
+  for (int C : {1, 4, 8})
+    if (fits(C, true)) return C == 8 && words * 8 > sms && fits(4, false) ? 4 : C;
+  return 0;
+}
+
+cudaError_t launch_graph(const Args& args, int64_t Nmax, int64_t bonds_max, int64_t class_max, int z,
+                         int m, unsigned words, int C, cudaStream_t st) {
+  if (m < 0 || z < 1 || z > 8 || !graph_fits(Nmax) || class_max > 1024 * C)
+    return cudaErrorInvalidValue;
+  Args a = args;
+  a.fsmem = smem_for(Nmax, class_max, bonds_max, C, true) <= kGraphSmem;
+  a.fslots = (int)fslots_for(bonds_max, C);
+  a.entries = C > 1 ? (int)((class_max + 1) & ~1LL) : 0;  // n stays 16-byte aligned
+  const size_t smem = smem_for(Nmax, class_max, bonds_max, C, a.fsmem != 0);
+  if (smem > kGraphSmem) return cudaErrorInvalidValue;
+  const int threads = (int)std::max<int64_t>(64, ((class_max + C - 1) / C + 31) / 32 * 32);
+  return z <= 4 ? launch_z<4>(a, m, words, C, threads, smem, st)
+                : launch_z<8>(a, m, words, C, threads, smem, st);
+}
+
+}  // namespace resident
+}  // namespace ka
