@@ -7,13 +7,15 @@
 // of a shape class: the group kernels of three-dimensional lattices for the
 // units of one side and m (d = 3), the general pencil kernel for the cubic
 // units of one (d, V, m) otherwise; and ONE launch of the edge-gather kernel
-// covers class c of all graph units of a shape class (V, m).  Units carry their own sweep counter t_base and stop counter t_end
+// covers class c of all graph units of a shape class (V, m).  Units of small
+// topologies stay on chip: one launch runs their whole round.  Units carry their own sweep counter t_base and stop counter t_end
 // in a device table, so a job that reaches its next observation point (or
 // its target) inside the round simply idles.  The round's launch sequence
 // can be captured in a CUDA graph and replayed while the job set and the
 // round length stay the same (the unit tables are refreshed by a copy before
 // every replay).
 #include <algorithm>
+#include <array>
 #include <cstring>
 #include <map>
 #include <string>
@@ -33,6 +35,7 @@ struct Job {
   int64_t* obs_dev = nullptr;  // [cap][R][4]
   std::vector<int64_t> obs_t;
   bool finished = false;
+  int64_t units = 0;    // its units in the tables
   bool batched = true;  // false: runs with its own (single-instance) launches inside each round
 };
 
@@ -55,6 +58,19 @@ struct StreamClass {
   std::vector<int> plane;
   void* dev = nullptr;
   size_t count() const { return owner.size(); }
+};
+
+// Jobs on small topologies whose sweeps stay on chip (ka_resident.cuh): one
+// launch runs a whole round of every unit (a word of a job).  Cubic lattices of
+// one (d, L, m), or graphs of one m and record size whose tables fit together.
+struct ResidentClass {
+  int d = 0, L = 0;  // graphs: 0
+  int z = 0, m = 0;
+  int64_t N_max = 0, bonds_max = 0, class_max = 0;
+  int C = 0;
+  std::vector<ka::resident::Unit> units;
+  std::vector<Job*> owner;
+  ka::resident::Unit* dev = nullptr;
 };
 
 struct GraphClass {
@@ -93,8 +109,15 @@ struct ka_batch {
   std::vector<CubicClass> cubic;
   std::vector<StreamClass> sclass;  // three-dimensional lattices: the group kernels
   std::vector<GraphClass> graph;
+  std::vector<ResidentClass> resident;
   std::vector<void*> table_mem;  // device tables of the current job set
   bool own_stream = false;
+  struct Side {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t done = nullptr;
+  };
+  std::vector<Side> side;  // streams of the shape classes
+  cudaEvent_t fork = nullptr;
   cudaGraphExec_t exec = nullptr;
   int64_t exec_k = 0;
   int64_t last_k = 0;  // a round length is captured the second time it is used
@@ -108,6 +131,8 @@ struct ka_batch {
 
 namespace {
 
+constexpr size_t kSideStreams = 16;
+
 ka_status cuda_err(ka_batch* b, cudaError_t e, const char* what) {
   b->err = std::string(what) + ": " + cudaGetErrorString(e);
   return KA_ECUDA;
@@ -119,6 +144,7 @@ void free_tables(ka_batch* b) {
   b->cubic.clear();
   b->sclass.clear();
   b->graph.clear();
+  b->resident.clear();
   if (b->exec) {
     cudaGraphExecDestroy(b->exec);
     b->exec = nullptr;
@@ -134,15 +160,59 @@ cudaError_t dev_alloc(ka_batch* b, T** p, size_t count) {
   return e;
 }
 
+// Add a job's words to a class of on-chip units if its size runs there.
+// `words`: those of all jobs of its lattice (d, L, m).
+bool add_resident(ka_batch* b, Job* j, int64_t words) {
+  const ka_ctx* c = j->ctx;
+  if (!ka::resident_cluster(c, words)) return false;
+  const bool cubic = c->topo == KA_CUBIC;
+  ResidentClass* rc = nullptr;
+  for (auto& x : b->resident) {
+    if (x.m != c->m) continue;
+    if (cubic) {
+      if (x.L == c->L && x.d == c->d) rc = &x;
+    } else if (x.L == 0 && (x.z <= 4) == (c->z <= 4) && 2 * x.N_max > c->N && x.N_max < 2 * c->N &&
+               ka::resident::graph_cluster(std::max(x.N_max, c->N), std::max(x.bonds_max, c->nbonds),
+                                           std::max(x.class_max, c->class_max), 1, c->sms)) {
+      rc = &x;
+    }
+  }
+  if (!rc) {
+    b->resident.push_back(ResidentClass{});
+    rc = &b->resident.back();
+    rc->d = cubic ? c->d : 0;
+    rc->L = cubic ? c->L : 0;
+    rc->m = c->m;
+  }
+  rc->z = std::max(rc->z, c->z);
+  rc->N_max = std::max(rc->N_max, c->N);
+  rc->bonds_max = std::max(rc->bonds_max, c->nbonds);
+  rc->class_max = std::max(rc->class_max, c->class_max);
+  for (int w = 0; w < c->pl.W; ++w) {
+    rc->units.push_back(ka::resident_unit(c, w, 0, 0));
+    rc->owner.push_back(j);
+  }
+  return true;
+}
+
 // Group the unfinished batched jobs into shape classes and build the unit
 // tables (host copies; device copies are allocated here and filled per round).
 cudaError_t rebuild(ka_batch* b) {
   free_tables(b);
+  std::map<std::array<int, 3>, int64_t> lattice_words;
+  for (auto& kv : b->jobs) {
+    const ka_ctx* c = kv.second->ctx;
+    if (!kv.second->finished && kv.second->batched && c->topo == KA_CUBIC)
+      lattice_words[{c->d, c->L, c->m}] += c->pl.W;
+  }
   for (auto& kv : b->jobs) {
     Job* j = kv.second;
     if (j->finished || !j->batched) continue;
     ka_ctx* c = j->ctx;
     const int V = c->pl.V;
+    j->units = c->pl.W;
+    if (add_resident(b, j, c->topo == KA_CUBIC ? lattice_words[{c->d, c->L, c->m}] : c->pl.W)) continue;
+    j->units = c->pl.P;
     for (int q = 0; q < c->pl.P; ++q) {
       uint64_t* n = c->pl.n + (size_t)q * c->pl.plane_elems();
       uint64_t* p = c->pl.p + (size_t)q * c->pl.plane_elems();
@@ -265,9 +335,17 @@ cudaError_t rebuild(ka_batch* b) {
                                 cudaMemcpyHostToDevice, b->stream);
     if (e) return e;
   }
+  for (auto& rc : b->resident) {
+    const int64_t words = (int64_t)rc.units.size();
+    const int sms = rc.owner[0]->ctx->sms;
+    rc.C = rc.L ? ka::resident::cubic_cluster(rc.d, rc.L, words, sms)
+                : ka::resident::graph_cluster(rc.N_max, rc.bonds_max, rc.class_max, words, sms);
+    if ((e = dev_alloc(b, &rc.dev, rc.units.size()))) return e;
+  }
   b->dirty = false;
   b->last_k = 0;
   b->units = 0;
+  for (auto& rc : b->resident) b->units += (int64_t)rc.units.size();
   for (auto& cc : b->cubic) b->units += (int64_t)cc.units.size();
   for (auto& sc : b->sclass) b->units += (int64_t)sc.count();
   for (auto& gc : b->graph) b->units += (int64_t)gc.units.size();
@@ -275,13 +353,14 @@ cudaError_t rebuild(ka_batch* b) {
   return cudaStreamSynchronize(b->stream);
 }
 
-// Whether a job shares the batched launches: graphs always; a cubic lattice
+// Whether a job shares the batched launches: graphs and small lattices (on
+// chip) always; another cubic lattice
 // on the pencil kernels unless its groups have own_tiles tiles or more (it
 // then runs with its own launches inside each round: the group kernels of
 // three-dimensional lattices or the single-instance pencil kernel, arguments
 // in the constant bank); a cubic lattice on the edge-gather path never.
 bool shares_launches(const ka_batch* b, const ka_ctx* ctx) {
-  if (ctx->topo != KA_CUBIC) return true;
+  if (ctx->topo != KA_CUBIC || ka::resident_cluster(ctx, ctx->pl.W)) return true;
   if (!ctx->pencil) return false;
   int64_t pencils = 1;
   for (int k = 0; k < ctx->d - 1; ++k) pencils *= ctx->L;
@@ -297,33 +376,93 @@ int64_t allowance(const Job* j, int64_t k) {
   return std::max<int64_t>(0, std::min(k, stop - j->t));
 }
 
-// The launches of one round of length k (captured or run directly).
-cudaError_t issue_round(ka_batch* b, int64_t k) {
+// Streams for the shape classes of a round beside the batch's own, made when
+// first needed; kept until the batch is destroyed.
+cudaError_t side_streams(ka_batch* b, size_t count) {
   cudaError_t e = cudaSuccess;
-  for (int64_t s = 0; s < k && !e; ++s) {
-    for (auto& cc : b->cubic) {
-      const int npar = (cc.d == 1) ? 1 : 2;
+  if (!b->fork) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+  while (!e && b->side.size() < std::min(count, kSideStreams)) {
+    ka_batch::Side x;
+    e = cudaStreamCreateWithFlags(&x.stream, cudaStreamNonBlocking);
+    if (e) break;
+    e = cudaEventCreateWithFlags(&x.done, cudaEventDisableTiming);
+    if (e) {
+      cudaStreamDestroy(x.stream);
+      break;
+    }
+    b->side.push_back(x);
+  }
+  return e;
+}
+
+// The launches of one round of length k (captured or run directly).  The
+// shape classes share no state, and most of their launches are far from
+// filling the device (a class of small jobs is a chain of launches of a few
+// CTAs each), so the classes run side by side: class i on side stream i modulo
+// their number, forked from the batch's stream and joined to it at the end.
+cudaError_t issue_round(ka_batch* b, int64_t k) {
+  const size_t nclasses = b->cubic.size() + b->sclass.size() + b->graph.size() + b->resident.size();
+  cudaError_t e = cudaSuccess;
+  if (nclasses > 1) {
+    if ((e = side_streams(b, nclasses))) return e;
+    if ((e = cudaEventRecord(b->fork, b->stream))) return e;
+  }
+  size_t used = 0;  // classes begun
+  // the stream of the next class
+  auto stream = [&]() -> cudaStream_t {
+    if (nclasses <= 1) return b->stream;
+    const size_t i = used++;
+    ka_batch::Side& x = b->side[i % b->side.size()];
+    if (i < b->side.size() && !e) e = cudaStreamWaitEvent(x.stream, b->fork, 0);
+    return x.stream;
+  };
+  // the longest chains first: graphs have the most launches per sweep
+  for (auto& gc : b->graph) {
+    const cudaStream_t st = stream();
+    const int n = (int)gc.units.size();
+    for (int64_t s = 0; s < k && !e; ++s)
+      for (int c = 0; c < gc.cmax && !e; ++c)
+        e = ka::launch_graph_class_batch(gc.dev, gc.prefix_dev + (size_t)c * (n + 1),
+                                         gc.first_dev + (size_t)c * n, n, gc.total[c], gc.V, gc.m,
+                                         (uint32_t)c, (uint32_t)s, st);
+  }
+  for (auto& rc : b->resident) {
+    const cudaStream_t st = stream();
+    ka::resident::Args a{};
+    a.units = rc.dev;
+    a.most = (uint32_t)ka::resident::kMaxSweeps;
+    const unsigned words = (unsigned)rc.units.size();
+    for (int64_t s = 0; s < k && !e; s += ka::resident::kMaxSweeps) {
+      a.from = (uint32_t)s;
+      e = rc.L ? ka::resident::launch_cubic(a, rc.d, rc.L, rc.m, words, rc.C, st)
+               : ka::resident::launch_graph(a, rc.N_max, rc.bonds_max, rc.class_max, rc.z, rc.m, words,
+                                            rc.C, st);
+    }
+  }
+  for (auto& sc : b->sclass) {
+    const cudaStream_t st = stream();
+    for (int64_t s = 0; s < k && !e; ++s)
+      for (int mu = 0; mu < 3 && !e; ++mu)
+        for (int par = 0; par < 2 && !e; ++par)
+          e = ka::launch_stream_batch(sc.dev, (int)sc.count(), sc.L, sc.m, mu, par, (uint32_t)s, st);
+  }
+  for (auto& cc : b->cubic) {
+    const cudaStream_t st = stream();
+    const int npar = (cc.d == 1) ? 1 : 2;
+    for (int64_t s = 0; s < k && !e; ++s)
       for (int mu = 0; mu < cc.d && !e; ++mu)
         for (int par = 0; par < npar && !e; ++par) {
           const bool x = (mu == 0) || cc.d == 1;
           e = ka::launch_cubic_group_batch(cc.dev, cc.tile_unit_dev[x ? 0 : 1],
                                            (int)cc.units.size(), cc.ntiles[x ? 0 : 1],
-                                           cc.PSmax, cc.d, cc.V, cc.m, mu, par, (uint32_t)s,
-                                           b->stream);
+                                           cc.PSmax, cc.d, cc.V, cc.m, mu, par, (uint32_t)s, st);
         }
-    }
-    for (auto& sc : b->sclass)
-      for (int mu = 0; mu < 3 && !e; ++mu)
-        for (int par = 0; par < 2 && !e; ++par)
-          e = ka::launch_stream_batch(sc.dev, (int)sc.count(), sc.L, sc.m, mu, par, (uint32_t)s,
-                                      b->stream);
-    for (auto& gc : b->graph) {
-      const int n = (int)gc.units.size();
-      for (int c = 0; c < gc.cmax && !e; ++c)
-        e = ka::launch_graph_class_batch(gc.dev, gc.prefix_dev + (size_t)c * (n + 1),
-                                         gc.first_dev + (size_t)c * n, n, gc.total[c], gc.V, gc.m,
-                                         (uint32_t)c, (uint32_t)s, b->stream);
-    }
+  }
+  // join, also after an error: nothing is left running beside the batch's stream
+  for (size_t i = 0; i < std::min(used, b->side.size()); ++i) {
+    cudaError_t ej = cudaEventRecord(b->side[i].done, b->side[i].stream);
+    if (!ej) ej = cudaStreamWaitEvent(b->stream, b->side[i].done, 0);
+    if (!e) e = ej;
   }
   return e;
 }
@@ -399,6 +538,17 @@ ka_status run_round(ka_batch* b, int64_t k_req, int64_t* ran) {
                                b->stream)))
         return cuda_err(b, e, "unit table");
     }
+    for (auto& rc : b->resident) {
+      for (size_t u = 0; u < rc.units.size(); ++u) {
+        const Job* j = rc.owner[u];
+        const bool live = j && !j->finished;
+        rc.units[u].t_base = live ? (uint32_t)j->t : 0u;
+        rc.units[u].count = live ? (uint32_t)allowance(j, k) : 0u;
+      }
+      if ((e = cudaMemcpyAsync(rc.dev, rc.units.data(), rc.units.size() * sizeof(rc.units[0]),
+                               cudaMemcpyHostToDevice, b->stream)))
+        return cuda_err(b, e, "unit table");
+    }
     for (auto& gc : b->graph) {
       for (size_t u = 0; u < gc.units.size(); ++u) {
         const Job* j = gc.owner[u];
@@ -457,7 +607,7 @@ ka_status run_round(ka_batch* b, int64_t k_req, int64_t* ran) {
     }
     if (j->t >= j->target) {
       j->finished = true;
-      if (j->batched) b->idle_units += j->ctx->pl.P;  // idles in the tables until rebuilt
+      if (j->batched) b->idle_units += j->units;  // idles in the tables until rebuilt
     }
   }
   e = cudaStreamSynchronize(b->stream);
@@ -782,6 +932,12 @@ ka_status ka_batch_remove(ka_batch* b, int64_t job_id) {
         o = nullptr;
         ++in_tables;
       }
+  for (auto& rc : b->resident)
+    for (auto& o : rc.owner)
+      if (o == j) {
+        o = nullptr;
+        ++in_tables;
+      }
   for (auto& gc : b->graph)
     for (auto& o : gc.owner)
       if (o == j) {
@@ -818,6 +974,11 @@ ka_status ka_batch_destroy(ka_batch* b) {
     delete j;
   }
   free_tables(b);
+  for (auto& x : b->side) {
+    cudaStreamDestroy(x.stream);
+    cudaEventDestroy(x.done);
+  }
+  if (b->fork) cudaEventDestroy(b->fork);
   if (b->own_stream) cudaStreamDestroy(b->stream);
   delete b;
   return st;
