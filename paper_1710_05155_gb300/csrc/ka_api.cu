@@ -507,7 +507,7 @@ ka_status ka_observe_device(ka_ctx* c, int64_t* counts_device) {
   if (!c || !counts_device) return KA_EINVAL;
   if (!c->initialized) return fail(c, KA_ESTATE, "observe before init or set_state");
   DeviceGuard dg(c->device);
-  cudaError_t e = ka::launch_observe(c->pl, c->R, (unsigned long long*)counts_device, c->stream);
+  cudaError_t e = ka::launch_observe(c->pl, (unsigned long long*)counts_device, c->stream);
   if (e) return cuda_fail(c, e, "observe");
   return KA_OK;
 }
@@ -517,7 +517,7 @@ ka_status ka_observe(ka_ctx* c, int64_t* sweep_out, int64_t* counts) {
   if (!c || !counts) return KA_EINVAL;
   if (!c->initialized) return fail(c, KA_ESTATE, "observe before init or set_state");
   DeviceGuard dg(c->device);
-  cudaError_t e = ka::launch_observe(c->pl, c->R, c->counts_dev, c->stream);
+  cudaError_t e = ka::launch_observe(c->pl, c->counts_dev, c->stream);
   if (!e) e = cudaMemcpyAsync(counts, c->counts_dev, (size_t)c->R * 4 * sizeof(int64_t),
                               cudaMemcpyDeviceToHost, c->stream);
   if (e) return cuda_fail(c, e, "observe");

@@ -473,7 +473,7 @@ ka_status observe_job(ka_batch* b, Job* j) {
     return KA_ESTATE;
   }
   const int R = j->ctx->R;
-  cudaError_t e = ka::launch_observe(j->ctx->pl, R,
+  cudaError_t e = ka::launch_observe(j->ctx->pl,
                                      (unsigned long long*)(j->obs_dev + j->n_obs * R * 4),
                                      b->stream);
   if (e) return cuda_err(b, e, "observe");

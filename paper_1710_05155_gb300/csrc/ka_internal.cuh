@@ -264,7 +264,9 @@ void stream_unit_fill(void* unit, uint64_t* n, uint64_t* p, uint32_t word0, uint
 cudaError_t launch_stream_batch(const void* units_dev, int nunits, int L, int m, int mu, int par,
                                 uint32_t sweep_offset, cudaStream_t st);
 
-cudaError_t launch_observe(const Planes& pl, int R, unsigned long long* counts_dev,
-                           cudaStream_t st);
+// counts [R][4] of the observables; counts [R] of the particles of planes q0 .. q0 + nq - 1
+cudaError_t launch_observe(const Planes& pl, unsigned long long* counts_dev, cudaStream_t st);
+cudaError_t launch_particles(const Planes& pl, int q0, int nq, unsigned long long* counts_dev,
+                             cudaStream_t st);
 
 }  // namespace ka

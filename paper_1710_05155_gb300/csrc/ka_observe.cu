@@ -8,140 +8,202 @@
 //   persist_occ = sum_i n0_i & p_i
 //   persist_all = sum_i p_i
 //
-// Each thread adds up to 63 words into bit-sliced counters (6 slices: one
-// uint64 per binary digit, so all 64 replicas count in parallel with a
-// ripple adder); the words per thread are chosen so that the grid fills the
-// device, four independent loads in flight per thread.  Lanes holding the same word position are then summed in
-// bit-sliced form through warp shuffles, the warp total is turned into one
-// integer per replica, and blocks accumulate in shared memory before one
-// 64-bit atomic per counter goes to global memory.
+// Each thread adds up to 120 words of one word position into bit-sliced
+// counters (one uint64 per binary digit, so all 64 replicas count at once),
+// eight words at a time through a tree of full adders: 7 adders of two
+// operations a half-word for eight words, where a ripple adder per word takes
+// 12 on six digits.  Lanes of the same word position are then summed in
+// bit-sliced form (the first exchange splits the 64 replicas over two lanes),
+// the warp total is turned into one integer per replica, and blocks
+// accumulate in shared memory before one 64-bit atomic per counter goes to
+// global memory.  That summing costs about 200 operations a thread and
+// observable, so the grid is one wave, of threads with as many words as that
+// gives.
+//
+// What bounds it: the read of n, n0 and p (24 bytes a site-word).  L = 128, 256
+// replicas: 201 MB; before (14 words a thread, ripple adders) 106 us, bound by
+// the ALUs (82 %).
+#include <algorithm>
 #include <mutex>
+
 #include "ka_internal.cuh"
 
 namespace ka {
 namespace {
 
-constexpr int kSlices = 6;        // per-thread counters hold up to 63
-constexpr int kPerThread = 63;    // most words per thread
-constexpr int kWide = kSlices + 5;  // after summing 32 lanes
+// binary digits of a thread's counters: up to 120 words, or (small planes) 8
+constexpr int kDigits = 7, kFewDigits = 4;
+constexpr int kPerThread = 120, kFew = 8;
 
-__device__ __forceinline__ void ripple_add(uint64_t (&c)[kSlices], uint64_t x) {
+__device__ __forceinline__ uint64_t maj(uint64_t a, uint64_t b, uint64_t c) {
+  return (a & b) | (c & (a | b));
+}
+
+// full adder: s += x + y, returns the carry word
+__device__ __forceinline__ uint64_t add2(uint64_t& s, uint64_t x, uint64_t y) {
+  const uint64_t k = maj(s, x, y);
+  s ^= x ^ y;
+  return k;
+}
+
+// c += x[0] + .. + x[7]
+template <int S>
+__device__ __forceinline__ void add8(uint64_t (&c)[S], const uint64_t (&x)[8]) {
+  const uint64_t t0 = add2(c[0], x[0], x[1]), t1 = add2(c[0], x[2], x[3]);
+  const uint64_t t2 = add2(c[0], x[4], x[5]), t3 = add2(c[0], x[6], x[7]);
+  const uint64_t f0 = add2(c[1], t0, t1), f1 = add2(c[1], t2, t3);
+  uint64_t k = add2(c[2], f0, f1);
 #pragma unroll
-  for (int s = 0; s < kSlices; ++s) {
-    const uint64_t k = c[s] & x;
-    c[s] ^= x;
-    x = k;
+  for (int s = 3; s < S; ++s) {
+    const uint64_t n = c[s] & k;
+    c[s] ^= k;
+    k = n;
   }
 }
 
-// add the counter of lane (lane ^ off) into this lane's, bit-sliced
-__device__ __forceinline__ void shfl_add(uint64_t (&c)[kWide], int off) {
-  uint64_t carry = 0;
+// The warp total of one counter set, one integer per replica, into acc (word
+// position major).  Lanes of the same position are V apart.
+template <int V, int S>
+__device__ __forceinline__ void reduce(const uint64_t (&c)[S], unsigned int* acc) {
+  constexpr int kWide = S + 5;  // digits after summing 32 lanes
+  const int lane = threadIdx.x & 31;
+  const bool upper = lane & 16;
+  uint32_t w[kWide];
+  uint32_t carry = 0;
+  // lanes 0-15 go on with replicas 0-31 of both lanes, lanes 16-31 with 32-63
 #pragma unroll
-  for (int s = 0; s < kWide; ++s) {
-    const uint64_t o = __shfl_xor_sync(0xffffffffu, c[s], off);
-    const uint64_t sum = c[s] ^ o ^ carry;
-    carry = (c[s] & o) | (carry & (c[s] | o));
-    c[s] = sum;
+  for (int s = 0; s < S; ++s) {
+    const uint32_t lo = (uint32_t)c[s], hi = (uint32_t)(c[s] >> 32);
+    const uint32_t o = __shfl_xor_sync(0xffffffffu, upper ? lo : hi, 16), m = upper ? hi : lo;
+    w[s] = m ^ o ^ carry;
+    carry = (m & o) | (carry & (m | o));
   }
+  w[S] = carry;
+  int wide = S + 1;
+#pragma unroll
+  for (int off = 8; off >= V; off >>= 1) {
+    carry = 0;
+#pragma unroll
+    for (int s = 0; s < kWide; ++s) {
+      if (s < wide) {
+        const uint32_t o = __shfl_xor_sync(0xffffffffu, w[s], off), m = w[s];
+        w[s] = m ^ o ^ carry;
+        carry = (m & o) | (carry & (m | o));
+      }
+    }
+    w[wide++] = carry;
+  }
+  // lanes hh and 16 + hh hold the totals of word position hh
+#pragma unroll
+  for (int hh = 0; hh < V; ++hh)
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      unsigned int v = 0;
+#pragma unroll
+      for (int s = 0; s < kWide; ++s)
+        if (s < wide) v |= ((__shfl_sync(0xffffffffu, w[s], 16 * half + hh) >> lane) & 1u) << s;
+      if (v) atomicAdd(&acc[hh * 64 + 32 * half + lane], v);
+    }
 }
 
-template <int V>
+// ALL: the four observables; else only the particles
+template <int V, bool ALL, int S>
 __global__ void __launch_bounds__(256, 2) k_observe(Planes pl, unsigned long long* counts,
                                                  int per_thread) {
-  __shared__ unsigned int acc[4][64 * V];
+  constexpr int O = ALL ? 4 : 1;
+  __shared__ unsigned int acc[O][64 * V];
   const int q = blockIdx.y;
-  for (int k = threadIdx.x; k < 4 * 64 * V; k += blockDim.x) (&acc[0][0])[k] = 0;
+  for (int k = threadIdx.x; k < O * 64 * V; k += blockDim.x) (&acc[0][0])[k] = 0;
   __syncthreads();
 
   const size_t E = pl.plane_elems();
-  const size_t base = (size_t)q * E;
-  // element e of the plane holds word h = e % V of site e / V; blockDim and
-  // the stride are even, so a thread always sees the same h
+  const uint64_t* gn = pl.n + (size_t)q * E;
+  const uint64_t* g0 = ALL ? pl.n0 + (size_t)q * E : nullptr;
+  const uint64_t* gp = ALL ? pl.p + (size_t)q * E : nullptr;
+  // element e of the plane holds word h = e % V of site e / V; the block size
+  // is a multiple of V, so a thread always sees the same h
   const size_t e0 = (size_t)blockIdx.x * blockDim.x * per_thread + threadIdx.x;
-  uint64_t c[4][kSlices];
+  uint64_t c[O][S];
 #pragma unroll
-  for (int o = 0; o < 4; ++o)
+  for (int o = 0; o < O; ++o)
 #pragma unroll
-    for (int s = 0; s < kSlices; ++s) c[o][s] = 0;
-  for (int k = 0; k < per_thread; k += 4) {
-    uint64_t n[4], n0[4], p[4];
+    for (int s = 0; s < S; ++s) c[o][s] = 0;
+  for (int k = 0; k < per_thread; k += 8) {
+    uint64_t n[8], n0[8], p[8];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < 8; ++u) {
       const size_t e = e0 + (size_t)(k + u) * blockDim.x;
-      const bool in = (k + u < per_thread) && e < E;
-      n[u] = in ? pl.n[base + e] : 0ull;
-      n0[u] = in ? pl.n0[base + e] : 0ull;
-      p[u] = in ? pl.p[base + e] : 0ull;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      ripple_add(c[0], n[u]);
-      ripple_add(c[1], n[u] & n0[u]);
-      ripple_add(c[2], n0[u] & p[u]);
-      ripple_add(c[3], p[u]);
-    }
-  }
-
-  const int lane = threadIdx.x & 31;
-  const int h = lane % V;
-#pragma unroll
-  for (int o = 0; o < 4; ++o) {
-    uint64_t w[kWide];
-#pragma unroll
-    for (int s = 0; s < kWide; ++s) w[s] = (s < kSlices) ? c[o][s] : 0;
-    // sum lanes with the same word position (stride V)
-#pragma unroll
-    for (int off = 16; off >= V; off >>= 1) shfl_add(w, off);
-    // lanes 0 .. V-1 hold the totals of word positions 0 .. V-1; every lane
-    // extracts replicas (bit positions) lane and lane + 32 of each
-#pragma unroll
-    for (int hh = 0; hh < V; ++hh) {
-      unsigned int lo = 0, hi = 0;
-#pragma unroll
-      for (int s = 0; s < kWide; ++s) {
-        const uint64_t t = __shfl_sync(0xffffffffu, w[s], hh);
-        lo |= (unsigned int)((t >> lane) & 1u) << s;
-        hi |= (unsigned int)((t >> (lane + 32)) & 1u) << s;
+      const bool in = e < E;
+      n[u] = in ? gn[e] : 0ull;
+      if constexpr (ALL) {
+        n0[u] = in ? g0[e] : 0ull;
+        p[u] = in ? gp[e] : 0ull;
       }
-      if (lo) atomicAdd(&acc[o][hh * 64 + lane], lo);
-      if (hi) atomicAdd(&acc[o][hh * 64 + lane + 32], hi);
+    }
+    add8(c[0], n);
+    if constexpr (ALL) {
+      add8(c[3], p);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        n[u] &= n0[u];
+        p[u] &= n0[u];
+      }
+      add8(c[1], n);
+      add8(c[2], p);
     }
   }
-  (void)h;
+#pragma unroll
+  for (int o = 0; o < O; ++o) reduce<V, S>(c[o], acc[o]);
   __syncthreads();
-  for (int k = threadIdx.x; k < 4 * 64 * V; k += blockDim.x) {
+  for (int k = threadIdx.x; k < O * 64 * V; k += blockDim.x) {
     const int o = k / (64 * V), rb = k % (64 * V);  // rb = h * 64 + bit
     const unsigned int v = acc[o][rb];
     if (v) {
       const int r = (q * V + rb / 64) * 64 + (rb % 64);
-      atomicAdd(&counts[(size_t)r * 4 + o], (unsigned long long)v);
+      atomicAdd(&counts[(size_t)r * O + o], (unsigned long long)v);
     }
   }
 }
 
-}  // namespace
-
-cudaError_t launch_observe(const Planes& pl, int R, unsigned long long* counts_dev,
-                           cudaStream_t st) {
-  cudaError_t err = cudaMemsetAsync(counts_dev, 0, (size_t)R * 4 * sizeof(unsigned long long), st);
+template <bool ALL>
+cudaError_t launch_counts(const Planes& pl, unsigned long long* counts_dev, cudaStream_t st) {
+  cudaError_t err = cudaMemsetAsync(
+      counts_dev, 0, (size_t)pl.P * pl.V * 64 * (ALL ? 4 : 1) * sizeof(unsigned long long), st);
   if (err != cudaSuccess) return err;
-  // words per thread: enough blocks for four per SM, at most kPerThread
+  // words per thread, in eights: one wave of two blocks per SM over all planes
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const size_t E = pl.plane_elems();
-  const size_t want = (size_t)256 * 4 * (size_t)(sms > 0 ? sms : 148);
-  int per_thread = (int)((E + want - 1) / want);
-  per_thread = per_thread < 4 ? 4 : (per_thread > kPerThread ? kPerThread : per_thread);
-  const size_t per_block = (size_t)256 * per_thread;
-  dim3 grid((unsigned)((E + per_block - 1) / per_block), (unsigned)pl.P);
-  if (pl.V == 4)
-    k_observe<4><<<grid, 256, 0, st>>>(pl, counts_dev, per_thread);
-  else if (pl.V == 2)
-    k_observe<2><<<grid, 256, 0, st>>>(pl, counts_dev, per_thread);
-  else
-    k_observe<1><<<grid, 256, 0, st>>>(pl, counts_dev, per_thread);
+  const size_t wave = (size_t)256 * 2 * (size_t)(sms > 0 ? sms : 148);
+  size_t per_thread = (E * (size_t)pl.P + wave - 1) / wave;
+  per_thread = std::min<size_t>((per_thread + 7) / 8 * 8, kPerThread);
+  const size_t per_block = 256 * per_thread;
+  const dim3 grid((unsigned)((E + per_block - 1) / per_block), (unsigned)pl.P);
+  const bool few = per_thread <= kFew;
+#define KA_LAUNCH(V, S) k_observe<V, ALL, S><<<grid, 256, 0, st>>>(pl, counts_dev, (int)per_thread)
+  if (pl.V == 4) {
+    if (few) KA_LAUNCH(4, kFewDigits); else KA_LAUNCH(4, kDigits);
+  } else if (pl.V == 2) {
+    if (few) KA_LAUNCH(2, kFewDigits); else KA_LAUNCH(2, kDigits);
+  } else {
+    if (few) KA_LAUNCH(1, kFewDigits); else KA_LAUNCH(1, kDigits);
+  }
+#undef KA_LAUNCH
   return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_observe(const Planes& pl, unsigned long long* counts_dev, cudaStream_t st) {
+  return launch_counts<true>(pl, counts_dev, st);
+}
+
+cudaError_t launch_particles(const Planes& pl, int q0, int nq, unsigned long long* counts_dev,
+                             cudaStream_t st) {
+  Planes part = pl;
+  part.n += (size_t)q0 * pl.plane_elems();
+  part.P = nq;
+  return launch_counts<false>(part, counts_dev + (size_t)q0 * pl.V * 64, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -216,7 +278,7 @@ extern "C" ka_status ka_observe_static(const uint64_t* n, const uint64_t* n0, co
   pl.W = replicas / 64;
   pl.V = 1;
   pl.P = pl.W;
-  e = ka::launch_observe(pl, replicas, scratch, st);  // clears the scratch, then accumulates
+  e = ka::launch_observe(pl, scratch, st);  // clears the scratch, then accumulates
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(counts, scratch, (size_t)replicas * 4 * sizeof(int64_t),
                         cudaMemcpyDeviceToHost, st);
