@@ -20,7 +20,7 @@ constexpr size_t kAlign = 256;
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-  size_t n, n0, p, stage, counts, hist, pre_key, pre_idx, krem, unresolved, err, nbr, bu, bv, bid,
+  size_t n, n0, p, stage, counts, list, list_bytes, list_n, below, err, nbr, bu, bv, bid,
       perm, inv, rec, coff, total;
 };
 
@@ -96,13 +96,21 @@ Layout layout_of(const Shape& s) {
   l.n0 = take(plane);
   l.p = take(plane);
   // layout conversion of get/set_state (graphs: breadth-first storage order)
-  l.stage = (s.V > 1 || s.xs || s.topo != KA_CUBIC) ? take(plane) : 0;
+  const bool has_stage = s.V > 1 || s.xs || s.topo != KA_CUBIC;
+  l.stage = has_stage ? take(plane) : 0;
   l.counts = take((size_t)s.R * 4 * sizeof(unsigned long long));
-  l.hist = take((size_t)s.R * 256 * sizeof(uint32_t));
-  l.pre_key = take((size_t)s.R * sizeof(uint64_t));
-  l.pre_idx = take((size_t)s.R * sizeof(uint32_t));
-  l.krem = take((size_t)s.R * sizeof(int64_t));
-  l.unresolved = take(sizeof(int32_t));
+  // the initial state's lists: in the staging plane, idle meanwhile, if it
+  // holds those of sixteen words (or all), else in room of their own for that
+  const int planes = std::max(1, std::min(s.P, 16 / s.V));
+  l.list_bytes = (size_t)planes * s.V * 64 * (size_t)ka::init_list_cap(s.N) * sizeof(uint32_t);
+  if (has_stage && plane >= l.list_bytes) {
+    l.list = l.stage;
+    l.list_bytes = plane;
+  } else {
+    l.list = take(l.list_bytes);
+  }
+  l.list_n = take((size_t)s.R * sizeof(uint32_t));
+  l.below = take((size_t)s.R * sizeof(unsigned long long));
   l.err = take(sizeof(int32_t));
   if (!s.pencil) {
     l.nbr = take((size_t)s.N * s.z * sizeof(int32_t));
@@ -174,14 +182,11 @@ ka_status create_common(const ka_params* params, void* buf, size_t bytes, bool o
   c->err_dev = (int*)(base + l.err);
   c->counts_dev = (unsigned long long*)(base + l.counts);
   c->stage = (s.V > 1 || s.xs || s.topo != KA_CUBIC) ? (uint64_t*)(base + l.stage) : nullptr;
-  c->is.hist = (uint32_t*)(base + l.hist);
-  c->is.pre_key = (uint64_t*)(base + l.pre_key);
-  c->is.pre_idx = (uint32_t*)(base + l.pre_idx);
-  c->is.krem = (int64_t*)(base + l.krem);
-  c->is.unresolved = (int32_t*)(base + l.unresolved);
-  c->is.cand = c->stage ? (uint32_t*)c->stage : nullptr;  // idle during init
+  c->is.list = (uint32_t*)(base + l.list);
+  c->is.list_bytes = l.list_bytes;
+  c->is.list_n = (uint32_t*)(base + l.list_n);
+  c->is.below = (unsigned long long*)(base + l.below);
   cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, params->device);
-  c->is.cand_bytes = c->stage ? (size_t)s.N * s.W * sizeof(uint64_t) : 0;
 
   {
     const cudaError_t ez = cudaMemsetAsync(c->err_dev, 0, sizeof(int), c->stream);

@@ -6,240 +6,243 @@
 // counter (r / 2, 0xFFFFFFFF, i, 0): the first K entries of a uniformly
 // random permutation, so every K-subset is equally likely.
 //
-// The K-th smallest composite key of every replica is found exactly by a
-// most-significant-digit radix select over 8-bit digits: eight passes over
-// the 64-bit key, then (only if some replica's threshold key is tied)
-// passes over the site index.  Keys are recomputed instead of stored, which
-// keeps the scratch at R x 256 counters.  When the context has room (its
-// staging plane, idle during init), the sites whose key shares the threshold's
-// top byte -- about N / 256 per replica -- are collected into per-replica
-// lists after the first pass, and the later passes evaluate only those; a list
-// that would overflow its capacity sends the later passes back to scanning
-// all sites.  A final pass writes the bit planes: n = [composite <=
-// threshold], n0 = n, p = all ones.
+// The Philox blocks bound this (32 per site and word), so every key is drawn
+// once: the K-th smallest of N uniform keys lies within a few standard
+// deviations of K / N, a window that is the same for every replica, known
+// before any key is drawn.
+//  * k_init_draw: one thread per site and word writes n = [key below the
+//    window] and collects the sites whose key lies in it (6 deviations to
+//    either side: 6 sqrt(N) of them at most on average) in a list per replica.
+//  * the particles so far are counted per replica (ka_observe.cu).
+//  * k_init_select: one block per replica finds the exact K-th smallest
+//    composite key among the list and sets the bits of the list's sites up to
+//    it.  A replica whose K-th key is not in the window, or whose list is
+//    full (about one in 10^9), and every replica of a lattice of less than
+//    kListSites sites, takes all sites as its list.
+// L = 128, 256 replicas, one GB300: 3.24 ms for the radix select that was here
+// before (three full passes of 0.85 to 1.11 ms, 20 small launches and a wait
+// for the host in between), 0.86 ms now; 268 million blocks at the 4.9e11 a
+// second that a bare loop of them reaches take 0.55 ms.
 #include <algorithm>
-#include <vector>
+#include <cmath>
 
 #include "ka_internal.cuh"
 
 namespace ka {
 namespace {
 
-constexpr int kSitesPerThread = 32;
+constexpr int kThreads = 256;       // of a draw block
+constexpr int kStage = 2048;        // candidates a draw block collects before the lists
+constexpr int kSelect = 512;        // threads of a select block, and most keys it ranks directly
+constexpr int kBuckets = 1024;
+constexpr int64_t kListSites = 2048;
 
 struct InitArgs {
-  uint32_t* hist;
-  uint32_t* cand_n;  // [R] candidates collected per replica
-  uint32_t* cand;    // [R][cap] their site indices
-  int64_t cap;
-  uint64_t* pre_key;
-  uint32_t* pre_idx;
-  int64_t* krem;
-  int32_t* unresolved;
-  int64_t N;
-  int idx_bits;  // bits of the site index digits (a multiple of 8)
-  int pass;      // 0..7 key bytes from the top, then index bytes from the top
+  uint32_t* list_n;    // [R] sites in each replica's list
+  uint32_t* list;      // [replicas of the launch][cap] their storage positions
+  const unsigned long long* below;  // [R] keys below the window
+  uint32_t cap;
+  uint32_t lo, span;   // the window of a key's high word: lo .. lo + span
+  int64_t K;
+  int q0;              // first plane of the launch
+  bool all;            // no lists: all sites
   RoundKeys rk;
 };
 
-// does the composite (key, i) agree with the decided digits of the threshold
-// of replica r, and which digit does it have in this pass?
-__device__ __forceinline__ bool digit_of(const InitArgs& a, uint64_t key, uint32_t i,
-                                         uint64_t pk, uint32_t pi, int& digit) {
-  const int p = a.pass;
-  if (p < 8) {
-    if (p > 0 && (key >> (64 - 8 * p)) != (pk >> (64 - 8 * p))) return false;
-    digit = (int)((key >> (56 - 8 * p)) & 0xFF);
-    return true;
-  }
-  if (key != pk) return false;
-  const int ip = p - 8;  // index byte from the top
-  const int top = a.idx_bits - 8 * ip;
-  if (ip > 0 && (i >> top) != (pi >> top)) return false;
-  digit = (int)((i >> (top - 8)) & 0xFF);
-  return true;
+// the half of replica r's block at site i
+__device__ __forceinline__ uint64_t init_key(const RoundKeys& rk, uint32_t r, uint32_t i) {
+  const uint4 b = philox(make_uint4(r >> 1, kTagInit, i, 0u), rk);
+  return (r & 1u) ? hi64(b) : lo64(b);
 }
 
-// grid: x over site chunks, y over replica pairs
-__global__ void __launch_bounds__(256) k_init_hist(const InitArgs a) {
-  __shared__ uint32_t sh[2][256];
-  const int rp = blockIdx.y;
-  if (a.pass >= 8 && *a.unresolved == 0) return;  // uniform early exit
-  for (int k = threadIdx.x; k < 512; k += blockDim.x) (&sh[0][0])[k] = 0;
-  __syncthreads();
-  const int r0 = 2 * rp;
-  const bool live0 = a.krem[r0] > 0, live1 = a.krem[r0 + 1] > 0;
-  if (live0 || live1) {
-    const uint64_t pk0 = a.pre_key[r0], pk1 = a.pre_key[r0 + 1];
-    const uint32_t pi0 = a.pre_idx[r0], pi1 = a.pre_idx[r0 + 1];
-    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x * kSitesPerThread + threadIdx.x;
-    for (int s = 0; s < kSitesPerThread; ++s) {
-      const int64_t i = i0 + (int64_t)s * blockDim.x;
-      if (i >= a.N) break;
-      const uint4 b = philox(make_uint4((uint32_t)rp, kTagInit, (uint32_t)i, 0u), a.rk);
-      int dg;
-      if (live0 && digit_of(a, lo64(b), (uint32_t)i, pk0, pi0, dg)) atomicAdd(&sh[0][dg], 1u);
-      if (live1 && digit_of(a, hi64(b), (uint32_t)i, pk1, pi1, dg)) atomicAdd(&sh[1][dg], 1u);
-    }
-  }
-  __syncthreads();
-  for (int k = threadIdx.x; k < 512; k += blockDim.x) {
-    const uint32_t c = (&sh[0][0])[k];
-    if (c) atomicAdd(&a.hist[(size_t)(r0 + (k >> 8)) * 256 + (k & 255)], c);
-  }
-}
-
-// After pass 0: collect the sites whose key has the threshold's top byte
-// (the only ones later passes can count), per replica.
-__global__ void __launch_bounds__(256) k_init_collect(const InitArgs a) {
-  const int rp = blockIdx.y;
-  const int r0 = 2 * rp;
-  const bool live0 = a.krem[r0] > 0, live1 = a.krem[r0 + 1] > 0;
-  if (!live0 && !live1) return;
-  const uint64_t top0 = a.pre_key[r0] >> 56, top1 = a.pre_key[r0 + 1] >> 56;
-  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x * kSitesPerThread + threadIdx.x;
-  for (int s = 0; s < kSitesPerThread; ++s) {
-    const int64_t i = i0 + (int64_t)s * blockDim.x;
-    if (i >= a.N) break;
-    const uint4 b = philox(make_uint4((uint32_t)rp, kTagInit, (uint32_t)i, 0u), a.rk);
-    if (live0 && (lo64(b) >> 56) == top0) {
-      const uint32_t k = atomicAdd(&a.cand_n[r0], 1u);
-      if (k < (uint64_t)a.cap) a.cand[(size_t)r0 * a.cap + k] = (uint32_t)i;
-    }
-    if (live1 && (hi64(b) >> 56) == top1) {
-      const uint32_t k = atomicAdd(&a.cand_n[r0 + 1], 1u);
-      if (k < (uint64_t)a.cap) a.cand[(size_t)(r0 + 1) * a.cap + k] = (uint32_t)i;
-    }
-  }
-}
-
-// a histogram pass over the candidate list of each replica (grid: x over
-// list chunks, y over replicas)
-__global__ void __launch_bounds__(256) k_init_hist_cand(const InitArgs a) {
-  __shared__ uint32_t sh[256];
-  const int r = blockIdx.y;
-  if (a.pass >= 8 && *a.unresolved == 0) return;  // uniform early exit
-  if (a.krem[r] <= 0) return;
-  for (int k = threadIdx.x; k < 256; k += blockDim.x) sh[k] = 0;
-  __syncthreads();
-  const int64_t n = a.cand_n[r];
-  const uint64_t pk = a.pre_key[r];
-  const uint32_t pi = a.pre_idx[r];
-  const int64_t c0 = (int64_t)blockIdx.x * blockDim.x * kSitesPerThread + threadIdx.x;
-  for (int s = 0; s < kSitesPerThread; ++s) {
-    const int64_t c = c0 + (int64_t)s * blockDim.x;
-    if (c >= n) break;
-    const uint32_t i = a.cand[(size_t)r * a.cap + c];
-    const uint4 b = philox(make_uint4((uint32_t)(r >> 1), kTagInit, i, 0u), a.rk);
-    int dg;
-    if (digit_of(a, (r & 1) ? hi64(b) : lo64(b), i, pk, pi, dg)) atomicAdd(&sh[dg], 1u);
-  }
-  __syncthreads();
-  for (int k = threadIdx.x; k < 256; k += blockDim.x) {
-    const uint32_t v = sh[k];
-    if (v) atomicAdd(&a.hist[(size_t)r * 256 + k], v);
-  }
-}
-
-// one warp per replica: pick the bucket holding rank krem, fix that digit
-__global__ void k_init_select(const InitArgs a, int R) {
-  const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (r >= R) return;
-  if (a.pass >= 8 && *a.unresolved == 0) return;
-  const int64_t want = a.krem[r];
-  uint32_t* h = a.hist + (size_t)r * 256;
-  if (want <= 0) {  // resolved replica: only clear the counters
-    for (int k = lane; k < 256; k += 32) h[k] = 0;
-    return;
-  }
-  // lane l owns buckets 8l .. 8l+7
-  uint32_t c[8];
-  int64_t mine = 0;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    c[j] = h[8 * lane + j];
-    mine += c[j];
-  }
-  int64_t incl = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int64_t v = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += v;
-  }
-  const int64_t excl = incl - mine;
-  const bool here = (excl < want) && (want <= incl);
-  const unsigned who = __ballot_sync(0xffffffffu, here);
-  const int src = __ffs(who) - 1;
-  if (lane == src) {
-    int64_t before = excl;
-    int dg = 8 * lane;
-    for (int j = 0; j < 8; ++j) {
-      if (before + c[j] >= want) {
-        dg = 8 * lane + j;
-        break;
-      }
-      before += c[j];
-    }
-    const int64_t in_bucket = c[dg - 8 * lane];
-    const int64_t rank = want - before;  // 1-based rank inside the bucket
-    const int p = a.pass;
-    if (p < 8) {
-      a.pre_key[r] |= (uint64_t)dg << (56 - 8 * p);
-      if (p == 7) {
-        if (rank == in_bucket) {
-          // every key equal to the threshold is taken: no index passes
-          a.pre_idx[r] = 0xFFFFFFFFu;
-          a.krem[r] = 0;
-        } else {
-          a.krem[r] = rank;
-          atomicOr(a.unresolved, 1);
-        }
-      } else {
-        a.krem[r] = rank;
-      }
-    } else {
-      const int top = a.idx_bits - 8 * (p - 8);
-      a.pre_idx[r] |= (uint32_t)dg << (top - 8);
-      a.krem[r] = (top - 8 == 0) ? 0 : rank;
-    }
-  }
-  __syncwarp();
-  for (int k = lane; k < 256; k += 32) h[k] = 0;
-}
-
-__global__ void k_init_rank(int64_t* krem, int R, int64_t K) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < R) krem[r] = K;
-}
-
-// one thread per (site position, word of a plane element): write n, n0, p
+// one thread per element of a plane (site position e / V, word e % V)
 template <int V>
-__global__ void __launch_bounds__(256) k_init_mark(const InitArgs a, Planes pl) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int q = blockIdx.y;
-  if (e >= a.N * V) return;
-  const int64_t i = canon_pos(pl.inv, pl.xs, e / V);  // canonical site held at this position
-  const int w = q * V + (int)(e % V);  // word index, replicas 64w .. 64w+63
-  uint64_t word = 0;
-  for (int j = 0; j < 32; ++j) {
-    const int r = 64 * w + 2 * j;
-    const uint4 b = philox(make_uint4((uint32_t)(r >> 1), kTagInit, (uint32_t)i, 0u), a.rk);
-    const uint64_t k0 = lo64(b), k1 = hi64(b);
-    const uint64_t t0 = a.pre_key[r], t1 = a.pre_key[r + 1];
-    const uint32_t x0 = a.pre_idx[r], x1 = a.pre_idx[r + 1];
-    const bool in0 = (k0 < t0) || (k0 == t0 && (uint32_t)i <= x0);
-    const bool in1 = (k1 < t1) || (k1 == t1 && (uint32_t)i <= x1);
-    word |= (uint64_t)in0 << (2 * j);
-    word |= (uint64_t)in1 << (2 * j + 1);
+__global__ void __launch_bounds__(kThreads) k_init_draw(const __grid_constant__ InitArgs a,
+                                                        const __grid_constant__ Planes pl) {
+  __shared__ uint32_t staged;
+  __shared__ uint16_t stage[kStage];  // thread << 6 | replica of the word
+  if (threadIdx.x == 0) staged = 0;
+  __syncthreads();
+  const int q = a.q0 + (int)blockIdx.y;
+  const int64_t e0 = (int64_t)blockIdx.x * kThreads;
+  const int64_t e = e0 + threadIdx.x;
+  // record bit j of thread t's word in the list of its replica
+  auto append = [&](int t, uint32_t j) {
+    const int64_t et = e0 + t;
+    const uint32_t r = (uint32_t)(q * V + (int)(et % V)) * 64u + j;
+    const uint32_t k = atomicAdd(&a.list_n[r], 1u);
+    if (k < a.cap) a.list[(size_t)(r - (uint32_t)(a.q0 * V) * 64u) * a.cap + k] = (uint32_t)(et / V);
+  };
+  if (e < pl.N * V) {
+    const uint32_t i = (uint32_t)canon_pos(pl.inv, pl.xs, e / V);  // canonical site held here
+    const uint32_t w = (uint32_t)(q * V + (int)(e % V));           // replicas 64 w .. 64 w + 63
+    uint32_t half[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      uint32_t bits = 0;
+#pragma unroll 4
+      for (uint32_t j = 0; j < 16; ++j) {
+        const uint4 b = philox(make_uint4(32u * w + 16u * (uint32_t)h + j, kTagInit, i, 0u), a.rk);
+        // the high words of the two keys
+        const bool in0 = b.y - a.lo <= a.span, in1 = b.w - a.lo <= a.span;
+        bits |= (uint32_t)(b.y < a.lo) << (2 * j) | (uint32_t)(b.w < a.lo) << (2 * j + 1);
+        if (in0 || in1) {
+          const uint32_t at = 32u * (uint32_t)h + 2 * j;
+          const uint32_t k = atomicAdd(&staged, (uint32_t)in0 + (uint32_t)in1);
+          if (k + 2 <= (uint32_t)kStage) {
+            if (in0) stage[k] = (uint16_t)(threadIdx.x << 6 | at);
+            if (in1) stage[k + in0] = (uint16_t)(threadIdx.x << 6 | (at + 1));
+          } else {
+            if (k < (uint32_t)kStage) stage[k] = 0xFFFFu;  // no room: a void entry
+            if (in0) append(threadIdx.x, at);
+            if (in1) append(threadIdx.x, at + 1);
+          }
+        }
+      }
+      half[h] = bits;
+    }
+    const size_t off = (size_t)q * pl.plane_elems() + (size_t)e;
+    pl.n[off] = (uint64_t)half[0] | (uint64_t)half[1] << 32;
+    pl.p[off] = ~0ull;
   }
-  const size_t off = (size_t)q * pl.plane_elems() + (size_t)e;
-  pl.n[off] = word;
-  pl.n0[off] = word;
-  pl.p[off] = ~0ull;
+  __syncthreads();
+  const uint32_t n = min(staged, (uint32_t)kStage);
+  for (uint32_t k = threadIdx.x; k < n; k += kThreads)
+    if (stage[k] != 0xFFFFu) append(stage[k] >> 6, stage[k] & 63u);
+}
+
+// one block per replica
+__global__ void __launch_bounds__(kSelect) k_init_select(const __grid_constant__ InitArgs a,
+                                                         const __grid_constant__ Planes pl) {
+  __shared__ uint32_t hist[kBuckets];
+  __shared__ uint64_t gkey[kSelect];
+  __shared__ uint32_t gsite[kSelect];
+  __shared__ uint32_t found, bucket, before, held, tsite;
+  __shared__ uint64_t tkey;
+  const uint32_t tid = threadIdx.x;
+  const uint32_t rl = blockIdx.x, r = (uint32_t)(a.q0 * pl.V) * 64u + rl;
+  int64_t need = a.K, m = pl.N;
+  uint64_t lo = 0, hi = ~0ull;
+  bool all = a.all;
+  if (!all) {
+    const int64_t left = a.K - (int64_t)a.below[r], in = (int64_t)a.list_n[r];
+    all = left < 1 || left > in || in > (int64_t)a.cap;
+    if (!all) {
+      need = left;
+      m = in;
+      lo = (uint64_t)a.lo << 32;
+      hi = (uint64_t)(a.lo + a.span) << 32 | 0xFFFFFFFFull;
+    }
+  }
+  const uint32_t* list = a.list + (size_t)rl * a.cap;
+  auto position = [&](int64_t k) -> int64_t { return all ? k : (int64_t)list[k]; };
+  auto site_at = [&](int64_t pos) { return (uint32_t)canon_pos(pl.inv, pl.xs, pos); };
+
+  // Narrow [lo, hi] to the bucket of the need-th smallest value until few
+  // enough keys are left to rank directly: values are keys, then (should more
+  // than kSelect keys be equal) the sites of the key `tied`.
+  bool ties = false;
+  uint64_t tied = 0;
+  auto value_in = [&](uint64_t key, uint32_t site, uint64_t& v) {
+    v = ties ? (uint64_t)site : key;
+    return (!ties || key == tied) && v >= lo && v <= hi;
+  };
+  for (;;) {
+    const int width = 64 - __clzll((long long)(hi - lo));  // bits of hi - lo
+    const int shift = width > 10 ? width - 10 : 0;
+    for (uint32_t k = tid; k < kBuckets; k += kSelect) hist[k] = 0;
+    __syncthreads();
+    for (int64_t k = tid; k < m; k += kSelect) {
+      const uint32_t site = site_at(position(k));
+      uint64_t v;
+      if (value_in(init_key(a.rk, r, site), site, v)) atomicAdd(&hist[(v - lo) >> shift], 1u);
+    }
+    __syncthreads();
+    if (tid < 32) {  // the bucket: lane l sums buckets 32 l .. 32 l + 31
+      uint32_t mine = 0;
+      for (int k = 0; k < kBuckets / 32; ++k) mine += hist[tid * (kBuckets / 32) + k];
+      uint32_t incl = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if ((int)tid >= o) incl += v;
+      }
+      uint32_t excl = incl - mine;
+      if ((int64_t)excl < need && need <= (int64_t)incl) {
+        uint32_t k = tid * (kBuckets / 32);
+        while ((int64_t)(excl + hist[k]) < need) excl += hist[k++];
+        bucket = k;
+        before = excl;
+        held = hist[k];
+      }
+    }
+    __syncthreads();
+    need -= (int64_t)before;
+    lo += (uint64_t)bucket << shift;
+    const uint64_t end = lo + ((1ull << shift) - 1);
+    if (end < hi) hi = end;
+    if (held <= (uint32_t)kSelect) break;
+    if (shift == 0) {
+      ties = true;
+      tied = lo;
+      lo = 0;
+      hi = 0xFFFFFFFFull;
+    }
+    __syncthreads();
+  }
+  if (tid == 0) found = 0;
+  __syncthreads();
+  for (int64_t k = tid; k < m; k += kSelect) {
+    const uint32_t site = site_at(position(k));
+    const uint64_t key = init_key(a.rk, r, site);
+    uint64_t v;
+    if (value_in(key, site, v)) {
+      const uint32_t at = atomicAdd(&found, 1u);
+      gkey[at] = key;
+      gsite[at] = site;
+    }
+  }
+  __syncthreads();
+  if (tid < found) {
+    int64_t rank = 1;
+    for (uint32_t k = 0; k < found; ++k)
+      rank += gkey[k] < gkey[tid] || (gkey[k] == gkey[tid] && gsite[k] < gsite[tid]);
+    if (rank == need) {
+      tkey = gkey[tid];
+      tsite = gsite[tid];
+    }
+  }
+  __syncthreads();
+  // the sites up to the threshold (of all sites: also none beyond it)
+  const uint32_t w = r >> 6;
+  unsigned long long* n = reinterpret_cast<unsigned long long*>(
+      pl.n + (size_t)(w / (uint32_t)pl.V) * pl.plane_elems() + w % (uint32_t)pl.V);
+  const unsigned long long bit = 1ull << (r & 63u);
+  for (int64_t k = tid; k < m; k += kSelect) {
+    const int64_t pos = position(k);
+    const uint32_t site = site_at(pos);
+    const uint64_t key = init_key(a.rk, r, site);
+    if (key < tkey || (key == tkey && site <= tsite))
+      atomicOr(n + pos * pl.V, bit);
+    else if (all)
+      atomicAnd(n + pos * pl.V, ~bit);
+  }
+}
+
+// half the window in sites: 6 standard deviations of the number of keys below K / N
+double window_sites(int64_t N, int64_t K) {
+  const double f = (double)K / (double)N;
+  return 6.0 * std::sqrt((double)K * (1.0 - f)) + 8.0;
 }
 
 }  // namespace
+
+// entries of a replica's list: its mean at density 1/2 and 8 deviations
+int64_t init_list_cap(int64_t N) {
+  if (N < kListSites) return 0;
+  const double mean = 2.0 * window_sites(N, N / 2);
+  return (int64_t)(mean + 8.0 * std::sqrt(mean)) + 32;
+}
 
 cudaError_t launch_init(const Planes& pl, const InitScratch& s, int R, int64_t K,
                         const RoundKeys& rk, cudaStream_t st) {
@@ -251,80 +254,45 @@ cudaError_t launch_init(const Planes& pl, const InitScratch& s, int R, int64_t K
     if ((err = cudaMemsetAsync(pl.n0, fill, bytes, st)) != cudaSuccess) return err;
     return cudaMemsetAsync(pl.p, 0xFF, bytes, st);
   }
-  InitArgs a;
-  a.hist = s.hist;
-  a.pre_key = s.pre_key;
-  a.pre_idx = s.pre_idx;
-  a.krem = s.krem;
-  a.unresolved = s.unresolved;
-  a.N = pl.N;
-  int bits = 1;
-  while (bits < 32 && ((int64_t)1 << bits) < pl.N) ++bits;
-  a.idx_bits = ((bits + 7) / 8) * 8;
+  InitArgs a{};
+  a.K = K;
   a.rk = rk;
-  // threshold state: rank K, nothing decided
-  if ((err = cudaMemsetAsync(s.hist, 0, (size_t)R * 256 * sizeof(uint32_t), st))) return err;
-  if ((err = cudaMemsetAsync(s.pre_key, 0, (size_t)R * sizeof(uint64_t), st))) return err;
-  if ((err = cudaMemsetAsync(s.pre_idx, 0, (size_t)R * sizeof(uint32_t), st))) return err;
-  if ((err = cudaMemsetAsync(s.unresolved, 0, sizeof(int32_t), st))) return err;
-  k_init_rank<<<(R + 255) / 256, 256, 0, st>>>(s.krem, R, K);
-  if ((err = cudaGetLastError())) return err;
-
-  const int64_t chunk = 256LL * kSitesPerThread;
-  dim3 hgrid((unsigned)((pl.N + chunk - 1) / chunk), (unsigned)(R / 2));
-  const int passes = 8 + a.idx_bits / 8;
-  // candidate lists: about N / 256 entries expected per replica; take them
-  // when the room holds N / 128 + 1024 (a list longer than that falls back)
-  a.cand_n = nullptr;
-  a.cand = nullptr;
-  a.cap = 0;
-  bool lists = false;
-  if (s.cand && pl.N >= 65536) {
-    const int64_t room = (int64_t)(s.cand_bytes / sizeof(uint32_t)) - R;
-    const int64_t cap = room / R;
-    if (cap >= pl.N / 128 + 1024) {
-      a.cand_n = s.cand;
-      a.cand = s.cand + R;
-      a.cap = cap;
-      lists = true;
-    }
-  }
-  for (int p = 0; p < passes; ++p) {
-    a.pass = p;
-    if (lists && p == 1) {
-      // collect the candidates of every replica, then check the lists fit
-      if ((err = cudaMemsetAsync(a.cand_n, 0, (size_t)R * sizeof(uint32_t), st))) return err;
-      k_init_collect<<<hgrid, 256, 0, st>>>(a);
+  a.list_n = s.list_n;
+  a.list = s.list;
+  a.below = s.below;
+  a.cap = (uint32_t)init_list_cap(pl.N);
+  a.all = a.cap == 0;
+  if (a.all) {
+    if ((err = cudaMemsetAsync(pl.p, 0xFF, bytes, st))) return err;
+    k_init_select<<<R, kSelect, 0, st>>>(a, pl);
+    if ((err = cudaGetLastError())) return err;
+  } else {
+    const double h = window_sites(pl.N, K), unit = 4294967296.0 / (double)pl.N;
+    const double lo = std::max(0.0, std::floor(((double)K - h) * unit));
+    const double hi = std::min(4294967295.0, std::ceil(((double)K + h) * unit));
+    a.lo = (uint32_t)lo;
+    a.span = (uint32_t)hi - a.lo;
+    if ((err = cudaMemsetAsync(s.list_n, 0, (size_t)R * sizeof(uint32_t), st))) return err;
+    // as many planes at a time as there is room for their lists
+    const size_t plane_list = (size_t)64 * pl.V * a.cap * sizeof(uint32_t);
+    const int most = (int)std::max<size_t>(1, std::min<size_t>((size_t)pl.P, s.list_bytes / plane_list));
+    for (int q = 0; q < pl.P; q += most) {
+      const int nq = std::min(most, pl.P - q);
+      a.q0 = q;
+      const dim3 grid((unsigned)((pl.N * pl.V + kThreads - 1) / kThreads), (unsigned)nq);
+      if (pl.V == 4)
+        k_init_draw<4><<<grid, kThreads, 0, st>>>(a, pl);
+      else if (pl.V == 2)
+        k_init_draw<2><<<grid, kThreads, 0, st>>>(a, pl);
+      else
+        k_init_draw<1><<<grid, kThreads, 0, st>>>(a, pl);
       if ((err = cudaGetLastError())) return err;
-      std::vector<uint32_t> counts(R);
-      if ((err = cudaMemcpyAsync(counts.data(), a.cand_n, (size_t)R * sizeof(uint32_t),
-                                 cudaMemcpyDeviceToHost, st)))
-        return err;
-      if ((err = cudaStreamSynchronize(st))) return err;
-      int64_t longest = 0;
-      for (uint32_t c : counts) longest = std::max<int64_t>(longest, c);
-      lists = longest <= a.cap;
+      if ((err = launch_particles(pl, q, nq, s.below, st))) return err;
+      k_init_select<<<nq * 64 * pl.V, kSelect, 0, st>>>(a, pl);
+      if ((err = cudaGetLastError())) return err;
     }
-    if (lists && p >= 1) {
-      const int64_t cchunk = 256LL * kSitesPerThread;
-      const unsigned cx = (unsigned)std::max<int64_t>(1, (a.cap + cchunk - 1) / cchunk);
-      // the grid covers the capacity; blocks past a replica's count return at once
-      k_init_hist_cand<<<dim3(cx, (unsigned)R), 256, 0, st>>>(a);
-    } else {
-      k_init_hist<<<hgrid, 256, 0, st>>>(a);
-    }
-    if ((err = cudaGetLastError())) return err;
-    k_init_select<<<(R + 7) / 8, 256, 0, st>>>(a, R);
-    if ((err = cudaGetLastError())) return err;
   }
-  dim3 mgrid((unsigned)((pl.N * pl.V + 255) / 256), (unsigned)pl.P);
-  if (pl.V == 4)
-    k_init_mark<4><<<mgrid, 256, 0, st>>>(a, pl);
-  else if (pl.V == 2)
-    k_init_mark<2><<<mgrid, 256, 0, st>>>(a, pl);
-  else
-    k_init_mark<1><<<mgrid, 256, 0, st>>>(a, pl);
-  return cudaGetLastError();
+  return cudaMemcpyAsync(pl.n0, pl.n, bytes, cudaMemcpyDeviceToDevice, st);
 }
 
 }  // namespace ka

@@ -224,17 +224,17 @@ cudaError_t launch_graph_class_batch(const GraphUnit* units_dev, const int64_t* 
                                      int V, int m, uint32_t cls, uint32_t sweep_offset,
                                      cudaStream_t s);
 
+// Scratch of the initial state: the lists of replicas' candidate sites (room
+// for those of one plane at least; ka_init.cu), their lengths, and the
+// particles below the candidates' window.
 struct InitScratch {
-  uint32_t* hist;      // [R][256]
-  uint64_t* pre_key;   // [R] decided high bits of the threshold key
-  uint32_t* pre_idx;   // [R] decided high bits of the threshold site
-  int64_t* krem;       // [R] rank still to place inside the current bucket
-  int32_t* unresolved; // [1] any replica whose threshold key is tied
-  // optional: room for per-replica candidate lists (the staging plane, idle
-  // during init); null or too small -> every pass scans all sites
-  uint32_t* cand;
-  size_t cand_bytes;
+  uint32_t* list;
+  size_t list_bytes;
+  uint32_t* list_n;           // [R]
+  unsigned long long* below;  // [R]
 };
+// entries per replica of those lists, 0 if a lattice of N sites needs none
+int64_t init_list_cap(int64_t N);
 cudaError_t launch_init(const Planes& pl, const InitScratch& s, int R, int64_t K,
                         const RoundKeys& rk, cudaStream_t st);
 
