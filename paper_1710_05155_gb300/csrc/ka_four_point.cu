@@ -10,190 +10,199 @@
 //   psi[s]    = sum over pairs in shell s of M_i M_j,  M_i = sum_r q_i^r
 // (psi gives the <q_i><q_j> term of g_4).
 //
-// phi: one launch per shell; a thread takes a few site-words (site i, word
-// h of plane q) and all vectors of the shell, and adds q_i & q_{i+delta}
-// into bit-sliced counters (all 64 replicas of the word at once); lanes of
-// the same word position are summed by warp shuffles, then per block in
-// shared memory, then one atomic per (replica, shell).  psi: the per-site
-// counts M_i are computed once, then a thread per site sums M_i M_{i+delta}
-// over the shell's vectors.
+// The sums for delta and -delta are equal, so one of the two is run with
+// weight 2.  q (and M) are first written as words in site order with a margin
+// of the largest component on every side, filled periodically: site i + delta
+// is then a fixed offset from i for all sites, and neighbouring threads read
+// neighbouring words.  A thread takes eight sites and, shell by shell, adds
+// q_i & q_{i + delta} for all of them into bit-sliced counters, eight words at
+// a time (ka_count.cuh); a block sums a shell's counters in shared memory and
+// adds 64 integers to phi.  One launch covers all shells; small lattices
+// split the vectors over more blocks.
+//
+// Bound by the ALUs: about 12 instructions per site-word and vector (the
+// adders 5, the AND 2, the load and its address 2, the sums over lanes the
+// rest).  L = 64, 256 replicas, smax = 25 (515 vectors), the whole call: 4.56 ms
+// before, when each shell was a launch and a thread worked out periodic
+// coordinates for each vector; 0.50 ms now.
 #include <algorithm>
 #include <string>
 #include <vector>
 
+#include "ka_count.cuh"
 #include "ka_ctx.cuh"
 
 namespace ka {
 namespace {
 
-constexpr int kSlices = 8;            // per-thread counters hold up to 255
-constexpr int kWide = kSlices + 5;    // after summing 32 lanes
+constexpr int kDigits = 7;            // per-thread counters hold up to 127
+constexpr int kSites = 8;             // sites per thread
+constexpr int kSegment = 15;          // vectors per segment: 120 words per thread
+constexpr int kThreads = 256;
 constexpr int kMaxVectors = 1 << 16;  // displacement vectors per call
+// Scratch when the context's staging plane does not hold one word's padded
+// lattice: this much, or one word's, a slab of layers at a time.
+constexpr size_t kArena = (size_t)256 << 20;
 
-struct Vec {
-  int16_t dx[4];
+// Vectors of one shell and weight: offsets [first, first + count).
+struct Segment {
+  int shell, first, count, weight;
 };
 
-struct Geometry {
-  int d, L;
-  int64_t st[4];  // L^k
+// A slab of the padded lattice: layers z0 .. z0 + zc - 1 of the last dimension
+// with a margin of rad all round.
+struct Slab {
+  int d, L, rad, z0, zc;
+  int64_t ps[4];     // strides of the padded lattice
+  int64_t padded;    // its elements
+  int64_t sites;     // sites of the slab
 };
 
-__device__ __forceinline__ void ripple_add(uint64_t (&c)[kSlices], uint64_t x) {
+// storage position of the site that padded element k shows
+__device__ __forceinline__ int64_t shown(const Slab& g, int xs, int64_t k) {
+  int64_t site = 0, stride = 1;
 #pragma unroll
-  for (int s = 0; s < kSlices; ++s) {
-    const uint64_t k = c[s] & x;
-    c[s] ^= x;
-    x = k;
-  }
-}
-
-__device__ __forceinline__ void shfl_add(uint64_t (&c)[kWide], int off) {
-  uint64_t carry = 0;
-#pragma unroll
-  for (int s = 0; s < kWide; ++s) {
-    const uint64_t o = __shfl_xor_sync(0xffffffffu, c[s], off);
-    const uint64_t sum = c[s] ^ o ^ carry;
-    carry = (c[s] & o) | (carry & (c[s] | o));
-    c[s] = sum;
-  }
-}
-
-// site index of (coordinates of i) + delta, periodic
-__device__ __forceinline__ int64_t shifted(const Geometry& g, const int (&x)[4], const Vec& v) {
-  int64_t j = 0;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    if (k < g.d) {
-      int y = x[k] + v.dx[k];
-      y += (y < 0) ? g.L : 0;
-      y -= (y >= g.L) ? g.L : 0;
-      j += (int64_t)y * g.st[k];
+  for (int m = 0; m < 4; ++m) {
+    if (m < g.d) {
+      const int64_t extent = m == g.d - 1 ? g.zc + 2 * g.rad : g.L + 2 * g.rad;
+      int64_t x = k % extent - g.rad + (m == g.d - 1 ? g.z0 : 0);
+      k /= extent;
+      x += x < 0 ? g.L : 0;
+      x -= x >= g.L ? g.L : 0;
+      site += x * stride;
+      stride *= g.L;
     }
   }
-  return j;
+  return dev_site(xs, site);
 }
 
-__device__ __forceinline__ void coords(const Geometry& g, int64_t i, int (&x)[4]) {
+// padded element of the slab's site k
+__device__ __forceinline__ int64_t centre(const Slab& g, int64_t k) {
+  int64_t e = 0;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    x[k] = 0;
-    if (k < g.d) {
-      x[k] = (int)(i % g.L);
-      i /= g.L;
+  for (int m = 0; m < 4; ++m) {
+    if (m < g.d) {
+      const int64_t x = m == g.d - 1 ? k : k % g.L;
+      if (m < g.d - 1) k /= g.L;
+      e += (x + g.rad) * g.ps[m];
     }
   }
+  return e;
 }
 
-// phi of one shell: vectors [v0, v1) of the table, `spt` site-words per
-// thread, plane blockIdx.y
-template <int V>
-__global__ void __launch_bounds__(256) k_phi(Planes pl, Geometry g, const Vec* __restrict__ vec,
-                                             int v0, int v1, int spt, int shell, int nshell,
-                                             unsigned long long* phi) {
-  __shared__ unsigned int acc[64 * V];
-  for (int k = threadIdx.x; k < 64 * V; k += blockDim.x) acc[k] = 0;
-  __syncthreads();
-  const int q = blockIdx.y;
-  const size_t E = pl.plane_elems();
-  const uint64_t* n = pl.n + (size_t)q * E;
-  const uint64_t* n0 = pl.n0 + (size_t)q * E;
-  uint64_t c[kSlices];
-#pragma unroll
-  for (int s = 0; s < kSlices; ++s) c[s] = 0;
-  // element e = site * V + h; the stride (blockDim) is a multiple of V, so
-  // a thread always sees the same word position h
-  const size_t e0 = (size_t)blockIdx.x * blockDim.x * spt + threadIdx.x;
-  for (int k = 0; k < spt; ++k) {
-    const size_t e = e0 + (size_t)k * blockDim.x;
-    if (e >= E) break;
-    const int64_t i = canon_site(pl.xs, (int64_t)(e / V));  // the site held at element e
-    const int h = (int)(e % V);
-    const uint64_t qi = n[e] & n0[e];
-    if (qi == 0) continue;
-    int x[4];
-    coords(g, i, x);
-    for (int t = v0; t < v1; ++t) {
-      const int64_t j = shifted(g, x, vec[t]);
-      const size_t f = (size_t)dev_site(pl.xs, j) * V + h;
-      ripple_add(c, qi & n[f] & n0[f]);
-    }
-  }
-  const int lane = threadIdx.x & 31;
-  uint64_t w[kWide];
-#pragma unroll
-  for (int s = 0; s < kWide; ++s) w[s] = (s < kSlices) ? c[s] : 0;
-#pragma unroll
-  for (int off = 16; off >= V; off >>= 1) shfl_add(w, off);
-  // lanes 0 .. V-1 hold the warp totals of word positions 0 .. V-1; every
-  // lane extracts replicas (bits) lane and lane + 32 of each
-#pragma unroll
-  for (int hh = 0; hh < V; ++hh) {
-    unsigned int lo = 0, hi = 0;
-#pragma unroll
-    for (int s = 0; s < kWide; ++s) {
-      const uint64_t t = __shfl_sync(0xffffffffu, w[s], hh);
-      lo |= (unsigned int)((t >> lane) & 1u) << s;
-      hi |= (unsigned int)((t >> (lane + 32)) & 1u) << s;
-    }
-    if (lo) atomicAdd(&acc[hh * 64 + lane], lo);
-    if (hi) atomicAdd(&acc[hh * 64 + lane + 32], hi);
-  }
-  __syncthreads();
-  for (int k = threadIdx.x; k < 64 * V; k += blockDim.x) {
-    const unsigned int v = acc[k];
-    if (v) {
-      const int r = (q * V + k / 64) * 64 + (k % 64);
-      atomicAdd(&phi[(size_t)r * nshell + shell], (unsigned long long)v);
-    }
-  }
+// q = n & n0 of words w0 .. w0 + gridDim.y - 1, padded
+__global__ void __launch_bounds__(kThreads) k_pad(const __grid_constant__ Planes pl,
+                                                  const __grid_constant__ Slab g, int w0,
+                                                  uint64_t* __restrict__ out) {
+  const int64_t k = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  if (k >= g.padded) return;
+  const int w = w0 + (int)blockIdx.y;
+  const size_t e = (size_t)(w / pl.V) * pl.plane_elems() + (size_t)shown(g, pl.xs, k) * pl.V + w % pl.V;
+  out[(size_t)blockIdx.y * g.padded + k] = pl.n[e] & pl.n0[e];
 }
 
-// M_i = number of replicas with q_i = 1
-template <int V>
-__global__ void k_site_counts(Planes pl, uint32_t* M) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= pl.N) return;
-  const size_t E = pl.plane_elems();
+// M = number of replicas with q = 1, padded
+__global__ void __launch_bounds__(kThreads) k_pad_counts(const __grid_constant__ Planes pl,
+                                                         const __grid_constant__ Slab g,
+                                                         uint32_t* __restrict__ M) {
+  const int64_t k = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  if (k >= g.padded) return;
+  const size_t at = (size_t)shown(g, pl.xs, k) * pl.V;
   uint32_t m = 0;
-  for (int q = 0; q < pl.P; ++q)
-#pragma unroll
-    for (int h = 0; h < V; ++h) {
-      const size_t e = (size_t)q * E + (size_t)dev_site(pl.xs, i) * V + h;
-      m += (uint32_t)__popcll(pl.n[e] & pl.n0[e]);
-    }
-  M[i] = m;
+  for (int w = 0; w < pl.W; ++w) {
+    const size_t e = (size_t)(w / pl.V) * pl.plane_elems() + at + w % pl.V;
+    m += (uint32_t)__popcll(pl.n[e] & pl.n0[e]);
+  }
+  M[k] = m;
 }
 
-// psi of one shell: a thread per site, all vectors of the shell
-__global__ void __launch_bounds__(256) k_psi(Geometry g, int64_t N, const uint32_t* __restrict__ M,
-                                             const Vec* __restrict__ vec, int v0, int v1,
-                                             unsigned long long* psi_s) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned long long acc = 0;
-  if (i < N && M[i] != 0) {
-    int x[4];
-    coords(g, i, x);
-    unsigned long long sum = 0;
-    for (int t = v0; t < v1; ++t) sum += M[shifted(g, x, vec[t])];
-    acc = sum * M[i];
-  }
+// phi of words w0 + blockIdx.y over the segments of blockIdx.z
+__global__ void __launch_bounds__(kThreads) k_phi(const __grid_constant__ Slab g,
+                                                  const uint64_t* __restrict__ padded,
+                                                  const Segment* __restrict__ seg,
+                                                  const int32_t* __restrict__ offset, int nseg,
+                                                  int w0, int nshell, unsigned long long* phi) {
+  __shared__ unsigned int acc[64];
+  const uint64_t* q = padded + (size_t)blockIdx.y * g.padded;
+  const int64_t s0 = (int64_t)blockIdx.x * (kThreads * kSites) + threadIdx.x;
+  int32_t at[kSites];
+  uint64_t own[kSites];
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  __shared__ unsigned long long part[8];
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+  for (int u = 0; u < kSites; ++u) {
+    const int64_t s = s0 + u * kThreads;
+    const bool in = s < g.sites;
+    at[u] = (int32_t)centre(g, in ? s : 0);
+    own[u] = in ? q[at[u]] : 0ull;
+  }
+  const int b0 = (int)((int64_t)nseg * blockIdx.z / gridDim.z);
+  const int b1 = (int)((int64_t)nseg * (blockIdx.z + 1) / gridDim.z);
+  if (threadIdx.x < 64) acc[threadIdx.x] = 0;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long s = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += part[w];
-    if (s) atomicAdd(psi_s, s);
+  for (int b = b0; b < b1; ++b) {
+    const Segment sg = seg[b];
+    uint64_t c[kDigits];
+#pragma unroll
+    for (int s = 0; s < kDigits; ++s) c[s] = 0;
+    for (int v = 0; v < sg.count; ++v) {
+      const int32_t off = __ldg(offset + sg.first + v);
+      uint64_t x[kSites];
+#pragma unroll
+      for (int u = 0; u < kSites; ++u) x[u] = __ldg(q + (at[u] + off));
+#pragma unroll
+      for (int u = 0; u < kSites; ++u) x[u] &= own[u];
+      add8(c, x);
+    }
+    reduce<1, kDigits>(c, acc, (unsigned)sg.weight);
+    if (b + 1 == b1 || seg[b + 1].shell != sg.shell) {
+      __syncthreads();
+      if (threadIdx.x < 64) {
+        const unsigned int v = acc[threadIdx.x];
+        acc[threadIdx.x] = 0;
+        if (v)
+          atomicAdd(&phi[((size_t)(w0 + (int)blockIdx.y) * 64 + threadIdx.x) * nshell + sg.shell],
+                    (unsigned long long)v);
+      }
+      __syncthreads();
+    }
   }
 }
 
-}  // namespace
-}  // namespace ka
-
-namespace {
+// psi over the segments of blockIdx.z
+__global__ void __launch_bounds__(kThreads) k_psi(const __grid_constant__ Slab g,
+                                                  const uint32_t* __restrict__ M,
+                                                  const Segment* __restrict__ seg,
+                                                  const int32_t* __restrict__ offset, int nseg,
+                                                  unsigned long long* psi) {
+  const int64_t s0 = (int64_t)blockIdx.x * (kThreads * kSites) + threadIdx.x;
+  int32_t at[kSites];
+  uint32_t own[kSites];
+#pragma unroll
+  for (int u = 0; u < kSites; ++u) {
+    const int64_t s = s0 + u * kThreads;
+    const bool in = s < g.sites;
+    at[u] = (int32_t)centre(g, in ? s : 0);
+    own[u] = in ? M[at[u]] : 0u;
+  }
+  const int b0 = (int)((int64_t)nseg * blockIdx.z / gridDim.z);
+  const int b1 = (int)((int64_t)nseg * (blockIdx.z + 1) / gridDim.z);
+  unsigned long long sum = 0;
+  for (int b = b0; b < b1; ++b) {
+    const Segment sg = seg[b];
+    unsigned long long part = 0;
+    for (int v = 0; v < sg.count; ++v) {
+      const int32_t off = __ldg(offset + sg.first + v);
+#pragma unroll
+      for (int u = 0; u < kSites; ++u) part += (unsigned long long)own[u] * __ldg(M + (at[u] + off));
+    }
+    sum += part * (unsigned)sg.weight;
+    if (b + 1 == b1 || seg[b + 1].shell != sg.shell) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if ((threadIdx.x & 31) == 0 && sum) atomicAdd(psi + sg.shell, sum);
+      sum = 0;
+    }
+  }
+}
 
 struct Scope {
   int prev = -1;
@@ -214,6 +223,7 @@ ka_status four_point_fail(ka_ctx* c, ka_status st, const std::string& msg) {
 }
 
 }  // namespace
+}  // namespace ka
 
 extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_t* psi) {
   ka::NvtxRange nvtx_range("ka_four_point");
@@ -226,99 +236,133 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
   const int d = c->d, L = c->L, half = L / 2;
   if ((int64_t)smax > (int64_t)d * half * half)
     return four_point_fail(c, KA_EINVAL, "smax above d (L/2)^2, the largest shell");
-  // representative displacement vectors (components in [-L/2, L/2)) by shell
+  // representative displacement vectors (components in [-L/2, L/2))
   int rad = 0;
   while ((int64_t)(rad + 1) * (rad + 1) <= smax) ++rad;
-  const int lo = -std::min(rad, half), hi = std::min(rad, half - 1);
+  rad = std::min(rad, half);
+  const int lo = -rad, hi = std::min(rad, half - 1);
   const int S = smax + 1;
-  std::vector<std::vector<Vec>> shell(S);
+
+  // The padded lattice, a slab of its last dimension at a time if one word of
+  // the whole is too large, and where it is kept: the staging plane (idle
+  // here) if that holds a word of it and the rest, else an allocation.
+  Slab g{};
+  g.d = d;
+  g.L = L;
+  g.rad = rad;
+  g.ps[0] = 1;
+  for (int k = 1; k < 4; ++k) g.ps[k] = g.ps[k - 1] * (L + 2 * rad);
+  const int64_t layer = g.ps[d - 1];
+  const int64_t layer_sites = c->N / L;
+  const int64_t most = std::min<int64_t>((int64_t)1 << 30, (int64_t)(kArena / sizeof(uint64_t)));
+  const size_t stage_bytes = c->stage ? (size_t)c->N * c->pl.W * sizeof(uint64_t) : 0;
+
+  struct Vec {
+    int32_t shell, offset, weight;
+  };
+  std::vector<Vec> vecs;
   int64_t nvec = 0;
   int x[4] = {lo, lo, lo, lo};
   for (int k = d; k < 4; ++k) x[k] = 0;
   for (;;) {
-    int64_t s2 = 0;
-    for (int k = 0; k < d; ++k) s2 += (int64_t)x[k] * x[k];
+    int64_t s2 = 0, off = 0;
+    int sign = 0;  // of the first component that is not its own negative
+    for (int k = 0; k < d; ++k) {
+      s2 += (int64_t)x[k] * x[k];
+      off += x[k] * g.ps[k];
+      if (!sign && x[k] != 0 && x[k] != -half) sign = x[k] > 0 ? 1 : -1;
+    }
     if (s2 <= smax) {
-      Vec v{};
-      for (int k = 0; k < 4; ++k) v.dx[k] = (int16_t)x[k];
-      shell[s2].push_back(v);
       if (++nvec > kMaxVectors)
         return four_point_fail(c, KA_EINVAL, "more than 65536 displacement vectors: lower smax");
+      if (sign >= 0) vecs.push_back({(int32_t)s2, (int32_t)off, sign ? 2 : 1});
     }
     int k = 0;
     while (k < d && x[k] == hi) x[k++] = lo;
     if (k == d) break;
     ++x[k];
   }
-  std::vector<Vec> table;
-  std::vector<int> off(S + 1, 0);
-  for (int s2 = 0; s2 < S; ++s2) {
-    off[s2] = (int)table.size();
-    table.insert(table.end(), shell[s2].begin(), shell[s2].end());
+  std::stable_sort(vecs.begin(), vecs.end(), [](const Vec& a, const Vec& b) {
+    return a.shell != b.shell ? a.shell < b.shell : a.weight < b.weight;
+  });
+  std::vector<int32_t> offsets;
+  std::vector<Segment> segs;
+  for (const Vec& v : vecs) {
+    if (segs.empty() || segs.back().shell != v.shell || segs.back().weight != v.weight ||
+        segs.back().count == kSegment)
+      segs.push_back({v.shell, (int)offsets.size(), 0, v.weight});
+    ++segs.back().count;
+    offsets.push_back(v.offset);
   }
-  off[S] = (int)table.size();
+  const int nseg = (int)segs.size();
 
   Scope scope(c->device);
   const cudaStream_t st = c->stream;
-  const int R = c->R;
+  const int R = c->R, W = c->pl.W;
   const size_t phi_bytes = (size_t)R * S * sizeof(unsigned long long);
   const size_t psi_bytes = (size_t)S * sizeof(unsigned long long);
-  const size_t m_bytes = psi ? (size_t)c->N * sizeof(uint32_t) : 0;
-  const size_t v_bytes = std::max<size_t>(table.size(), 1) * sizeof(Vec);
-  const size_t a = 256;
-  auto up = [&](size_t b) { return (b + a - 1) / a * a; };
-  const size_t total = up(phi_bytes) + up(psi_bytes) + up(m_bytes) + up(v_bytes);
+  const size_t seg_bytes = segs.size() * sizeof(Segment), off_bytes = offsets.size() * sizeof(int32_t);
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  const size_t fixed = up(phi_bytes) + up(psi_bytes) + up(seg_bytes) + up(off_bytes);
+  auto m_bytes = [&](int64_t zc) { return psi ? up((size_t)(layer * (zc + 2 * rad)) * sizeof(uint32_t)) : 0; };
+  auto q_bytes = [&](int64_t zc) { return up((size_t)(layer * (zc + 2 * rad)) * sizeof(uint64_t)); };
+  int64_t zc = L;
+  int words = 0;  // per pass
+  char* own = nullptr;
   char* mem = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&mem, total, st);
-  if (e) return four_point_fail(c, KA_ENOMEM, std::string("scratch: ") + cudaGetErrorString(e));
+  if (layer * (L + 2 * rad) <= (int64_t)1 << 30 && stage_bytes >= fixed + m_bytes(L) + q_bytes(L)) {
+    mem = (char*)c->stage;
+    words = (int)std::min<size_t>((size_t)W, (stage_bytes - fixed - m_bytes(L)) / q_bytes(L));
+  } else {
+    if (layer * (zc + 2 * rad) > most) zc = std::max<int64_t>(1, most / layer - 2 * rad);
+    if (layer * (zc + 2 * rad) >= (int64_t)1 << 31)
+      return four_point_fail(c, KA_ENOMEM, "scratch: a padded layer is too large");
+    words = (int)std::max<size_t>(1, std::min<size_t>((size_t)W, kArena / q_bytes(zc)));
+    const size_t total = fixed + m_bytes(zc) + (size_t)words * q_bytes(zc);
+    const cudaError_t ea = cudaMallocAsync((void**)&own, total, st);
+    if (ea) return four_point_fail(c, KA_ENOMEM, std::string("scratch: ") + cudaGetErrorString(ea));
+    mem = own;
+  }
   unsigned long long* phi_dev = (unsigned long long*)mem;
   unsigned long long* psi_dev = (unsigned long long*)(mem + up(phi_bytes));
-  uint32_t* M = (uint32_t*)(mem + up(phi_bytes) + up(psi_bytes));
-  Vec* vec = (Vec*)(mem + up(phi_bytes) + up(psi_bytes) + up(m_bytes));
-  e = cudaMemsetAsync(mem, 0, up(phi_bytes) + up(psi_bytes), st);
-  if (!e && !table.empty())
-    e = cudaMemcpyAsync(vec, table.data(), table.size() * sizeof(Vec), cudaMemcpyHostToDevice, st);
-  Geometry g{};
-  g.d = d;
-  g.L = L;
-  g.st[0] = 1;
-  for (int k = 1; k < 4; ++k) g.st[k] = g.st[k - 1] * L;
+  Segment* seg_dev = (Segment*)(mem + up(phi_bytes) + up(psi_bytes));
+  int32_t* off_dev = (int32_t*)((char*)seg_dev + up(seg_bytes));
+  uint32_t* M = (uint32_t*)(mem + fixed);
+  uint64_t* q = (uint64_t*)(mem + fixed + m_bytes(zc));
+  cudaError_t e = cudaMemsetAsync(mem, 0, up(phi_bytes) + up(psi_bytes), st);
+  if (!e) e = cudaMemcpyAsync(seg_dev, segs.data(), seg_bytes, cudaMemcpyHostToDevice, st);
+  if (!e) e = cudaMemcpyAsync(off_dev, offsets.data(), off_bytes, cudaMemcpyHostToDevice, st);
   const Planes& pl = c->pl;
-  const size_t E = pl.plane_elems();
-  if (!e && psi) {
-    const unsigned blocks = (unsigned)((c->N + 255) / 256);
-    if (pl.V == 4)
-      k_site_counts<4><<<blocks, 256, 0, st>>>(pl, M);
-    else if (pl.V == 2)
-      k_site_counts<2><<<blocks, 256, 0, st>>>(pl, M);
-    else
-      k_site_counts<1><<<blocks, 256, 0, st>>>(pl, M);
-    e = cudaGetLastError();
-  }
-  for (int s2 = 0; s2 < S && !e; ++s2) {
-    // chunks of at most 255 vectors keep every per-thread counter below 256
-    for (int v0 = off[s2]; v0 < off[s2 + 1] && !e; v0 += 255) {
-      const int v1 = std::min(v0 + 255, off[s2 + 1]);
-      const int spt = std::max(1, std::min(32, 255 / (v1 - v0)));
-      const dim3 grid((unsigned)((E + (size_t)256 * spt - 1) / ((size_t)256 * spt)), (unsigned)pl.P);
-      if (pl.V == 4)
-        k_phi<4><<<grid, 256, 0, st>>>(pl, g, vec, v0, v1, spt, s2, S, phi_dev);
-      else if (pl.V == 2)
-        k_phi<2><<<grid, 256, 0, st>>>(pl, g, vec, v0, v1, spt, s2, S, phi_dev);
-      else
-        k_phi<1><<<grid, 256, 0, st>>>(pl, g, vec, v0, v1, spt, s2, S, phi_dev);
+  // blocks along z share out the segments until the grid has four blocks per SM
+  auto split = [&](int64_t blocks) {
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(nseg, 4 * (int64_t)c->sms / blocks));
+  };
+  for (int64_t z0 = 0; z0 < L && !e; z0 += zc) {
+    g.z0 = (int)z0;
+    g.zc = (int)std::min<int64_t>(zc, L - z0);
+    g.padded = layer * (g.zc + 2 * rad);
+    g.sites = layer_sites * g.zc;
+    const unsigned pads = (unsigned)((g.padded + kThreads - 1) / kThreads);
+    const unsigned tiles = (unsigned)((g.sites + kThreads * kSites - 1) / (kThreads * kSites));
+    if (psi) {
+      k_pad_counts<<<pads, kThreads, 0, st>>>(pl, g, M);
+      k_psi<<<dim3(tiles, 1, split(tiles)), kThreads, 0, st>>>(g, M, seg_dev, off_dev, nseg, psi_dev);
       e = cudaGetLastError();
-      if (!e && psi) {
-        k_psi<<<(unsigned)((c->N + 255) / 256), 256, 0, st>>>(g, c->N, M, vec, v0, v1,
-                                                              psi_dev + s2);
-        e = cudaGetLastError();
-      }
+    }
+    for (int w0 = 0; w0 < W && !e; w0 += words) {
+      const unsigned nw = (unsigned)std::min(words, W - w0);
+      k_pad<<<dim3(pads, nw), kThreads, 0, st>>>(pl, g, w0, q);
+      k_phi<<<dim3(tiles, nw, split((int64_t)tiles * nw)), kThreads, 0, st>>>(g, q, seg_dev, off_dev, nseg,
+                                                                            w0, S, phi_dev);
+      e = cudaGetLastError();
     }
   }
   if (!e) e = cudaMemcpyAsync(phi, phi_dev, phi_bytes, cudaMemcpyDeviceToHost, st);
   if (!e && psi) e = cudaMemcpyAsync(psi, psi_dev, psi_bytes, cudaMemcpyDeviceToHost, st);
-  const cudaError_t ef = cudaFreeAsync(mem, st);
-  if (!e) e = ef;
+  if (own) {
+    const cudaError_t ef = cudaFreeAsync(own, st);
+    if (!e) e = ef;
+  }
   const cudaError_t es = cudaStreamSynchronize(st);
   if (!e) e = es;
   if (e) return four_point_fail(c, KA_ECUDA, std::string("four-point: ") + cudaGetErrorString(e));
