@@ -16,7 +16,8 @@
 // CTA sends in a group are read in that group by no other CTA (a cubic group
 // reads its own pencils and the inactive ones; a graph class is a strong
 // matching), and a CTA starts a group only when all others have finished
-// reading for the one before, so two mbarriers in turn are enough.  The Philox
+// reading for the one before (each sends at least a word in every group), so
+// two mbarriers in turn are enough.  The Philox
 // gate words depend on no state: those of the next group are computed between
 // arriving at the barrier and waiting for it.
 //
@@ -56,7 +57,7 @@ struct Args {
   uint32_t from, most; // run at most `most` of a unit's sweeps, from this one on
   int L;               // cubic
   int fsmem;           // the swapped bits are collected in shared memory
-  int fslots, entries; // graphs: their words; entries of a buffer (the largest class)
+  int fslots, entries; // graphs: their words; entries of a buffer
 };
 
 // threads of a CTA that has one C-th of a cubic lattice's pencils: a thread per

@@ -31,7 +31,8 @@ int cubic_cluster(int d, int L, int64_t words, int sms) {
   while (cubic_threads(N, L, C) > 1024) C *= 2;
   // fewer once the words fill the device (L = 16, 128 words: 9.2 with one, 19.8 with four)
   while (C > 1 && words * C > sms && cubic_threads(N, L, C / 2) <= 1024) C /= 2;
-  return C;
+  // every CTA has pencils: each must send in every group
+  return (C - 1) * share_of((int)(N / L / 2), C) < N / L / 2 ? C : 0;
 }
 
 cudaError_t launch_cubic(const Args& a, int d, int L, int m, unsigned words, int C,

@@ -54,9 +54,9 @@ __global__ void __launch_bounds__(1024) k_resident_graph(const __grid_constant__
   constexpr int RW = Z / 4;  // 16-byte pieces of a record
   extern __shared__ __align__(16) unsigned char dsm[];
   __shared__ Unit su;
-  // class c: bonds [coff[c], coff[c + 1]), share[c] of them per CTA at most; the
-  // swapped bits of this CTA's are kept from slot[c] on
-  __shared__ int32_t coff[kMaxClasses + 1], share[kMaxClasses], slot[kMaxClasses];
+  // class c: bonds [coff[c], coff[c + 1]), share[c] of them per CTA at most, idle[c]
+  // CTAs without any; the swapped bits of this CTA's are kept from slot[c] on
+  __shared__ int32_t coff[kMaxClasses + 1], share[kMaxClasses], slot[kMaxClasses], idle[kMaxClasses];
   __shared__ __align__(8) uint64_t bars[2];
   const uint32_t rank = cluster_rank();
   unit_of<B>(a, blockIdx.x / C, su);
@@ -74,7 +74,11 @@ __global__ void __launch_bounds__(1024) k_resident_graph(const __grid_constant__
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   for (int c = tid; c <= nclass; c += blockDim.x) {
     coff[c] = su.coff[c];
-    if (c < nclass) share[c] = (su.coff[c + 1] - su.coff[c] + C - 1) / C;
+    if (c < nclass) {
+      const int count = su.coff[c + 1] - su.coff[c];
+      share[c] = (count + C - 1) / C;
+      idle[c] = C - (count + share[c] - 1) / share[c];
+    }
   }
   load_plane(su, n, N);
   if (tid == 0) n[N] = 0;  // the word of missing neighbours
@@ -153,7 +157,13 @@ __global__ void __launch_bounds__(1024) k_resident_graph(const __grid_constant__
         if constexpr (C > 1)
           peers.st(smem_addr(in + first(c, (int)rank) - coff[c] + tid), sw, ge.bar());
       }
-      ge.arrive((uint32_t)(coff[c + 1] - coff[c] - mine(c, (int)rank)) * 8u);
+      // a CTA without a bond in the class sends a word all the same: the
+      // others must not run two classes ahead of it
+      const int own = mine(c, (int)rank);
+      if constexpr (C > 1) {
+        if (own == 0 && tid == 0) peers.st(smem_addr(in + a.entries - C + (int)rank), 0ull, ge.bar());
+      }
+      ge.arrive((uint32_t)(coff[c + 1] - coff[c] - own + idle[c] - (own == 0)) * 8u);
       if (act) {
         if (fsmem) {
           f[slot[c] + tid] |= sw;
@@ -235,12 +245,15 @@ cudaError_t launch_z(const Args& a, int m, unsigned words, int C, int threads, s
 
 // shared memory: entry buffers, n of N sites, the swapped bits of a share of the bonds
 int64_t fslots_for(int64_t nbonds, int C) { return (nbonds + C - 1) / C + kMaxClasses; }
+// of a buffer: the largest class, and a place for each CTA without a bond (even:
+// n stays 16-byte aligned)
+int64_t entries_for(int64_t class_max, int C) { return C > 1 ? ((class_max + 1) & ~1LL) + C : 0; }
 size_t smem_for(int64_t N, int64_t class_max, int64_t nbonds, int C, bool f) {
-  return (C > 1 ? 2 * (size_t)((class_max + 1) & ~1LL) * 8 : 0) + (size_t)(N + 2) * 8 +
+  return 2 * (size_t)entries_for(class_max, C) * 8 + (size_t)(N + 2) * 8 +
          (f ? (size_t)fslots_for(nbonds, C) * 8 : 0);
 }
 
-constexpr size_t kGraphSmem = kSmemMax - 2048;  // beside the unit and the class tables
+constexpr size_t kGraphSmem = kSmemMax - 2560;  // beside the unit and the class tables
 
 }  // namespace
 
@@ -289,7 +302,7 @@ cudaError_t launch_graph(const Args& args, int64_t Nmax, int64_t bonds_max, int6
   Args a = args;
   a.fsmem = smem_for(Nmax, class_max, bonds_max, C, true) <= kGraphSmem;
   a.fslots = (int)fslots_for(bonds_max, C);
-  a.entries = C > 1 ? (int)((class_max + 1) & ~1LL) : 0;  // n stays 16-byte aligned
+  a.entries = (int)entries_for(class_max, C);
   const size_t smem = smem_for(Nmax, class_max, bonds_max, C, a.fsmem != 0);
   if (smem > kGraphSmem) return cudaErrorInvalidValue;
   const int threads = (int)std::max<int64_t>(64, ((class_max + C - 1) / C + 31) / 32 * 32);

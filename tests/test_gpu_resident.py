@@ -94,3 +94,26 @@ def test_last_sweep_number():
         st.t = (1 << 32) - 2
         O.sweeps(topo, 3, st, 3, 2)
         assert np.array_equal(sim.get_state()[0], O.pack_words(st.n))
+
+
+@pytest.mark.parametrize("N,z,R", [(16384, 4, 64), (16384, 4, 256), (8190, 4, 320), (1000, 5, 128)])
+def test_long_runs_equal_class_launches(N, z, R):
+    """Classes of fewer bonds than CTAs: no CTA may run ahead of one without a bond.
+
+    300 sweeps on chip, in a batch beside other jobs, against the same sweeps with a launch
+    per class (as profiling runs them)."""
+    kw = dict(topo=K.KA_RRG, N=N, z=z, m=2, replicas=R, graph_seed=7)
+    with K.Simulation(**kw) as sim:
+        sim.init(3, 0.7)
+        K.ka_profile_enable(sim.ctx, True)
+        sim.sweep(300)
+        n, _, p = sim.get_state()
+        K.ka_profile_enable(sim.ctx, False)
+    with K.Batch() as b:
+        ids = [b.add(300, 100, 3, 0.7, **kw) for _ in range(3)]
+        b.add(300, 100, 5, 0.7, topo=K.KA_CUBIC, d=3, L=32, m=3, replicas=256)
+        while b.step(25):
+            pass
+        for job in ids:
+            bn, _, bp = b.state(job, R // 64, N)
+            assert np.array_equal(bn, n) and np.array_equal(bp, p)
