@@ -73,14 +73,16 @@ struct ResidentClass {
   ka::resident::Unit* dev = nullptr;
 };
 
+// Graph jobs of one (V, m) and size (sites within a factor of two: sizes are
+// chains of launches side by side).
 struct GraphClass {
   int V = 0, m = 0, cmax = 0;
+  int64_t N = 0;  // of the first unit's job
   std::vector<ka::GraphUnit> units;
   std::vector<Job*> owner;
-  std::vector<int64_t> prefix, first, total;  // per class: [cmax][n+1], [cmax][n], [cmax]
+  std::vector<int64_t> block0;  // [cmax + 1]: the blocks of every class
   ka::GraphUnit* dev = nullptr;
-  int64_t* prefix_dev = nullptr;
-  int64_t* first_dev = nullptr;
+  ka::GraphBlock* blocks_dev = nullptr;
 };
 
 uint32_t cubic_tiles(int d, int L, int V, bool x) {
@@ -173,7 +175,7 @@ bool add_resident(ka_batch* b, Job* j, int64_t words) {
       if (x.L == c->L && x.d == c->d) rc = &x;
     } else if (x.L == 0 && (x.z <= 4) == (c->z <= 4) && 2 * x.N_max > c->N && x.N_max < 2 * c->N &&
                ka::resident::graph_cluster(std::max(x.N_max, c->N), std::max(x.bonds_max, c->nbonds),
-                                           std::max(x.class_max, c->class_max), 1, c->sms)) {
+                                           std::max(x.class_max, c->class_max))) {
       rc = &x;
     }
   }
@@ -259,12 +261,13 @@ cudaError_t rebuild(ka_batch* b) {
       } else {
         GraphClass* gc = nullptr;
         for (auto& x : b->graph)
-          if (x.V == V && x.m == c->m) gc = &x;
+          if (x.V == V && x.m == c->m && 2 * x.N > c->N && x.N < 2 * c->N) gc = &x;
         if (!gc) {
           b->graph.push_back(GraphClass{});
           gc = &b->graph.back();
           gc->V = V;
           gc->m = c->m;
+          gc->N = c->N;
         }
         ka::GraphUnit u{};
         u.n = n;
@@ -306,40 +309,32 @@ cudaError_t rebuild(ka_batch* b) {
     sc.dev = d;
   }
   for (auto& gc : b->graph) {
-    const int n = (int)gc.units.size();
-    gc.prefix.assign((size_t)gc.cmax * (n + 1), 0);
-    gc.first.assign((size_t)gc.cmax * n, 0);
-    gc.total.assign(gc.cmax, 0);
+    const int per = ka::kGraphBlock / gc.V;  // bonds per block
+    std::vector<ka::GraphBlock> blocks;
+    gc.block0.assign(1, 0);
     for (int c = 0; c < gc.cmax; ++c) {
-      int64_t acc = 0;
-      for (int u = 0; u < n; ++u) {
+      for (size_t u = 0; u < gc.units.size(); ++u) {
         const ka_ctx* x = gc.owner[u]->ctx;
-        int64_t cnt = 0, f = 0;
-        if (c < x->nclass) {
-          f = x->host.class_off[c];
-          cnt = x->host.class_off[c + 1] - f;
-        }
-        gc.prefix[(size_t)c * (n + 1) + u] = acc;
-        gc.first[(size_t)c * n + u] = f;
-        acc += cnt;
+        if (c >= x->nclass) continue;
+        const int64_t end = x->host.class_off[c + 1];
+        for (int64_t k = x->host.class_off[c]; k < end; k += per)
+          blocks.push_back({(int32_t)u, (int32_t)k, (int32_t)std::min<int64_t>(per, end - k)});
       }
-      gc.prefix[(size_t)c * (n + 1) + n] = acc;
-      gc.total[c] = acc;
+      gc.block0.push_back((int64_t)blocks.size());
     }
     if ((e = dev_alloc(b, &gc.dev, gc.units.size()))) return e;
-    if ((e = dev_alloc(b, &gc.prefix_dev, gc.prefix.size()))) return e;
-    if ((e = dev_alloc(b, &gc.first_dev, gc.first.size()))) return e;
-    e = cudaMemcpyAsync(gc.prefix_dev, gc.prefix.data(), gc.prefix.size() * sizeof(int64_t),
-                        cudaMemcpyHostToDevice, b->stream);
-    if (!e) e = cudaMemcpyAsync(gc.first_dev, gc.first.data(), gc.first.size() * sizeof(int64_t),
-                                cudaMemcpyHostToDevice, b->stream);
-    if (e) return e;
+    if ((e = dev_alloc(b, &gc.blocks_dev, blocks.size()))) return e;
+    if ((e = cudaMemcpyAsync(gc.blocks_dev, blocks.data(), blocks.size() * sizeof(ka::GraphBlock),
+                             cudaMemcpyHostToDevice, b->stream)))
+      return e;
+    // the host vector must outlive the copy
+    if ((e = cudaStreamSynchronize(b->stream))) return e;
   }
   for (auto& rc : b->resident) {
     const int64_t words = (int64_t)rc.units.size();
     const int sms = rc.owner[0]->ctx->sms;
     rc.C = rc.L ? ka::resident::cubic_cluster(rc.d, rc.L, words, sms)
-                : ka::resident::graph_cluster(rc.N_max, rc.bonds_max, rc.class_max, words, sms);
+                : ka::resident::graph_cluster(rc.N_max, rc.bonds_max, rc.class_max);
     if ((e = dev_alloc(b, &rc.dev, rc.units.size()))) return e;
   }
   b->dirty = false;
@@ -419,12 +414,11 @@ cudaError_t issue_round(ka_batch* b, int64_t k) {
   // the longest chains first: graphs have the most launches per sweep
   for (auto& gc : b->graph) {
     const cudaStream_t st = stream();
-    const int n = (int)gc.units.size();
     for (int64_t s = 0; s < k && !e; ++s)
       for (int c = 0; c < gc.cmax && !e; ++c)
-        e = ka::launch_graph_class_batch(gc.dev, gc.prefix_dev + (size_t)c * (n + 1),
-                                         gc.first_dev + (size_t)c * n, n, gc.total[c], gc.V, gc.m,
-                                         (uint32_t)c, (uint32_t)s, st);
+        e = ka::launch_graph_class_batch(gc.dev, gc.blocks_dev + gc.block0[c],
+                                         gc.block0[c + 1] - gc.block0[c], gc.V, gc.m, (uint32_t)c,
+                                         (uint32_t)s, st);
   }
   for (auto& rc : b->resident) {
     const cudaStream_t st = stream();

@@ -201,9 +201,10 @@ struct GraphDev {
   int z, m;
   int cubic_L;  // > 0: the bonds are those of a cubic lattice of this side (its gate stream)
 };
-// Class c (bonds [off, off + count) of the class-ordered bond arrays), all planes.
+// Class c (bonds [off, off + count) of the class-ordered bond arrays), planes q0 .. q0 + nq - 1.
 cudaError_t launch_graph_class(const Planes& pl, const GraphDev& g, int64_t off, int64_t count,
-                               uint32_t cls, uint32_t t, const RoundKeys& rk, cudaStream_t st);
+                               uint32_t cls, uint32_t t, const RoundKeys& rk, int q0, int nq,
+                               cudaStream_t st);
 
 // One graph work unit of a batched launch: one state plane of one job.
 struct GraphUnit {
@@ -218,11 +219,16 @@ struct GraphUnit {
   uint32_t t_base, t_end;
   RoundKeys rk;
 };
-// Class cls of sweep t_base + sweep_offset for every unit (all share V and m).
-cudaError_t launch_graph_class_batch(const GraphUnit* units_dev, const int64_t* prefix_dev,
-                                     const int64_t* first_dev, int nunits, int64_t total_edges,
-                                     int V, int m, uint32_t cls, uint32_t sweep_offset,
-                                     cudaStream_t s);
+// The bonds of one block of a batched launch: [first, first + count) of a
+// unit's class-ordered arrays, count <= kGraphBlock / V (a thread per word).
+constexpr int kGraphBlock = 128;
+struct GraphBlock {
+  int32_t unit, first, count;
+};
+// Class cls of sweep t_base + sweep_offset for the units' blocks (all share V and m).
+cudaError_t launch_graph_class_batch(const GraphUnit* units_dev, const GraphBlock* blocks_dev,
+                                     int64_t nblocks, int V, int m, uint32_t cls,
+                                     uint32_t sweep_offset, cudaStream_t s);
 
 // Scratch of the initial state: the lists of replicas' candidate sites (room
 // for those of one plane at least; ka_init.cu), their lengths, and the

@@ -23,7 +23,7 @@
 //
 // p is not read: the bits that swaps clear are collected in shared memory
 // (cubic: per site; graphs: per bond) and cleared in p by one atomic AND per
-// word at the end; where there is no room for that, at each swap.
+// word at the end; where a lattice leaves no room for that, at each swap.
 #pragma once
 
 #include "ka_internal.cuh"
@@ -56,8 +56,8 @@ struct Args {
   int words_per_plane;
   uint32_t from, most; // run at most `most` of a unit's sweeps, from this one on
   int L;               // cubic
-  int fsmem;           // the swapped bits are collected in shared memory
-  int fslots, entries; // graphs: their words; entries of a buffer
+  int fsmem;           // cubic: the swapped bits are collected in shared memory
+  int fslots, entries; // graphs: the words of the swapped bits; entries of a buffer
 };
 
 // threads of a CTA that has one C-th of a cubic lattice's pencils: a thread per
@@ -75,9 +75,9 @@ inline int cubic_threads(int64_t N, int L, int C) {
 int cubic_cluster(int d, int L, int64_t words, int sms);
 cudaError_t launch_cubic(const Args& a, int d, int L, int m, unsigned words, int C,
                          cudaStream_t st);
-// whether a graph of N sites runs here
+// whether a graph of N sites may run here, and its CTAs per word (0: it does not)
 bool graph_fits(int64_t N);
-int graph_cluster(int64_t N, int64_t nbonds, int64_t class_max, int64_t words, int sms);
+int graph_cluster(int64_t N, int64_t nbonds, int64_t class_max);
 // the packed record of every bond, from tables in storage positions
 int graph_record_bytes(int z);
 void graph_records(int64_t N, int z, const int32_t* nbr, const int32_t* bu, const int32_t* bv,

@@ -63,11 +63,10 @@ __global__ void __launch_bounds__(1024) k_resident_graph(const __grid_constant__
   uint32_t t = su.t_base + a.from, left_to_run = su.count > a.from ? min(su.count - a.from, a.most) : 0u;
   if (left_to_run == 0) return;  // the whole cluster: one unit
   const int N = su.N, nclass = su.nclass, tid = threadIdx.x;
-  // two entry buffers (C > 1), n, the swapped bits of this CTA's bonds (if fsmem)
+  // two entry buffers (C > 1), n, the swapped bits of this CTA's bonds
   uint64_t* buf = reinterpret_cast<uint64_t*>(dsm);
   uint64_t* n = buf + 2 * a.entries;
   uint64_t* f = n + N + 2;
-  const bool fsmem = a.fsmem != 0;
   const Peers<C> peers(smem_addr(dsm), rank);
   GroupEnd ge{smem_addr(bars), 0u, false};
   if (tid < 2) bar_init(ge.bars + 8 * tid, blockDim.x / 32);
@@ -90,8 +89,7 @@ __global__ void __launch_bounds__(1024) k_resident_graph(const __grid_constant__
       at += share[c];
     }
   }
-  if (fsmem)
-    for (int i = tid; i < a.fslots; i += blockDim.x) f[i] = 0;
+  for (int i = tid; i < a.fslots; i += blockDim.x) f[i] = 0;
   // how many bonds of class c CTA r has, and their first
   auto first = [&](int c, int r) { return coff[c] + r * share[c]; };
   auto mine = [&](int c, int r) {
@@ -164,14 +162,7 @@ __global__ void __launch_bounds__(1024) k_resident_graph(const __grid_constant__
         if (own == 0 && tid == 0) peers.st(smem_addr(in + a.entries - C + (int)rank), 0ull, ge.bar());
       }
       ge.arrive((uint32_t)(coff[c + 1] - coff[c] - own + idle[c] - (own == 0)) * 8u);
-      if (act) {
-        if (fsmem) {
-          f[slot[c] + tid] |= sw;
-        } else {
-          clear_bits(su.p + (size_t)u * su.stride, sw);
-          clear_bits(su.p + (size_t)v * su.stride, sw);
-        }
-      }
+      if (act) f[slot[c] + tid] |= sw;
       const int cn = c + 1 < nclass ? c + 1 : 0;
       turn(cn ? t : t + 1, cn);
       ge.wait(su.err);
@@ -191,15 +182,13 @@ __global__ void __launch_bounds__(1024) k_resident_graph(const __grid_constant__
     }
   }
   store_plane(su, n, N, rank, C);
-  if (fsmem) {
-    for (int c = 0; c < nclass; ++c) {
-      if (tid >= mine(c, (int)rank)) continue;
-      const uint32_t e =
-          *reinterpret_cast<const uint32_t*>(su.rec + (size_t)RW * (first(c, (int)rank) + tid));
-      const uint64_t sw = f[slot[c] + tid];
-      clear_bits(su.p + (size_t)(e & 0xFFFFu) * su.stride, sw);
-      clear_bits(su.p + (size_t)(e >> 16) * su.stride, sw);
-    }
+  for (int c = 0; c < nclass; ++c) {
+    if (tid >= mine(c, (int)rank)) continue;
+    const uint32_t e =
+        *reinterpret_cast<const uint32_t*>(su.rec + (size_t)RW * (first(c, (int)rank) + tid));
+    const uint64_t sw = f[slot[c] + tid];
+    clear_bits(su.p + (size_t)(e & 0xFFFFu) * su.stride, sw);
+    clear_bits(su.p + (size_t)(e >> 16) * su.stride, sw);
   }
   cluster_arrive();  // a CTA stays until the others have sent it all
   cluster_wait();
@@ -215,7 +204,6 @@ cudaError_t launch_m(const Args& a, unsigned words, int C, int threads, size_t s
              : launch_cluster(k_resident_graph<Z, M, CC, false>, a, words, CC, threads, smem, st);
     KA_C(1)
     KA_C(4)
-    KA_C(8)
 #undef KA_C
     default:
       return cudaErrorInvalidValue;
@@ -248,16 +236,17 @@ int64_t fslots_for(int64_t nbonds, int C) { return (nbonds + C - 1) / C + kMaxCl
 // of a buffer: the largest class, and a place for each CTA without a bond (even:
 // n stays 16-byte aligned)
 int64_t entries_for(int64_t class_max, int C) { return C > 1 ? ((class_max + 1) & ~1LL) + C : 0; }
-size_t smem_for(int64_t N, int64_t class_max, int64_t nbonds, int C, bool f) {
+size_t smem_for(int64_t N, int64_t class_max, int64_t nbonds, int C) {
   return 2 * (size_t)entries_for(class_max, C) * 8 + (size_t)(N + 2) * 8 +
-         (f ? (size_t)fslots_for(nbonds, C) * 8 : 0);
+         (size_t)fslots_for(nbonds, C) * 8;
 }
 
 constexpr size_t kGraphSmem = kSmemMax - 2560;  // beside the unit and the class tables
 
 }  // namespace
 
-bool graph_fits(int64_t N) { return N >= 2 && N < 65535 && (size_t)(N + 2) * 8 <= kGraphSmem; }
+// 16-bit positions, and the measured limit (graph_cluster)
+bool graph_fits(int64_t N) { return N >= 2 && N <= 11000; }
 
 int graph_record_bytes(int z) { return z <= 4 ? 16 : 32; }
 
@@ -281,17 +270,15 @@ void graph_records(int64_t N, int z, const int32_t* nbr, const int32_t* bu, cons
   }
 }
 
-int graph_cluster(int64_t N, int64_t nbonds, int64_t class_max, int64_t words, int sms) {
-  // a thread per bond of a class and all tables in shared memory; the fewest
-  // CTAs that do.  us a sweep (z = 4, one word) with 1, 4, 8 CTAs, and with one
-  // launch per class: N = 2^12 15.5, 17.4, 20.5; 37.  2^13: -, 21.7, 22.2; 40.
-  // 2^14: -, 45 (no room for the swapped bits), 31.5; 44.  With 32 words 2^14
-  // takes 48 with four CTAs and 94 with eight (they no longer run at once); 113.
-  auto fits = [&](int C, bool f) {
-    return class_max <= 1024 * C && smem_for(N, class_max, nbonds, C, f) <= kGraphSmem;
-  };
-  for (int C : {1, 4, 8})
-    if (fits(C, true)) return C == 8 && words * 8 > sms && fits(4, false) ? 4 : C;
+int graph_cluster(int64_t N, int64_t nbonds, int64_t class_max) {
+  // A thread per bond of a class and all tables in shared memory, on the fewest
+  // CTAs that do.  us a sweep (z = 4, 1 to 8 words) with one CTA, with four, and
+  // with one launch per class: N = 2^12 17, -, 26-28; 6000 -, 19, 28-31; 2^13
+  // -, 21, 27-30; 10^4 -, 24, 27-30; 12 000 -, 28, 27-31; 2^14 -, 45 (no room for
+  // the swapped bits; with eight CTAs 33), 27-33.
+  if (!graph_fits(N)) return 0;
+  for (int C : {1, 4})
+    if (class_max <= 1024 * C && smem_for(N, class_max, nbonds, C) <= kGraphSmem) return C;
   return 0;
 }
 
@@ -300,10 +287,9 @@ cudaError_t launch_graph(const Args& args, int64_t Nmax, int64_t bonds_max, int6
   if (m < 0 || z < 1 || z > 8 || !graph_fits(Nmax) || class_max > 1024 * C)
     return cudaErrorInvalidValue;
   Args a = args;
-  a.fsmem = smem_for(Nmax, class_max, bonds_max, C, true) <= kGraphSmem;
   a.fslots = (int)fslots_for(bonds_max, C);
   a.entries = (int)entries_for(class_max, C);
-  const size_t smem = smem_for(Nmax, class_max, bonds_max, C, a.fsmem != 0);
+  const size_t smem = smem_for(Nmax, class_max, bonds_max, C);
   if (smem > kGraphSmem) return cudaErrorInvalidValue;
   const int threads = (int)std::max<int64_t>(64, ((class_max + C - 1) / C + 31) / 32 * 32);
   return z <= 4 ? launch_z<4>(a, m, words, C, threads, smem, st)

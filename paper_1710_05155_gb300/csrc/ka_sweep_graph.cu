@@ -1,20 +1,28 @@
 // ka_sweep_graph.cu -- edge-gather sweep kernel for one bond class.
 //
-// One thread per (bond of the class, plane).  The bond (u, v) gathers the
-// words of u, v and of their other neighbours from the int32 neighbour
-// list, counts the occupied neighbours of u other than v and of v other
-// than u with bit-sliced adders (64 replicas per word), and applies the
-// exchange rule of section 2.1 (rules (a)-(c)) under the replica's Philox
-// gate bit.  Bonds of a class form a strong matching, so threads never
-// touch each other's sites.
+// One thread per (bond of the class, word): the bond (u, v) gathers its word
+// of u, v and of their other neighbours from the int32 neighbour list, counts
+// the occupied neighbours of u other than v and of v other than u with
+// bit-sliced adders (64 replicas per word), and applies the exchange rule of
+// section 2.1 (rules (a)-(c)) under the replica's Philox gate bit.  Bonds of a
+// class form a strong matching, so bonds never touch each other's sites.
 //
 // A plane holds V = 1, 2 or 4 words per site, so a site's words share one
 // 32-byte sector: every gather is a random access, and the sector is the
-// unit the memory system moves.  The partner's word is not gathered twice,
-// and p is never read: the bits of p that a swap clears are cleared by an
-// atomic AND in the L2.
+// unit the memory system moves.  The V words of a bond are V neighbouring
+// lanes, whose accesses to a site fall into its sector together; one thread
+// with all V words needed 110 registers (22 % of the warps) and V separate
+// atomics per site.  Blocks are small: what bounds the gathers is sectors in
+// flight and their reuse in the L1, and fewer, larger blocks (or more warps by
+// fewer registers) lose the reuse: 2^20 sites, 512 replicas 320 us a sweep with
+// 128 threads, 341 with 256, 395 with 1024, 376 with 5 instead of 4 blocks of
+// 256.  us a sweep, z = 4, m = 2, before and after: 2^20 sites 512 replicas 623,
+// 320; 256 replicas 301, 165; 2^17 256 replicas 117, 41; one word 2^15 47, 32;
+// 2^17 60, 45; 2^20 160, 135.
+// The partner's word is not gathered twice, and p is never read: the bits of
+// p that a swap clears are cleared by an atomic AND in the L2.
 // A thread first loads what depends only on static tables (its bond, the
-// two neighbour rows) and computes the gate words, then gathers the state.
+// two neighbour rows) and computes the gate word, then gathers the state.
 // Single-instance class launches are chained with programmatic dependent
 // launch, so that this prologue overlaps the previous class's tail (small
 // graphs are bound by launch latency); batched launches are not, since a
@@ -34,6 +42,7 @@ struct ClassArgs {
   size_t plane_elems;
   int64_t count;
   int z;
+  int q0;  // first plane of the launch
   uint32_t t, cls;
   uint32_t pair_stride;  // cubic lattices: stride of the bond direction, 0 on graphs
   RoundKeys rk;
@@ -62,34 +71,8 @@ __device__ __forceinline__ uint64_t le3(uint64_t b2, uint64_t b1, uint64_t b0) {
   }
 }
 
-// the V words of site i (16-byte vectors for V >= 2; a site's words are
-// 8 V-byte aligned)
-template <int V>
-__device__ __forceinline__ void ld(const uint64_t* base, int64_t i, uint64_t (&o)[V]) {
-  if constexpr (V == 1) {
-    o[0] = base[i];
-  } else {
-#pragma unroll
-    for (int h = 0; h < V; h += 2) {
-      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(base + V * i + h);
-      o[h] = v.x;
-      o[h + 1] = v.y;
-    }
-  }
-}
-
-template <int V>
-__device__ __forceinline__ void st(uint64_t* base, int64_t i, const uint64_t (&o)[V]) {
-  if constexpr (V == 1) {
-    base[i] = o[0];
-  } else {
-#pragma unroll
-    for (int h = 0; h < V; h += 2)
-      *reinterpret_cast<ulonglong2*>(base + V * i + h) = make_ulonglong2(o[h], o[h + 1]);
-  }
-}
-
 constexpr int kMaxZ = 8;
+constexpr int kThreads = 128;
 
 // neighbour row of x (z <= 8); z = 4 rows are one 16-byte load
 __device__ __forceinline__ void load_row(const int32_t* nbr, int z, int32_t x,
@@ -108,143 +91,104 @@ __device__ __forceinline__ void load_row(const int32_t* nbr, int z, int32_t x,
 }
 
 // Graph gate stream: word w of bond id takes half w mod 2 of the block
-// (t, class, id, w / 2).  Planes start at an even word when V >= 2.
-template <int V>
-__device__ __forceinline__ void graph_gates(uint32_t t, uint32_t cls, uint32_t id, uint32_t w0,
-                                            const RoundKeys& rk, uint64_t (&g)[V]) {
-  if constexpr (V == 1) {
-    const uint4 b = philox(make_uint4(t, cls, id, w0 >> 1), rk);
-    g[0] = (w0 & 1u) ? hi64(b) : lo64(b);
-  } else {
-#pragma unroll
-    for (int h = 0; h < V; h += 2) {
-      const uint4 b = philox(make_uint4(t, cls, id, (w0 + h) >> 1), rk);
-      g[h] = lo64(b);
-      g[h + 1] = hi64(b);
-    }
-  }
+// (t, class, id, w / 2).
+__device__ __forceinline__ uint64_t graph_gate(uint32_t t, uint32_t cls, uint32_t id, uint32_t w,
+                                               const RoundKeys& rk) {
+  const uint4 b = philox(make_uint4(t, cls, id, w >> 1), rk);
+  return (w & 1u) ? hi64(b) : lo64(b);
 }
 
-// The exchange on bond (u, v), V words: counts of the other neighbours of
-// u and of v, the rule, the gated swap, and the persistence update.
+// The exchange on bond (u, v) for one word of a plane (np and pp at that
+// word): counts of the other neighbours of u and of v, the rule, the gated
+// swap, and the persistence update.
 template <int V, int M>
 __device__ __forceinline__ void exchange(uint64_t* np, uint64_t* pp, int z, int32_t u, int32_t v,
                                          const int32_t (&ru)[kMaxZ], const int32_t (&rv)[kMaxZ],
-                                         const uint64_t (&g)[V]) {
-  uint64_t nu[V], nv[V];
-  ld<V>(np, u, nu);
-  ld<V>(np, v, nv);
-  uint64_t cu2[V], cu1[V], cu0[V], cv2[V], cv1[V], cv0[V];
+                                         uint64_t g) {
+  const uint64_t nu = np[(int64_t)u * V], nv = np[(int64_t)v * V];
+  uint64_t xu[kMaxZ], xv[kMaxZ];
 #pragma unroll
-  for (int h = 0; h < V; ++h) cu2[h] = cu1[h] = cu0[h] = cv2[h] = cv1[h] = cv0[h] = 0;
+  for (int k = 0; k < kMaxZ; ++k) {
+    if (k < z) {  // the partner is not one of the "other" neighbours
+      xu[k] = ru[k] != v ? np[(int64_t)ru[k] * V] : 0ull;
+      xv[k] = rv[k] != u ? np[(int64_t)rv[k] * V] : 0ull;
+    }
+  }
+  uint64_t cu2 = 0, cu1 = 0, cu0 = 0, cv2 = 0, cv1 = 0, cv0 = 0;
 #pragma unroll
   for (int k = 0; k < kMaxZ; ++k) {
     if (k < z) {
-      if (ru[k] != v) {  // the partner is not one of the "other" neighbours
-        uint64_t x[V];
-        ld<V>(np, ru[k], x);
-#pragma unroll
-        for (int h = 0; h < V; ++h) add3(cu2[h], cu1[h], cu0[h], x[h]);
-      }
-      if (rv[k] != u) {
-        uint64_t x[V];
-        ld<V>(np, rv[k], x);
-#pragma unroll
-        for (int h = 0; h < V; ++h) add3(cv2[h], cv1[h], cv0[h], x[h]);
-      }
+      add3(cu2, cu1, cu0, xu[k]);
+      add3(cv2, cv1, cv0, xv[k]);
     }
   }
-  uint64_t sw[V];
-  bool any = false;
-#pragma unroll
-  for (int h = 0; h < V; ++h) {
-    const uint64_t ok = le3<M>(cu2[h], cu1[h], cu0[h]) & le3<M>(cv2[h], cv1[h], cv0[h]);
-    sw[h] = (nu[h] ^ nv[h]) & g[h] & ok;
-    nu[h] ^= sw[h];
-    nv[h] ^= sw[h];
-    any |= (sw[h] != 0);
-  }
-  if (any) {
-    st<V>(np, u, nu);
-    st<V>(np, v, nv);
+  const uint64_t sw = (nu ^ nv) & g & le3<M>(cu2, cu1, cu0) & le3<M>(cv2, cv1, cv0);
+  if (sw) {
+    np[(int64_t)u * V] = nu ^ sw;
+    np[(int64_t)v * V] = nv ^ sw;
     // Persistence: an atomic AND performed in the L2 (no reply), not a load
     // of p after the swap is known and a store: random gathers are bound by
     // the misses an SM keeps in flight, and this removes two of them per bond
     // and a dependent round trip.
-    unsigned long long* pw = reinterpret_cast<unsigned long long*>(pp);
-#pragma unroll
-    for (int h = 0; h < V; ++h) {
-      if (sw[h]) {
-        atomicAnd(pw + (size_t)V * u + h, (unsigned long long)~sw[h]);
-        atomicAnd(pw + (size_t)V * v + h, (unsigned long long)~sw[h]);
-      }
-    }
+    atomicAnd(reinterpret_cast<unsigned long long*>(pp + (int64_t)u * V), (unsigned long long)~sw);
+    atomicAnd(reinterpret_cast<unsigned long long*>(pp + (int64_t)v * V), (unsigned long long)~sw);
   }
 }
 
-template <int V, int M>
-__global__ void __launch_bounds__(256) k_graph_class(const __grid_constant__ ClassArgs a) {
+template <int V, int M, int MINB>
+__global__ void __launch_bounds__(kThreads, MINB) k_graph_class(const __grid_constant__ ClassArgs a) {
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t e = i / V;
+  const int h = (int)(i % V);
   if (e >= a.count) return;
-  const int q = blockIdx.y;
-  uint64_t* np = a.n + (size_t)q * a.plane_elems;
-  uint64_t* pp = a.p + (size_t)q * a.plane_elems;
+  const int q = a.q0 + (int)blockIdx.y;
   const int32_t u = a.bu[e], v = a.bv[e];
   const uint32_t id = a.bid[e];
   int32_t ru[kMaxZ], rv[kMaxZ];
   load_row(a.nbr, a.z, u, ru);
   load_row(a.nbr, a.z, v, rv);
-  // gate words.  Graphs: the graph stream.  Cubic lattices on this path:
+  // gate word.  Graphs: the graph stream.  Cubic lattices on this path:
   // bonds of classes 4g+2b and 4g+2b+1 that start at neighbouring pencil
   // positions share the block (t, 4g+2b, base site of the first, word),
   // half = class parity.
-  uint64_t g[V];
-  const uint32_t w0 = (uint32_t)(q * V);
+  const uint32_t w = (uint32_t)(q * V + h);
+  uint64_t g;
   if (a.pair_stride != 0) {
     const uint32_t odd = a.cls & 1u;
-#pragma unroll
-    for (int h = 0; h < V; ++h) {
-      const uint4 b = philox(make_uint4(a.t, a.cls - odd, id - odd * a.pair_stride, w0 + h), a.rk);
-      g[h] = odd ? hi64(b) : lo64(b);
-    }
+    const uint4 b = philox(make_uint4(a.t, a.cls - odd, id - odd * a.pair_stride, w), a.rk);
+    g = odd ? hi64(b) : lo64(b);
   } else {
-    graph_gates<V>(a.t, a.cls, id, w0, a.rk, g);
+    g = graph_gate(a.t, a.cls, id, w, a.rk);
   }
   asm volatile("griddepcontrol.wait;\n" ::: "memory");  // the previous class is complete
-  exchange<V, M>(np, pp, a.z, u, v, ru, rv, g);
+  exchange<V, M>(a.n + (size_t)q * a.plane_elems + h, a.p + (size_t)q * a.plane_elems + h, a.z, u, v,
+                 ru, rv, g);
 }
 
-// Batched form: one launch runs class c of every graph unit (one state plane
-// of one job); edges of all units are numbered consecutively, unit u owning
-// [prefix[u], prefix[u+1]) of them, which start at edge first[u] of its
-// class-ordered edge arrays.  Units whose sweep counter reached t_end skip.
+// Batched form: one launch runs class cls of every graph unit (one state plane
+// of one job); block b takes the bonds that blocks[b] says, up to
+// kGraphBlock / V of one unit.  Units whose sweep counter reached t_end skip.
 template <int V, int M>
-__global__ void __launch_bounds__(256) k_graph_class_batch(const GraphUnit* __restrict__ units,
-                                                           const int64_t* __restrict__ prefix,
-                                                           const int64_t* __restrict__ first,
-                                                           int nunits, uint32_t cls,
-                                                           uint32_t sweep_offset) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= prefix[nunits]) return;
-  int lo = 0, hi = nunits - 1;  // last unit with prefix <= e
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (prefix[mid] <= e) lo = mid; else hi = mid - 1;
-  }
-  const GraphUnit& gu = units[lo];
+__global__ void __launch_bounds__(kGraphBlock) k_graph_class_batch(const GraphUnit* __restrict__ units,
+                                                           const GraphBlock* __restrict__ blocks,
+                                                           uint32_t cls, uint32_t sweep_offset) {
+  __shared__ GraphUnit gu;
+  const GraphBlock b = blocks[blockIdx.x];
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(units + b.unit);
+  if (threadIdx.x < sizeof(GraphUnit) / 4) reinterpret_cast<uint32_t*>(&gu)[threadIdx.x] = src[threadIdx.x];
+  const int e = (int)threadIdx.x / V, h = (int)threadIdx.x % V;
+  __syncthreads();
   const uint32_t t = gu.t_base + sweep_offset;
-  if (t >= gu.t_end) return;
-  const int64_t k = first[lo] + (e - prefix[lo]);
+  if (t >= gu.t_end || e >= b.count) return;
+  const int64_t k = (int64_t)b.first + e;
   const int32_t u = gu.bu[k], v = gu.bv[k];
   const uint32_t id = gu.bid[k];
-  const int z = gu.z;
   int32_t ru[kMaxZ], rv[kMaxZ];
-  load_row(gu.nbr, z, u, ru);
-  load_row(gu.nbr, z, v, rv);
-  uint64_t g[V];
-  graph_gates<V>(t, cls, id, gu.word0, gu.rk, g);
-  exchange<V, M>(gu.n, gu.p, z, u, v, ru, rv, g);
+  load_row(gu.nbr, gu.z, u, ru);
+  load_row(gu.nbr, gu.z, v, rv);
+  const uint64_t g = graph_gate(t, cls, id, gu.word0 + (uint32_t)h, gu.rk);
+  exchange<V, M>(gu.n + h, gu.p + h, gu.z, u, v, ru, rv, g);
 }
 
 // single-instance launch with programmatic stream serialisation
@@ -252,7 +196,7 @@ template <typename Kern>
 cudaError_t launch_pdl(Kern kern, dim3 grid, cudaStream_t s, const ClassArgs& a) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -263,12 +207,12 @@ cudaError_t launch_pdl(Kern kern, dim3 grid, cudaStream_t s, const ClassArgs& a)
   return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
-template <int V>
+template <int V, int MINB>
 cudaError_t launch_v(const ClassArgs& a, int m, dim3 grid, cudaStream_t s) {
   switch (m < 7 ? m : 7) {
 #define KA_CASE(MM) \
   case MM:          \
-    return launch_pdl(k_graph_class<V, MM>, grid, s, a);
+    return launch_pdl(k_graph_class<V, MM, MINB>, grid, s, a);
     KA_CASE(0)
     KA_CASE(1)
     KA_CASE(2)
@@ -284,13 +228,12 @@ cudaError_t launch_v(const ClassArgs& a, int m, dim3 grid, cudaStream_t s) {
 }
 
 template <int V>
-cudaError_t launch_batch_v(const GraphUnit* units, const int64_t* prefix, const int64_t* first,
-                           int nunits, int m, uint32_t cls, uint32_t off, dim3 grid,
-                           cudaStream_t s) {
+cudaError_t launch_batch_v(const GraphUnit* units, const GraphBlock* blocks, unsigned nblocks, int m,
+                           uint32_t cls, uint32_t off, cudaStream_t s) {
   switch (m < 7 ? m : 7) {
-#define KA_CASE(MM)                                                                     \
-  case MM:                                                                              \
-    k_graph_class_batch<V, MM><<<grid, 256, 0, s>>>(units, prefix, first, nunits, cls, off); \
+#define KA_CASE(MM)                                                               \
+  case MM:                                                                        \
+    k_graph_class_batch<V, MM><<<nblocks, kGraphBlock, 0, s>>>(units, blocks, cls, off); \
     return cudaGetLastError();
     KA_CASE(0)
     KA_CASE(1)
@@ -308,23 +251,19 @@ cudaError_t launch_batch_v(const GraphUnit* units, const int64_t* prefix, const 
 
 }  // namespace
 
-cudaError_t launch_graph_class_batch(const GraphUnit* units_dev, const int64_t* prefix_dev,
-                                     const int64_t* first_dev, int nunits, int64_t total_edges,
-                                     int V, int m, uint32_t cls, uint32_t sweep_offset,
-                                     cudaStream_t s) {
-  if (nunits <= 0 || total_edges <= 0) return cudaSuccess;
-  const dim3 grid((unsigned)((total_edges + 255) / 256));
-  if (V == 4)
-    return launch_batch_v<4>(units_dev, prefix_dev, first_dev, nunits, m, cls, sweep_offset, grid, s);
-  if (V == 2)
-    return launch_batch_v<2>(units_dev, prefix_dev, first_dev, nunits, m, cls, sweep_offset, grid, s);
-  if (V == 1)
-    return launch_batch_v<1>(units_dev, prefix_dev, first_dev, nunits, m, cls, sweep_offset, grid, s);
+cudaError_t launch_graph_class_batch(const GraphUnit* units_dev, const GraphBlock* blocks_dev,
+                                     int64_t nblocks, int V, int m, uint32_t cls,
+                                     uint32_t sweep_offset, cudaStream_t s) {
+  if (nblocks <= 0) return cudaSuccess;
+  if (V == 4) return launch_batch_v<4>(units_dev, blocks_dev, (unsigned)nblocks, m, cls, sweep_offset, s);
+  if (V == 2) return launch_batch_v<2>(units_dev, blocks_dev, (unsigned)nblocks, m, cls, sweep_offset, s);
+  if (V == 1) return launch_batch_v<1>(units_dev, blocks_dev, (unsigned)nblocks, m, cls, sweep_offset, s);
   return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_graph_class(const Planes& pl, const GraphDev& g, int64_t off, int64_t count,
-                               uint32_t cls, uint32_t t, const RoundKeys& rk, cudaStream_t s) {
+                               uint32_t cls, uint32_t t, const RoundKeys& rk, int q0, int nq,
+                               cudaStream_t s) {
   if (count <= 0) return cudaSuccess;
   ClassArgs a;
   a.n = pl.n;
@@ -345,10 +284,15 @@ cudaError_t launch_graph_class(const Planes& pl, const GraphDev& g, int64_t off,
     a.pair_stride = s;
   }
   a.rk = rk;
-  const dim3 grid((unsigned)((count + 255) / 256), (unsigned)pl.P);
-  if (pl.V == 4) return launch_v<4>(a, g.m, grid, s);
-  if (pl.V == 2) return launch_v<2>(a, g.m, grid, s);
-  return launch_v<1>(a, g.m, grid, s);
+  a.q0 = q0;
+  const dim3 grid((unsigned)((count * pl.V + kThreads - 1) / kThreads), (unsigned)nq);
+  if (pl.V == 4) return launch_v<4, 1>(a, g.m, grid, s);
+  if (pl.V == 2) return launch_v<2, 1>(a, g.m, grid, s);
+  // one word: a full device wants more warps (48 registers) once the gathers
+  // miss the L1 anyway.  us a sweep with 8 and 10 blocks per SM: 2^17 sites 45,
+  // 47; 2^19 109, 113; 2^20 155, 135; 3 planes of 2^18 121, 125, of 2^19 203, 175.
+  return (int64_t)pl.N * nq >= (1 << 20) ? launch_v<1, 10>(a, g.m, grid, s)
+                                         : launch_v<1, 1>(a, g.m, grid, s);
 }
 
 }  // namespace ka

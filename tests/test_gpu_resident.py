@@ -41,8 +41,8 @@ def test_lattices(d, L, R, m):
 
 @pytest.mark.parametrize("N,z,R,m", [
     (6, 3, 64, 1), (32, 1, 64, 0), (50, 5, 128, 3), (1001, 4, 192, 3), (1000, 2, 64, 0),
-    (4096, 4, 64, 2), (8190, 4, 320, 2), (12000, 3, 64, 1), (16384, 4, 64, 2), (16384, 4, 64 * 20, 2),
-    (28000, 4, 64, 2),
+    (4096, 4, 64, 2), (8190, 4, 320, 2), (10998, 3, 64, 1), (11000, 4, 64 * 20, 2), (11001, 4, 64, 2),
+    (16384, 4, 64, 2),
 ])
 def test_random_regular_graphs(N, z, R, m):
     _same(dict(topo=K.KA_RRG, N=N, z=z, m=m, replicas=R, graph_seed=3), O.rrg(N, z, 3), 5, 0.6,
@@ -96,7 +96,7 @@ def test_last_sweep_number():
         assert np.array_equal(sim.get_state()[0], O.pack_words(st.n))
 
 
-@pytest.mark.parametrize("N,z,R", [(16384, 4, 64), (16384, 4, 256), (8190, 4, 320), (1000, 5, 128)])
+@pytest.mark.parametrize("N,z,R", [(10999, 4, 64), (10999, 4, 256), (8190, 4, 320), (1000, 5, 128)])
 def test_long_runs_equal_class_launches(N, z, R):
     """Classes of fewer bonds than CTAs: no CTA may run ahead of one without a bond.
 
