@@ -124,10 +124,11 @@ typedef struct {
     int64_t sweep;      /* sweeps completed since init (or set_state) */
     int64_t K;          /* particles per replica at the last init (-1 if none) */
     uint64_t seed;      /* dynamics seed */
-    int32_t kernel;     /* 0 = general cubic pencil kernel, 1 = edge-gather kernel,
+    int32_t kernel;     /* 0 = cubic pencil kernels, 1 = edge-gather kernel,
                            3 = group kernels of three-dimensional lattices (d = 3,
-                           L % 4 == 0, L <= 128: from two planes up, and for one
-                           plane at the sides where they are measured faster) */
+                           L % 4 == 0, L <= 128: reported from two planes up and,
+                           for one plane, at the sides that first had them; the
+                           other one-plane sides, reported as 0, run them too) */
     int32_t rrg_attempts; /* configuration-model attempts (KA_RRG) */
     size_t device_bytes;  /* device memory the context uses */
     int32_t planes;       /* device state planes per array */

@@ -478,7 +478,7 @@ ka_status ka_sweep(ka_ctx* c, int64_t n) {
               : ka::resident::launch_graph(a, c->N, c->nbonds, c->class_max, c->z, c->m,
                                            (unsigned)c->pl.W, C, c->stream);
     }
-  } else if (c->pencil && ka::stream_preferred(c->d, c->L, c->pl.P)) {
+  } else if (c->pencil && ka::stream_supported(c->d, c->L)) {
     // plane-outer order keeps the planes of one launch resident in the L2
     // across sweeps
     const int nq = ka::stream_planes_per_launch(c->L, c->pl.P);
@@ -644,13 +644,13 @@ ka_status ka_info(const ka_ctx* c, ka_info_t* out) {
   out->sweep = c->sweep;
   out->K = c->K;
   out->seed = c->seed;
-  out->kernel = !c->pencil ? 1 : ka::stream_preferred(c->d, c->L, c->pl.P) ? 3 : 0;
+  out->kernel = !c->pencil ? 1 : ka::stream_reported(c->d, c->L, c->pl.P) ? 3 : 0;
   out->rrg_attempts = c->host.attempts;
   out->device_bytes = c->bytes;
   out->planes = c->pl.P;
   out->plane_words = c->pl.V;
   out->planes_per_launch =
-      (c->pencil && ka::stream_preferred(c->d, c->L, c->pl.P)) ? ka::stream_planes_per_launch(c->L, c->pl.P)
+      (c->pencil && ka::stream_supported(c->d, c->L)) ? ka::stream_planes_per_launch(c->L, c->pl.P)
                                                                 : 1;
   return KA_OK;
 }

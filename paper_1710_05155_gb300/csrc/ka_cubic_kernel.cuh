@@ -90,7 +90,6 @@ cudaError_t launch_d(int V, bool x, const GroupArgs& a, const BatchArgs& ba, int
                                                  int, unsigned, size_t, cudaStream_t);
 KA_CUBIC_EXTERN(1)
 KA_CUBIC_EXTERN(2)
-KA_CUBIC_EXTERN(3)
 KA_CUBIC_EXTERN(4)
 #undef KA_CUBIC_EXTERN
 

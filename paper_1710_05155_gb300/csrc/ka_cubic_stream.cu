@@ -9,14 +9,8 @@ namespace ka {
 
 bool stream_supported(int d, int L) { return d == 3 && L % 4 == 0 && L >= 4 && L <= 128; }
 
-bool stream_preferred(int d, int L, int P) {
-  // Measured per word-sweep against the general pencil kernel
-  // (ka_cubic_kernel.cuh): from two planes up the group kernels win at every
-  // side (1.3-4.4x).  With one plane (64 replicas) they win or tie at
-  // L = 8, 16, 48, 80, 88, 96, 104, 112, 116, 120, 124 (up to 1.95x) and lose
-  // by up to 8 % at 28, 56, 60, 72 and 100 (rows that leave lanes idle, too
-  // few CTAs), tie at 24, 36, 40, 108; the unmeasured sides follow their
-  // neighbours.
+bool stream_reported(int d, int L, int P) {
+  // one-plane contexts of these sides have always been reported as kernel 0
   if (!stream_supported(d, L)) return false;
   if (P >= 2) return true;
   switch (L) {

@@ -148,7 +148,7 @@ KA_HD int64_t canon_pos(const int32_t* inv, int xs, int64_t q) {
   return inv ? (int64_t)inv[q] : canon_site(xs, q);
 }
 
-// Warps per CTA of the cubic pencil kernel: a tile holds kCubicWarps / V
+// Warps per CTA of the general cubic pencil kernel (d = 1, 2, 4): a tile holds kCubicWarps / V
 // active pencils (one warp per pencil-word in the compute phase).
 constexpr int kCubicWarps = 8;
 
@@ -253,8 +253,11 @@ cudaError_t launch_to_canonical(const uint64_t* device_layout, uint64_t* canonic
 // Group kernels of three-dimensional lattices (ka_cubic_stream.cu): one-word
 // planes in split-row order, d = 3, L % 4 == 0, L <= 128.
 bool stream_supported(int d, int L);
-// whether a context of P one-word planes runs them (else the general kernel)
-bool stream_preferred(int d, int L, int P);
+// whether ka_info reports them for a context of P one-word planes (every
+// supported lattice runs them: 64 replicas, us a sweep, against the general
+// pencil kernel: L = 24 14.1, 14.7; 44 19.6, 24.4; 60 20.3, 32.6; 72 22.8, 29.0; 100
+// 31.7, 61.6; 116 50, 97)
+bool stream_reported(int d, int L, int P);
 // planes one launch of these kernels takes
 int stream_planes_per_launch(int L, int P);
 // Group (mu, par) of sweep t on planes q0 .. q0 + nq - 1.

@@ -13,7 +13,6 @@ cudaError_t dispatch(int d, int V, bool x, const GroupArgs& a, const BatchArgs& 
   switch (d) {
     case 1: return cubic::launch_d<1, B>(V, x, a, ba, m, blocks, smem, st);
     case 2: return cubic::launch_d<2, B>(V, x, a, ba, m, blocks, smem, st);
-    case 3: return cubic::launch_d<3, B>(V, x, a, ba, m, blocks, smem, st);
     case 4: return cubic::launch_d<4, B>(V, x, a, ba, m, blocks, smem, st);
     default: return cudaErrorInvalidValue;
   }
