@@ -150,6 +150,12 @@ struct DeviceGuard {
   }
 };
 
+void free_side(ka_ctx* c) {
+  if (c->side) cudaStreamDestroy(c->side);
+  if (c->fork) cudaEventDestroy(c->fork);
+  if (c->join) cudaEventDestroy(c->join);
+}
+
 ka_status create_common(const ka_params* params, void* buf, size_t bytes, bool owns, ka_ctx** out) {
   Shape s{};
   if (const char* e = check_params(params, s)) return KA_EINVAL;
@@ -272,6 +278,18 @@ ka_status create_common(const ka_params* params, void* buf, size_t bytes, bool o
                           cudaMemcpyHostToDevice, c->stream);
     if (!e) e = cudaStreamSynchronize(c->stream);
     if (e) {
+      if (owns) cudaFree(buf);
+      delete c;
+      return KA_ECUDA;
+    }
+  }
+  int per = 0;
+  if (c->pencil && ka::stream_supported(c->d, c->L) && ka::stream_chains(c->L, c->pl.P, &per) > 1) {
+    cudaError_t e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
+    if (!e) e = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming);
+    if (!e) e = cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming);
+    if (e) {
+      free_side(c);
       if (owns) cudaFree(buf);
       delete c;
       return KA_ECUDA;
@@ -479,19 +497,34 @@ ka_status ka_sweep(ka_ctx* c, int64_t n) {
                                            (unsigned)c->pl.W, C, c->stream);
     }
   } else if (c->pencil && ka::stream_supported(c->d, c->L)) {
-    // plane-outer order keeps the planes of one launch resident in the L2
-    // across sweeps
-    const int nq = ka::stream_planes_per_launch(c->L, c->pl.P);
-    for (int q0 = 0; q0 < c->pl.P && !e; q0 += nq) {
-      const int cnt = std::min(nq, c->pl.P - q0);
+    // Plane groups run chain by chain, all sweeps of a group before the
+    // chain's next: the planes in flight stay resident in the L2.
+    int per = ka::stream_planes_per_launch(c->L, c->pl.P);
+    const int chains = c->side && !c->prof ? ka::stream_chains(c->L, c->pl.P, &per) : 1;
+    if (chains > 1) {
+      e = cudaEventRecord(c->fork, c->stream);
+      if (!e) e = cudaStreamWaitEvent(c->side, c->fork, 0);
+    }
+    // a sweep of one chain, then of the other, so that both have work queued
+    for (int q0 = 0; q0 < c->pl.P && !e; q0 += chains * per)
       for (int64_t s = 0; s < n && !e; ++s)
-        for (int mu = 0; mu < 3 && !e; ++mu)
-          for (int par = 0; par < 2 && !e; ++par) {
-            cudaEvent_t e1 = prof_begin(c, mu);
-            e = ka::launch_stream_group(c->pl, q0, cnt, c->L, c->m, mu, par,
-                                        (uint32_t)(c->sweep + s), c->rk, c->stream);
-            if (e1) cudaEventRecord(e1, c->stream);
-          }
+        for (int k = 0; k < chains && !e; ++k) {
+          const int q = q0 + k * per, cnt = std::min(per, c->pl.P - q);
+          if (cnt <= 0) break;
+          const cudaStream_t st = k ? c->side : c->stream;
+          for (int mu = 0; mu < 3 && !e; ++mu)
+            for (int par = 0; par < 2 && !e; ++par) {
+              cudaEvent_t e1 = prof_begin(c, mu);
+              e = ka::launch_stream_group(c->pl, q, cnt, c->L, c->m, mu, par,
+                                          (uint32_t)(c->sweep + s), c->rk, st);
+              if (e1) cudaEventRecord(e1, c->stream);
+            }
+        }
+    // join, also after an error: nothing is left running beside the context's stream
+    if (chains > 1) {
+      cudaError_t ej = cudaEventRecord(c->join, c->side);
+      if (!ej) ej = cudaStreamWaitEvent(c->stream, c->join, 0);
+      if (!e) e = ej;
     }
   } else if (c->pencil) {
     const ka::CubicShape sh{c->d, c->L, c->m};
@@ -745,6 +778,7 @@ ka_status ka_destroy(ka_ctx* c) {
   if (e) st = KA_ECUDA;
   else st = check_device_error(c);
   for (cudaEvent_t ev : c->ev) cudaEventDestroy(ev);
+  free_side(c);
   if (c->owns && c->buf) cudaFree(c->buf);
   delete c;
   return st;

@@ -27,6 +27,11 @@ struct ka_ctx {
   const int32_t* coff = nullptr;
   int64_t class_max = 0;            // bonds of the largest class
   int sms = 0;
+  // side stream of the second chain of planes of large three-dimensional
+  // lattices (ka_internal.cuh: stream_chains), made with the context; the
+  // context's stream waits for it before a sweep call returns
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
   ka::Topology host;  // class offsets (graphs) and tables for inspection
   bool initialized = false;
   int64_t sweep = 0, K = -1;

@@ -33,6 +33,24 @@ int stream_planes_per_launch(int L, int P) {
   return P < cap ? P : cap;
 }
 
+int stream_chains(int L, int P, int* per) {
+  // A launch ends in a tail of CTAs that do not fill the device, and the next
+  // starts with loads (the SMs of one chain are busy 71-74 % of the time): two
+  // chains of planes on two streams fill each other's gaps.  us a sweep, one
+  // chain / two: L = 128 4 planes 126 / 98.6, 3 98 / 84.7, 2 61.7 / 49.8; 112 4
+  // 105 / 87.2, 3 69.8 / 62.5; 100 3 63.7 / 56.3; 80 4 45.7 / 37.0; 64 4 25.1 / 23.6, 2
+  // 24.2 / 19.9; 48 4 21.3 / 21.3, 3 20.3 / 20.9 (launches of 3 us, no gap to fill).
+  *per = stream_planes_per_launch(L, P);
+  if (P < 2 || L < 60) return 1;
+  // All planes at once while their n and p stay in the L2 (85 MB: L = 120 3 planes
+  // two a launch 80.4, one 88.2; 128 3 planes 89.3, 84.7), else one half of what
+  // one chain would hold.
+  const double bytes = 16.0 * (double)L * L * L * P;
+  const int half = bytes <= 85.0e6 ? (P + 1) / 2 : *per / 2;
+  *per = half < 1 ? 1 : half > stream::kMaxPlanes ? stream::kMaxPlanes : half;
+  return 2;
+}
+
 cudaError_t launch_stream_group(const Planes& pl, int q0, int nq, int L, int m, int mu, int par,
                                 uint32_t t, const RoundKeys& rk, cudaStream_t st) {
   using namespace stream;

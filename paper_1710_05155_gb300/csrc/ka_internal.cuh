@@ -260,6 +260,9 @@ bool stream_supported(int d, int L);
 bool stream_reported(int d, int L, int P);
 // planes one launch of these kernels takes
 int stream_planes_per_launch(int L, int P);
+// Chains of launches that P planes run in, side by side, and the planes per
+// launch of each.
+int stream_chains(int L, int P, int* per);
 // Group (mu, par) of sweep t on planes q0 .. q0 + nq - 1.
 cudaError_t launch_stream_group(const Planes& pl, int q0, int nq, int L, int m, int mu, int par,
                                 uint32_t t, const RoundKeys& rk, cudaStream_t st);
