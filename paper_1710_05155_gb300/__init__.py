@@ -226,8 +226,8 @@ def ka_info(ctx: Ctx) -> dict:
 
 def ka_observe(ctx: Ctx, out: np.ndarray | None = None):
     """(sweep, int64 [R, 4]): particles, overlap, persist_occ, persist_all per replica."""
-    R = ka_info(ctx)["replicas"]
     if out is None:
+        R = (ctx.info if ctx.info is not None else ka_info(ctx))["replicas"]
         out = np.zeros((R, 4), np.int64)
     sweep = C.c_int64(0)
     _check(load().ka_observe(ctx.handle, C.byref(sweep), _ptr(out)), "ka_observe", ctx)

@@ -98,7 +98,9 @@ Layout layout_of(const Shape& s) {
   // layout conversion of get/set_state (graphs: breadth-first storage order)
   const bool has_stage = s.V > 1 || s.xs || s.topo != KA_CUBIC;
   l.stage = has_stage ? take(plane) : 0;
-  l.counts = take((size_t)s.R * 4 * sizeof(unsigned long long));
+  // the device error word follows the counts: an observation reads both at once
+  l.counts = take((size_t)s.R * 4 * sizeof(unsigned long long) + sizeof(int32_t));
+  l.err = l.counts + (size_t)s.R * 4 * sizeof(unsigned long long);
   // the initial state's lists: in the staging plane, idle meanwhile, if it
   // holds those of sixteen words (or all), else in room of their own for that
   const int planes = std::max(1, std::min(s.P, 16 / s.V));
@@ -111,7 +113,6 @@ Layout layout_of(const Shape& s) {
   }
   l.list_n = take((size_t)s.R * sizeof(uint32_t));
   l.below = take((size_t)s.R * sizeof(unsigned long long));
-  l.err = take(sizeof(int32_t));
   if (!s.pencil) {
     l.nbr = take((size_t)s.N * s.z * sizeof(int32_t));
     l.bu = take((size_t)s.E * sizeof(int32_t));
@@ -352,22 +353,25 @@ ka_status drain_profile(ka_ctx* c) {
   return KA_OK;
 }
 
-// Read (and clear) the device error word of the bounded waits; synchronises
-// the context stream.  KA_ETIMEOUT when a wait ran out since the last check.
+// KA_ETIMEOUT (and the word cleared) when a bounded wait ran out since the
+// last check: h is the device error word as just read.
+ka_status report_device_error(ka_ctx* c, int h) {
+  if (!h) return KA_OK;
+  cudaError_t e = cudaMemsetAsync(c->err_dev, 0, sizeof(int), c->stream);
+  if (!e) e = cudaStreamSynchronize(c->stream);
+  if (e) return cuda_fail(c, e, "sync");
+  return fail(c, KA_ETIMEOUT,
+              std::string("a bounded device wait ran out (code ") +
+                  std::to_string(h) + "); the state of this context is not valid");
+}
+
+// Read the device error word; synchronises the context stream.
 ka_status check_device_error(ka_ctx* c) {
   int h = 0;
   cudaError_t e = cudaMemcpyAsync(&h, c->err_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
   if (!e) e = cudaStreamSynchronize(c->stream);
   if (e) return cuda_fail(c, e, "sync");
-  if (h) {
-    e = cudaMemsetAsync(c->err_dev, 0, sizeof(int), c->stream);
-    if (!e) e = cudaStreamSynchronize(c->stream);
-    if (e) return cuda_fail(c, e, "sync");
-    return fail(c, KA_ETIMEOUT,
-                std::string("a bounded device wait ran out (code ") +
-                    std::to_string(h) + "); the state of this context is not valid");
-  }
-  return KA_OK;
+  return report_device_error(c, h);
 }
 
 }  // namespace
@@ -483,7 +487,10 @@ ka_status ka_sweep(ka_ctx* c, int64_t n) {
   cudaError_t e = cudaSuccess;
   // profiling times one group or class per launch
   const int C = c->prof ? 0 : ka::resident_cluster(c, c->pl.W);
-  if (C) {
+  const bool on_chip = C && (c->topo == KA_CUBIC
+                                 ? ka::resident::cubic_pays(c->d, c->L, c->pl.P, C, c->sms, n)
+                                 : ka::resident::graph_pays(c->N, c->pl.W, C, c->sms, n));
+  if (on_chip) {
     ka::resident::Args a{};
     a.plane_elems = c->pl.plane_elems();
     a.words_per_plane = c->pl.V;
@@ -573,10 +580,18 @@ ka_status ka_observe(ka_ctx* c, int64_t* sweep_out, int64_t* counts) {
   if (!c->initialized) return fail(c, KA_ESTATE, "observe before init or set_state");
   DeviceGuard dg(c->device);
   cudaError_t e = ka::launch_observe(c->pl, c->counts_dev, c->stream);
-  if (!e) e = cudaMemcpyAsync(counts, c->counts_dev, (size_t)c->R * 4 * sizeof(int64_t),
+  // counts and error word in one copy: each copy to pageable memory waits for
+  // the stream (10 sweeps and an observation at L = 16: 109 us with two)
+  const size_t bytes = (size_t)c->R * 4 * sizeof(int64_t);
+  c->observed.resize((size_t)c->R * 4 + 1);
+  if (!e) e = cudaMemcpyAsync(c->observed.data(), c->counts_dev, bytes + sizeof(int32_t),
                               cudaMemcpyDeviceToHost, c->stream);
+  if (!e) e = cudaStreamSynchronize(c->stream);
   if (e) return cuda_fail(c, e, "observe");
-  if (ka_status st = check_device_error(c)) return st;
+  std::memcpy(counts, c->observed.data(), bytes);
+  int32_t timed_out = 0;
+  std::memcpy(&timed_out, c->observed.data() + (size_t)c->R * 4, sizeof(timed_out));
+  if (ka_status st = report_device_error(c, timed_out)) return st;
   if (sweep_out) *sweep_out = c->sweep;
   return KA_OK;
 }

@@ -166,8 +166,12 @@ cudaError_t dev_alloc(ka_batch* b, T** p, size_t count) {
 // `words`: those of all jobs of its lattice (d, L, m).
 bool add_resident(ka_batch* b, Job* j, int64_t words) {
   const ka_ctx* c = j->ctx;
-  if (!ka::resident_cluster(c, words)) return false;
+  const int C = ka::resident_cluster(c, words);
   const bool cubic = c->topo == KA_CUBIC;
+  // rounds are of several sweeps; one launch per group covers all planes of a
+  // lattice (d, L, m), so only their time on chip counts here
+  if (!C || (cubic && !ka::resident::cubic_pays(c->d, c->L, c->d == 3 ? 1 : words, C, c->sms, 16)))
+    return false;
   ResidentClass* rc = nullptr;
   for (auto& x : b->resident) {
     if (x.m != c->m) continue;
@@ -355,7 +359,9 @@ cudaError_t rebuild(ka_batch* b) {
 // three-dimensional lattices or the single-instance pencil kernel, arguments
 // in the constant bank); a cubic lattice on the edge-gather path never.
 bool shares_launches(const ka_batch* b, const ka_ctx* ctx) {
-  if (ctx->topo != KA_CUBIC || ka::resident_cluster(ctx, ctx->pl.W)) return true;
+  if (ctx->topo != KA_CUBIC) return true;
+  const int C = ka::resident_cluster(ctx, ctx->pl.W);
+  if (C && ka::resident::cubic_pays(ctx->d, ctx->L, ctx->d == 3 ? 1 : ctx->pl.W, C, ctx->sms, 16)) return true;
   if (!ctx->pencil) return false;
   int64_t pencils = 1;
   for (int k = 0; k < ctx->d - 1; ++k) pencils *= ctx->L;

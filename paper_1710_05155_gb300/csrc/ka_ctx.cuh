@@ -20,7 +20,8 @@ struct ka_ctx {
   ka::Planes pl{};
   ka::InitScratch is{};
   unsigned long long* counts_dev = nullptr;
-  int* err_dev = nullptr;  // device error word of bounded device waits (0 = none)
+  int* err_dev = nullptr;  // device error word of bounded device waits (0 = none), after the counts
+  std::vector<int64_t> observed;  // host copy of the counts and that word
   uint64_t* stage = nullptr;
   ka::GraphDev g{};
   const uint4* rec = nullptr;       // small graphs: packed bonds and class offsets (ka_resident.cuh)

@@ -34,6 +34,7 @@ namespace {
 // binary digits of a thread's counters: up to 120 words, or (small planes) 8
 constexpr int kDigits = 7, kFewDigits = 4;
 constexpr int kPerThread = 120, kFew = 8;
+constexpr size_t kOneBlock = 8192;  // words of a plane that one block takes
 
 // ALL: the four observables; else only the particles
 template <int V, bool ALL, int S>
@@ -87,27 +88,31 @@ __global__ void __launch_bounds__(256, 2) k_observe(Planes pl, unsigned long lon
   for (int k = threadIdx.x; k < O * 64 * V; k += blockDim.x) {
     const int o = k / (64 * V), rb = k % (64 * V);  // rb = h * 64 + bit
     const unsigned int v = acc[o][rb];
-    if (v) {
-      const int r = (q * V + rb / 64) * 64 + (rb % 64);
-      atomicAdd(&counts[(size_t)r * O + o], (unsigned long long)v);
-    }
+    const int r = (q * V + rb / 64) * 64 + (rb % 64);
+    if (gridDim.x == 1) counts[(size_t)r * O + o] = v;  // the plane's only block
+    else if (v) atomicAdd(&counts[(size_t)r * O + o], (unsigned long long)v);
   }
 }
 
 template <bool ALL>
 cudaError_t launch_counts(const Planes& pl, unsigned long long* counts_dev, cudaStream_t st) {
-  cudaError_t err = cudaMemsetAsync(
-      counts_dev, 0, (size_t)pl.P * pl.V * 64 * (ALL ? 4 : 1) * sizeof(unsigned long long), st);
-  if (err != cudaSuccess) return err;
   // words per thread, in eights: one wave of two blocks per SM over all planes
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const size_t E = pl.plane_elems();
   const size_t wave = (size_t)256 * 2 * (size_t)(sms > 0 ? sms : 148);
   size_t per_thread = (E * (size_t)pl.P + wave - 1) / wave;
+  // a small plane is one block's, which stores its counts: no clearing launch
+  // before (2 us; 16 more words a thread take a fraction of that)
+  if (E <= kOneBlock) per_thread = std::max(per_thread, (E + 255) / 256);
   per_thread = std::min<size_t>((per_thread + 7) / 8 * 8, kPerThread);
   const size_t per_block = 256 * per_thread;
   const dim3 grid((unsigned)((E + per_block - 1) / per_block), (unsigned)pl.P);
+  if (grid.x > 1) {
+    const cudaError_t err = cudaMemsetAsync(
+        counts_dev, 0, (size_t)pl.P * pl.V * 64 * (ALL ? 4 : 1) * sizeof(unsigned long long), st);
+    if (err != cudaSuccess) return err;
+  }
   const bool few = per_thread <= kFew;
 #define KA_LAUNCH(V, S) k_observe<V, ALL, S><<<grid, 256, 0, st>>>(pl, counts_dev, (int)per_thread)
   if (pl.V == 4) {

@@ -73,11 +73,15 @@ inline int cubic_threads(int64_t N, int L, int C) {
 // CTAs per word for `words` words of a cubic lattice (d, L) in one launch, or
 // 0 when the lattice does not run here.
 int cubic_cluster(int d, int L, int64_t words, int sms);
+// whether n sweeps of `planes` one-word planes take less time on chip (C CTAs per
+// word) than with a launch per group
+bool cubic_pays(int d, int L, int64_t planes, int C, int sms, int64_t n);
 cudaError_t launch_cubic(const Args& a, int d, int L, int m, unsigned words, int C,
                          cudaStream_t st);
 // whether a graph of N sites may run here, and its CTAs per word (0: it does not)
 bool graph_fits(int64_t N);
 int graph_cluster(int64_t N, int64_t nbonds, int64_t class_max);
+bool graph_pays(int64_t N, int64_t words, int C, int sms, int64_t n);
 // the packed record of every bond, from tables in storage positions
 int graph_record_bytes(int z);
 void graph_records(int64_t N, int z, const int32_t* nbr, const int32_t* bu, const int32_t* bv,
@@ -232,7 +236,8 @@ __device__ __forceinline__ void store_plane(const Unit& su, const uint64_t* n, i
 template <typename Kern>
 cudaError_t launch_cluster(Kern kern, const Args& a, unsigned words, int C, int threads, size_t smem,
                            cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(words * (unsigned)C);

@@ -17,12 +17,6 @@ int cubic_cluster(int d, int L, int64_t words, int sms) {
   for (int k = 0; k < d; ++k) N *= L;
   // n and the exchange slots (24 bytes for each of at most 1024 threads) in shared memory
   if (N * 8 + 24 * 1024 > (int64_t)kSmemMax - 512) return 0;
-  // us a sweep of one word on chip, against a launch per group: d = 3, L = 16
-  // 6.4 / 9.9, L = 20 9.7 / 14.4, L = 24 14.8 / 14.6, L = 28 22.3 / 15.2; d = 2,
-  // L = 128 10.6 / 12.  On chip up to 19 words run at once in that time, while
-  // group launches grow with them: four words 6.4 / 11.6, 9.7 / 18.2, 14.8 / 16.9,
-  // 22.4 / 24.5 (three: 22.3 / 22.6) and 10.6 / 48.
-  if (d > 2 && words < (N > 16384 ? 4 : N > 8192 ? 2 : 1)) return 0;
   // CTAs per word: a segment's latency bounds small shares, what a group sends
   // large clusters.  us a sweep with 1, 2, 4, 8: L = 8 4.5, 4.9, 5.2, 5.5; L = 12
   // 6.0, 5.1, 5.3, 5.8; L = 16 9.2, 6.6, 6.4, 7.0; L = 20 -, 11.5, 9.7, 10.3; L = 24
@@ -33,6 +27,22 @@ int cubic_cluster(int d, int L, int64_t words, int sms) {
   while (C > 1 && words * C > sms && cubic_threads(N, L, C / 2) <= 1024) C /= 2;
   // every CTA has pencils: each must send in every group
   return (C - 1) * share_of((int)(N / L / 2), C) < N / L / 2 ? C : 0;
+}
+
+bool cubic_pays(int d, int L, int64_t planes, int C, int sms, int64_t n) {
+  // us of a sweep, measured and fitted.  On chip: d = 3, L = 8 to 28 4.5, 5.2,
+  // 6.4, 9.7, 14.8, 22.3; d = 2, L = 16, 64, 128 2.5, 3.6, 10.6; d = 4, L = 8, 12 10.8, 34;
+  // for as many words as run at once.  A launch per group: 10 (L <= 16) to 15 for
+  // up to four planes of a three-dimensional lattice; 12 and 18 to 22 for every
+  // plane of the others.  A launch on chip (planes in and out, the cluster) costs 12
+  // us more: single sweeps of L = 16 10.6, on chip 16.4.
+  double N = 1.0;
+  for (int k = 0; k < d; ++k) N *= L;
+  const double group = d == 3 ? (L <= 16 ? 10.2 : 14.0) * (double)((planes + 3) / 4)
+                              : (d == 2 ? 12.0 : 18.0) * (double)planes;
+  const double chip = d == 3 ? 3.0 + 8.8e-4 * N : d == 2 ? 2.5 + 5.0e-4 * N : 5.0 + 1.4e-3 * N;
+  const double waves = (double)((planes * C + sms - 1) / (sms > 0 ? sms : 1));
+  return group * (double)n > (12.0 + chip * (double)n) * waves;
 }
 
 cudaError_t launch_cubic(const Args& a, int d, int L, int m, unsigned words, int C,

@@ -282,6 +282,15 @@ int graph_cluster(int64_t N, int64_t nbonds, int64_t class_max) {
   return 0;
 }
 
+bool graph_pays(int64_t N, int64_t words, int C, int sms, int64_t n) {
+  // us of a sweep (above): 28 with a launch per class, whatever the words up to
+  // a few hundred thousand site-words, then with them; on chip 12 + 0.0012 N for
+  // as many words as run at once, and 12 for the launch
+  const double group = 28.0 + 2.0e-5 * (double)N * (double)words;
+  const double waves = (double)((words * C + sms - 1) / (sms > 0 ? sms : 1));
+  return group * (double)n > (12.0 + (12.0 + 1.2e-3 * (double)N) * (double)n) * waves;
+}
+
 cudaError_t launch_graph(const Args& args, int64_t Nmax, int64_t bonds_max, int64_t class_max, int z,
                          int m, unsigned words, int C, cudaStream_t st) {
   if (m < 0 || z < 1 || z > 8 || !graph_fits(Nmax) || class_max > 1024 * C)

@@ -31,12 +31,12 @@ def _same(params, topo, seed, rho, steps):
 @pytest.mark.parametrize("d,L,R,m", [
     (2, 4, 64, 1), (2, 12, 192, 0), (2, 36, 128, 3), (2, 64, 64, 1), (2, 68, 64, 2),
     (2, 128, 128, 1), (3, 4, 64, 3), (3, 8, 320, 0), (3, 12, 192, 5), (3, 16, 64, 3),
-    (3, 20, 64, 2), (3, 24, 128, 4), (3, 28, 256, 3), (4, 4, 64, 7), (4, 8, 128, 4),
+    (3, 20, 64, 2), (3, 24, 320, 4), (3, 28, 320, 3), (4, 4, 64, 7), (4, 8, 128, 4),
     (4, 12, 256, 3), (3, 16, 64 * 160, 3),
 ])
 def test_lattices(d, L, R, m):
     _same(dict(topo=K.KA_CUBIC, d=d, L=L, m=m, replicas=R), O.cubic(d, L), 11, 0.65,
-          (1, 2) if L ** d * R < 1 << 22 else (2,))
+          (1, 12) if L ** d * R < 1 << 20 else (3,))
 
 
 @pytest.mark.parametrize("N,z,R,m", [
@@ -46,7 +46,7 @@ def test_lattices(d, L, R, m):
 ])
 def test_random_regular_graphs(N, z, R, m):
     _same(dict(topo=K.KA_RRG, N=N, z=z, m=m, replicas=R, graph_seed=3), O.rrg(N, z, 3), 5, 0.6,
-          (1, 2) if N * R < 1 << 22 else (2,))
+          (1, 5) if N * R < 1 << 20 else (4,))
 
 
 @pytest.mark.parametrize("z,m", [(8, 0), (8, 5), (8, 7), (7, 3)])
@@ -56,7 +56,7 @@ def test_wide_neighbour_rows(z, m):
     nbr = np.array([sorted([(i + k) % N for k in steps] + [(i - k) % N for k in steps] +
                            ([(i + N // 2) % N] if z % 2 else [])) for i in range(N)], np.int32)
     _same(dict(topo=K.KA_GRAPH, N=N, z=z, m=m, replicas=128, nbr=nbr), O.graph(N, z, nbr.reshape(-1)),
-          9, 0.6, (1, 2))
+          9, 0.6, (1, 5))
 
 
 def test_batches_of_small_jobs():
@@ -88,11 +88,11 @@ def test_last_sweep_number():
     with K.Simulation(topo=K.KA_CUBIC, d=3, L=8, m=3, replicas=64) as sim:
         sim.init(3, 0.6)
         n, n0, p = sim.get_state()
-        sim.set_state(n, n0, p, (1 << 32) - 2, 3)
-        sim.sweep(2)
+        sim.set_state(n, n0, p, (1 << 32) - 9, 3)
+        sim.sweep(9)
         st = O.init(topo.N, 64, 3, 0.6)
-        st.t = (1 << 32) - 2
-        O.sweeps(topo, 3, st, 3, 2)
+        st.t = (1 << 32) - 9
+        O.sweeps(topo, 3, st, 3, 9)
         assert np.array_equal(sim.get_state()[0], O.pack_words(st.n))
 
 
