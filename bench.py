@@ -384,7 +384,7 @@ def run_rrg(dev: int, stream, sweeps: int) -> dict:
     ev1.record(stream)
     torch.cuda.synchronize(dev)
     packed_ms = ev0.elapsed_time(ev1)
-    packed_words = packed.info["plane_words"]
+    packed_words, packed_planes = packed.info["plane_words"], packed.info["planes"]
     packed.close()
     packed_value = RRG_N * 64 * len(RRG_RHOS) * sweeps / (packed_ms / 1000.0)
     launches = nclass * sweeps * len(RRG_RHOS)
@@ -395,7 +395,7 @@ def run_rrg(dev: int, stream, sweeps: int) -> dict:
     peak, peak_kind = _peaks()
     traffic = measured_traffic(PROFILE_GRAPH, SRC_GRAPH)
     # packed: one sweep moves all eight densities' words
-    p_launches = nclass * sweeps
+    p_launches = nclass * sweeps * packed_planes  # planes of this size run one by one
     p_achieved = bytes_per_sweep * len(RRG_RHOS) * sweeps / (packed_ms / 1000.0) / 1e9
     return {
         "metric": METRIC, "value": packed_value, "unit": UNIT,
@@ -604,7 +604,9 @@ def run_native(args, rank: int, world: int) -> None:
     counts_dev = [torch.zeros((R, 4), dtype=torch.int64, device=f"cuda:{dev}") for _ in sims]
     info = sims[0].info
     P, nq = info["planes"], info["planes_per_launch"]
-    sets = -(-P // nq)  # launches per group and sweep
+    # outside profiling the planes of a launch run as two chains of half as many
+    nq_run = max(1, nq // 2)
+    sets = -(-P // nq_run)  # launches per group and sweep
     sweep_launches_per_step = len(sims) * sets * S * GROUPS
     launches_per_step = sweep_launches_per_step + len(sims)  # + one observation each
 
@@ -651,7 +653,8 @@ def run_native(args, rank: int, world: int) -> None:
     # one with events around each (ka_profile_read_dirs, by direction), give
     # each kernel's share of the region: k_rows runs the groups along x,
     # k_pencils those along y and z (two thirds of the launches).  A launch
-    # covers nq planes of one group: 32 bytes per site-word-sweep / 6 groups.
+    # covers nq_run planes of one group: 32 bytes per site-word-sweep / 6 groups
+    # (two chains run side by side: the average time is the region's share).
     iso_ms, iso_n = np.zeros(4), np.zeros(4, np.int64)
     for sim in sims:
         K.ka_profile_enable(sim.ctx, True)
@@ -663,7 +666,7 @@ def run_native(args, rank: int, world: int) -> None:
     region_launches = sweep_launches_per_step * args.steps
     pencil_launches = region_launches * 2 // 3
     row_launches = region_launches - pencil_launches
-    bytes_per_launch = BYTES_PER_SITE_WORD_SWEEP * N_SITES * nq / GROUPS
+    bytes_per_launch = BYTES_PER_SITE_WORD_SWEEP * N_SITES * nq_run / GROUPS
     pencil_ms = _apportion(local_ms, iso_ms, (1, 2), pencil_launches)
     row_ms = _apportion(local_ms, iso_ms, (0,), row_launches)
     achieved = bytes_per_launch / (pencil_ms / 1000.0) / 1e9

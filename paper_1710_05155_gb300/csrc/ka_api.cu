@@ -153,8 +153,7 @@ struct DeviceGuard {
 
 void free_side(ka_ctx* c) {
   if (c->side) cudaStreamDestroy(c->side);
-  if (c->fork) cudaEventDestroy(c->fork);
-  if (c->join) cudaEventDestroy(c->join);
+  if (c->turn) cudaEventDestroy(c->turn);
 }
 
 ka_status create_common(const ka_params* params, void* buf, size_t bytes, bool owns, ka_ctx** out) {
@@ -287,8 +286,7 @@ ka_status create_common(const ka_params* params, void* buf, size_t bytes, bool o
   int per = 0;
   if (c->pencil && ka::stream_supported(c->d, c->L) && ka::stream_chains(c->L, c->pl.P, &per) > 1) {
     cudaError_t e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
-    if (!e) e = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming);
-    if (!e) e = cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming);
+    if (!e) e = cudaEventCreateWithFlags(&c->turn, cudaEventDisableTiming);
     if (e) {
       free_side(c);
       if (owns) cudaFree(buf);
@@ -509,8 +507,8 @@ ka_status ka_sweep(ka_ctx* c, int64_t n) {
     int per = ka::stream_planes_per_launch(c->L, c->pl.P);
     const int chains = c->side && !c->prof ? ka::stream_chains(c->L, c->pl.P, &per) : 1;
     if (chains > 1) {
-      e = cudaEventRecord(c->fork, c->stream);
-      if (!e) e = cudaStreamWaitEvent(c->side, c->fork, 0);
+      e = cudaEventRecord(c->turn, c->stream);
+      if (!e) e = cudaStreamWaitEvent(c->side, c->turn, 0);
     }
     // a sweep of one chain, then of the other, so that both have work queued
     for (int q0 = 0; q0 < c->pl.P && !e; q0 += chains * per)
@@ -529,8 +527,8 @@ ka_status ka_sweep(ka_ctx* c, int64_t n) {
         }
     // join, also after an error: nothing is left running beside the context's stream
     if (chains > 1) {
-      cudaError_t ej = cudaEventRecord(c->join, c->side);
-      if (!ej) ej = cudaStreamWaitEvent(c->stream, c->join, 0);
+      cudaError_t ej = cudaEventRecord(c->turn, c->side);
+      if (!ej) ej = cudaStreamWaitEvent(c->stream, c->turn, 0);
       if (!e) e = ej;
     }
   } else if (c->pencil) {

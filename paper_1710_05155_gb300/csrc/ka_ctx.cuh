@@ -32,7 +32,7 @@ struct ka_ctx {
   // lattices (ka_internal.cuh: stream_chains), made with the context; the
   // context's stream waits for it before a sweep call returns
   cudaStream_t side = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr;
+  cudaEvent_t turn = nullptr;  // the fork, then the join, of a call
   ka::Topology host;  // class offsets (graphs) and tables for inspection
   bool initialized = false;
   int64_t sweep = 0, K = -1;

@@ -35,14 +35,17 @@
 namespace ka {
 namespace {
 
-constexpr int kDigits = 7;            // per-thread counters hold up to 127
-constexpr int kSites = 8;             // sites per thread
-constexpr int kSegment = 15;          // vectors per segment: 120 words per thread
+constexpr int kDigits = 8;            // per-thread counters hold up to 255
+constexpr int kSites = 16;            // sites per thread
+constexpr int kPsiSites = 4;          // of the sum over counts: more blocks
+constexpr int kSegment = 15;          // vectors per segment: 240 words per thread
 constexpr int kThreads = 256;
 constexpr int kMaxVectors = 1 << 16;  // displacement vectors per call
 // Scratch when the context's staging plane does not hold one word's padded
 // lattice: this much, or one word's, a slab of layers at a time.
 constexpr size_t kArena = (size_t)256 << 20;
+
+constexpr int64_t kMostPadded = (int64_t)1 << 29;  // elements: 32-bit byte offsets
 
 // Vectors of one shell and weight: offsets [first, first + count).
 struct Segment {
@@ -117,7 +120,7 @@ __global__ void __launch_bounds__(kThreads) k_pad_counts(const __grid_constant__
 }
 
 // phi of words w0 + blockIdx.y over the segments of blockIdx.z
-__global__ void __launch_bounds__(kThreads) k_phi(const __grid_constant__ Slab g,
+__global__ void __launch_bounds__(kThreads, 2) k_phi(const __grid_constant__ Slab g,
                                                   const uint64_t* __restrict__ padded,
                                                   const Segment* __restrict__ seg,
                                                   const int32_t* __restrict__ offset, int nseg,
@@ -125,14 +128,14 @@ __global__ void __launch_bounds__(kThreads) k_phi(const __grid_constant__ Slab g
   __shared__ unsigned int acc[64];
   const uint64_t* q = padded + (size_t)blockIdx.y * g.padded;
   const int64_t s0 = (int64_t)blockIdx.x * (kThreads * kSites) + threadIdx.x;
-  int32_t at[kSites];
+  uint32_t at[kSites];  // byte offsets
   uint64_t own[kSites];
 #pragma unroll
   for (int u = 0; u < kSites; ++u) {
     const int64_t s = s0 + u * kThreads;
     const bool in = s < g.sites;
-    at[u] = (int32_t)centre(g, in ? s : 0);
-    own[u] = in ? q[at[u]] : 0ull;
+    at[u] = 8u * (uint32_t)centre(g, in ? s : 0);
+    own[u] = in ? *reinterpret_cast<const uint64_t*>(reinterpret_cast<const char*>(q) + at[u]) : 0ull;
   }
   const int b0 = (int)((int64_t)nseg * blockIdx.z / gridDim.z);
   const int b1 = (int)((int64_t)nseg * (blockIdx.z + 1) / gridDim.z);
@@ -144,13 +147,16 @@ __global__ void __launch_bounds__(kThreads) k_phi(const __grid_constant__ Slab g
 #pragma unroll
     for (int s = 0; s < kDigits; ++s) c[s] = 0;
     for (int v = 0; v < sg.count; ++v) {
-      const int32_t off = __ldg(offset + sg.first + v);
-      uint64_t x[kSites];
+      const uint32_t off = 8u * (uint32_t)__ldg(offset + sg.first + v);
+      uint64_t x[2][8];
 #pragma unroll
-      for (int u = 0; u < kSites; ++u) x[u] = __ldg(q + (at[u] + off));
+      for (int u = 0; u < kSites; ++u)
+        x[u / 8][u % 8] =
+            __ldg(reinterpret_cast<const uint64_t*>(reinterpret_cast<const char*>(q) + (at[u] + off)));
 #pragma unroll
-      for (int u = 0; u < kSites; ++u) x[u] &= own[u];
-      add8(c, x);
+      for (int u = 0; u < kSites; ++u) x[u / 8][u % 8] &= own[u];
+      add8(c, x[0]);
+      add8(c, x[1]);
     }
     reduce<1, kDigits>(c, acc, (unsigned)sg.weight);
     if (b + 1 == b1 || seg[b + 1].shell != sg.shell) {
@@ -173,11 +179,11 @@ __global__ void __launch_bounds__(kThreads) k_psi(const __grid_constant__ Slab g
                                                   const Segment* __restrict__ seg,
                                                   const int32_t* __restrict__ offset, int nseg,
                                                   unsigned long long* psi) {
-  const int64_t s0 = (int64_t)blockIdx.x * (kThreads * kSites) + threadIdx.x;
-  int32_t at[kSites];
-  uint32_t own[kSites];
+  const int64_t s0 = (int64_t)blockIdx.x * (kThreads * kPsiSites) + threadIdx.x;
+  int32_t at[kPsiSites];
+  uint32_t own[kPsiSites];
 #pragma unroll
-  for (int u = 0; u < kSites; ++u) {
+  for (int u = 0; u < kPsiSites; ++u) {
     const int64_t s = s0 + u * kThreads;
     const bool in = s < g.sites;
     at[u] = (int32_t)centre(g, in ? s : 0);
@@ -192,7 +198,7 @@ __global__ void __launch_bounds__(kThreads) k_psi(const __grid_constant__ Slab g
     for (int v = 0; v < sg.count; ++v) {
       const int32_t off = __ldg(offset + sg.first + v);
 #pragma unroll
-      for (int u = 0; u < kSites; ++u) part += (unsigned long long)own[u] * __ldg(M + (at[u] + off));
+      for (int u = 0; u < kPsiSites; ++u) part += (unsigned long long)own[u] * __ldg(M + (at[u] + off));
     }
     sum += part * (unsigned)sg.weight;
     if (b + 1 == b1 || seg[b + 1].shell != sg.shell) {
@@ -254,7 +260,7 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
   for (int k = 1; k < 4; ++k) g.ps[k] = g.ps[k - 1] * (L + 2 * rad);
   const int64_t layer = g.ps[d - 1];
   const int64_t layer_sites = c->N / L;
-  const int64_t most = std::min<int64_t>((int64_t)1 << 30, (int64_t)(kArena / sizeof(uint64_t)));
+  const int64_t most = (int64_t)(kArena / sizeof(uint64_t));
   const size_t stage_bytes = c->stage ? (size_t)c->N * c->pl.W * sizeof(uint64_t) : 0;
 
   struct Vec {
@@ -310,12 +316,12 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
   int words = 0;  // per pass
   char* own = nullptr;
   char* mem = nullptr;
-  if (layer * (L + 2 * rad) <= (int64_t)1 << 30 && stage_bytes >= fixed + m_bytes(L) + q_bytes(L)) {
+  if (layer * (L + 2 * rad) < kMostPadded && stage_bytes >= fixed + m_bytes(L) + q_bytes(L)) {
     mem = (char*)c->stage;
     words = (int)std::min<size_t>((size_t)W, (stage_bytes - fixed - m_bytes(L)) / q_bytes(L));
   } else {
     if (layer * (zc + 2 * rad) > most) zc = std::max<int64_t>(1, most / layer - 2 * rad);
-    if (layer * (zc + 2 * rad) >= (int64_t)1 << 31)
+    if (layer * (zc + 2 * rad) >= kMostPadded)
       return four_point_fail(c, KA_ENOMEM, "scratch: a padded layer is too large");
     words = (int)std::max<size_t>(1, std::min<size_t>((size_t)W, kArena / q_bytes(zc)));
     const size_t total = fixed + m_bytes(zc) + (size_t)words * q_bytes(zc);
@@ -346,7 +352,8 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
     const unsigned tiles = (unsigned)((g.sites + kThreads * kSites - 1) / (kThreads * kSites));
     if (psi) {
       k_pad_counts<<<pads, kThreads, 0, st>>>(pl, g, M);
-      k_psi<<<dim3(tiles, 1, split(tiles)), kThreads, 0, st>>>(g, M, seg_dev, off_dev, nseg, psi_dev);
+      const unsigned psi_tiles = (unsigned)((g.sites + kThreads * kPsiSites - 1) / (kThreads * kPsiSites));
+      k_psi<<<dim3(psi_tiles, 1, split(psi_tiles)), kThreads, 0, st>>>(g, M, seg_dev, off_dev, nseg, psi_dev);
       e = cudaGetLastError();
     }
     for (int w0 = 0; w0 < W && !e; w0 += words) {
