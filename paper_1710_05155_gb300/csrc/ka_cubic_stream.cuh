@@ -534,7 +534,7 @@ cudaError_t launch_pencils(const Args& a, cudaStream_t st) {
   // Chunks per warp: with more, pencils are cut into shorter chunks and spread
   // over more CTAs, at the price of shorter runs.  Up to L = 24 a chunk is a
   // single segment anyway; up to L = 64 it is with two.  us a sweep, 64 / 192
-  // replicas, with one, two and four: L = 40 22.3, 16.8, 15.7 / 23.9, 20.2, 22.8; 48 22.7, 17.2, 17.3 / 25.9,
+  // replicas, with one, two and four: L = 24 15.1, 15.1, 14.1 / 15.2 each; L = 40 22.3, 16.8, 15.7 / 23.9, 20.2, 22.8; 48 22.7, 17.2, 17.3 / 25.9,
   // 20.4, 20.2; 60 23.8, 20.3, 26.0 / 27.4, 22.6, 28.8; 64 25.4, 21.4, 24.1 / 25.9,
   // 24.8, 26.9.  Above, one plane leaves SMs idle up to L = 100 unless four share
   // it: L = 72 27.8, 25.3, 22.8 / 37.9, 34.0, 33.5; 88 27.1, 29.3, 26.5 / 43.8, 51.4,
@@ -542,7 +542,7 @@ cudaError_t launch_pencils(const Args& a, cudaStream_t st) {
   if constexpr (LT > 24 && LT <= 64) {
     return launch_pencils_ch<LT, M, 2>(a, st);
   } else {
-    if constexpr (LT > 64 && LT <= 100)
+    if constexpr (LT == 24 || (LT > 64 && LT <= 100))
       if (a.nplanes == 1) return launch_pencils_ch<LT, M, 4>(a, st);
     return launch_pencils_ch<LT, M, 1>(a, st);
   }
