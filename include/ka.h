@@ -168,7 +168,7 @@ ka_status ka_sweep(ka_ctx *ctx, int64_t n);
  * key = the dynamics seed, draw = 0, 1, ... until accepted, and takes site
  * i = r / z and its neighbour in slot r mod z (on cubic lattices slot 2 mu is
  * the up and 2 mu + 1 the down neighbour along mu; on graphs the slots are
- * the neighbour row in ascending order, as ka_graph_tables returns it).  One warp per word runs
+ * the neighbour row in ascending order, as ka_graph_tables returns it).  One CTA per word runs
  * the chain, 32 attempts at a time, applying together the attempts that do
  * not touch each other's sites (the result is the in-order chain's), in
  * shared memory when the lattice has at most 10240 sites.  Advances the sweep

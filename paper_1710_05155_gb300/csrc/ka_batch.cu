@@ -5,7 +5,7 @@
 // advances all unfinished jobs by up to k sweeps: for every sweep offset s
 // and every bond-class group, ONE launch covers all work units (job planes)
 // of a shape class: the group kernels of three-dimensional lattices for the
-// units of one side and m (d = 3), the general pencil kernel for the cubic
+// units of one side and m (d = 3), the general pencil kernel for the other cubic
 // units of one (d, V, m) otherwise; and ONE launch of the edge-gather kernel
 // covers class c of all graph units of a shape class (V, m).  Units of small
 // topologies stay on chip: one launch runs their whole round.  Units carry their own sweep counter t_base and stop counter t_end
