@@ -18,12 +18,16 @@ __device__ __forceinline__ uint64_t add2(uint64_t& s, uint64_t x, uint64_t y) {
   return k;
 }
 
-// c += x[0] + .. + x[7]
+// the first two digits of c += x[0] + .. + x[3]; returns the carry of weight four
 template <int S>
-__device__ __forceinline__ void add8(uint64_t (&c)[S], const uint64_t (&x)[8]) {
+__device__ __forceinline__ uint64_t add4(uint64_t (&c)[S], const uint64_t (&x)[4]) {
   const uint64_t t0 = add2(c[0], x[0], x[1]), t1 = add2(c[0], x[2], x[3]);
-  const uint64_t t2 = add2(c[0], x[4], x[5]), t3 = add2(c[0], x[6], x[7]);
-  const uint64_t f0 = add2(c[1], t0, t1), f1 = add2(c[1], t2, t3);
+  return add2(c[1], t0, t1);
+}
+
+// the digits from weight four on: c += 4 (f0 + f1)
+template <int S>
+__device__ __forceinline__ void carry8(uint64_t (&c)[S], uint64_t f0, uint64_t f1) {
   uint64_t k = add2(c[2], f0, f1);
 #pragma unroll
   for (int s = 3; s < S; ++s) {
@@ -31,6 +35,14 @@ __device__ __forceinline__ void add8(uint64_t (&c)[S], const uint64_t (&x)[8]) {
     c[s] ^= k;
     k = n;
   }
+}
+
+// c += x[0] + .. + x[7]
+template <int S>
+__device__ __forceinline__ void add8(uint64_t (&c)[S], const uint64_t (&x)[8]) {
+  const uint64_t lo[4] = {x[0], x[1], x[2], x[3]}, hi[4] = {x[4], x[5], x[6], x[7]};
+  const uint64_t f0 = add4(c, lo), f1 = add4(c, hi);
+  carry8(c, f0, f1);
 }
 
 // The warp total of one counter set, one integer per replica times weight, added

@@ -21,8 +21,14 @@
 // gives.
 //
 // What bounds it: the read of n, n0 and p (24 bytes a site-word).  L = 128, 256
-// replicas: 201 MB; before (14 words a thread, ripple adders) 106 us, bound by
-// the ALUs (82 %).
+// replicas: 201 MB, 39 us (5.1 TB/s, 0.76 of the copy rate).  With ripple adders
+// 106 us (ALUs 82 %); eight words loaded, then added, 49; the next four words in
+// flight meanwhile 42.4 (a ring of cp.async in shared memory with twice as many in
+// flight gave the same, so that is enough).  The rest was around the reads:
+// counts cleared by a launch that this one starts beside (instead of a memset
+// before), additions to the counts in the order of the result (a warp's used to
+// touch 32 sectors, now 8), words a thread in fours for a fuller wave: 39.2, and
+// 16.6 -> 8.4 us for 2^18 sites with 128 replicas.
 #include <algorithm>
 #include <mutex>
 
@@ -58,72 +64,112 @@ __global__ void __launch_bounds__(256, 2) k_observe(Planes pl, unsigned long lon
   for (int o = 0; o < O; ++o)
 #pragma unroll
     for (int s = 0; s < S; ++s) c[o][s] = 0;
-  for (int k = 0; k < per_thread; k += 8) {
-    uint64_t n[8], n0[8], p[8];
+  // four words of each array at a time, the next four in flight meanwhile
+  struct Four {
+    uint64_t n[4], n0[ALL ? 4 : 1], p[ALL ? 4 : 1];
+  };
+  auto load = [&](int k, Four& x) {
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < 4; ++u) {
       const size_t e = e0 + (size_t)(k + u) * blockDim.x;
-      const bool in = e < E;
-      n[u] = in ? gn[e] : 0ull;
+      const bool in = k < per_thread && e < E;
+      x.n[u] = in ? gn[e] : 0ull;
       if constexpr (ALL) {
-        n0[u] = in ? g0[e] : 0ull;
-        p[u] = in ? gp[e] : 0ull;
+        x.n0[u] = in ? g0[e] : 0ull;
+        x.p[u] = in ? gp[e] : 0ull;
       }
     }
-    add8(c[0], n);
+  };
+  // the first two digits take four words; their carries of weight four
+  auto first = [&](Four& x, uint64_t (&f)[O]) {
+    f[0] = add4(c[0], x.n);
     if constexpr (ALL) {
-      add8(c[3], p);
+      f[3] = add4(c[3], x.p);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        n[u] &= n0[u];
-        p[u] &= n0[u];
+      for (int u = 0; u < 4; ++u) {
+        x.n[u] &= x.n0[u];
+        x.p[u] &= x.n0[u];
       }
-      add8(c[1], n);
-      add8(c[2], p);
+      f[1] = add4(c[1], x.n);
+      f[2] = add4(c[2], x.p);
     }
+  };
+  Four a, b;
+  uint64_t f0[O], f1[O];
+  load(0, a);
+  for (int k = 0; k < per_thread; k += 8) {
+    load(k + 4, b);
+    first(a, f0);
+    load(k + 8, a);
+    first(b, f1);
+#pragma unroll
+    for (int o = 0; o < O; ++o) carry8(c[o], f0[o], f1[o]);
   }
 #pragma unroll
   for (int o = 0; o < O; ++o) reduce<V, S>(c[o], acc[o]);
   __syncthreads();
+  // the clearing launch is complete
+  if (gridDim.x > 1) asm volatile("griddepcontrol.wait;" ::: "memory");
+  // in the order of the result, so that a warp's additions share sectors
+  unsigned long long* out = counts + (size_t)q * V * 64 * O;
   for (int k = threadIdx.x; k < O * 64 * V; k += blockDim.x) {
-    const int o = k / (64 * V), rb = k % (64 * V);  // rb = h * 64 + bit
-    const unsigned int v = acc[o][rb];
-    const int r = (q * V + rb / 64) * 64 + (rb % 64);
-    if (gridDim.x == 1) counts[(size_t)r * O + o] = v;  // the plane's only block
-    else if (v) atomicAdd(&counts[(size_t)r * O + o], (unsigned long long)v);
+    const unsigned int v = acc[k % O][k / O];  // k / O = h * 64 + bit
+    if (gridDim.x == 1) out[k] = v;  // the plane's only block
+    else if (v) atomicAdd(&out[k], (unsigned long long)v);
   }
+}
+
+// Sets the counts to zero; the counting launch starts at once beside it.  This
+// launch itself starts when all work before it on the stream is complete.
+__global__ void k_clear(unsigned long long* counts, int n) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < n) counts[k] = 0;
 }
 
 template <bool ALL>
 cudaError_t launch_counts(const Planes& pl, unsigned long long* counts_dev, cudaStream_t st) {
-  // words per thread, in eights: one wave of two blocks per SM over all planes
+  // words per thread, in fours: one wave of two blocks per SM over all planes
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const size_t E = pl.plane_elems();
   const size_t wave = (size_t)256 * 2 * (size_t)(sms > 0 ? sms : 148);
   size_t per_thread = (E * (size_t)pl.P + wave - 1) / wave;
   // a small plane is one block's, which stores its counts: no clearing launch
-  // before (2 us; 16 more words a thread take a fraction of that)
+  // before (1 us; 16 more words a thread take a fraction of that)
   if (E <= kOneBlock) per_thread = std::max(per_thread, (E + 255) / 256);
-  per_thread = std::min<size_t>((per_thread + 7) / 8 * 8, kPerThread);
+  per_thread = std::min<size_t>((per_thread + 3) / 4 * 4, kPerThread);
   const size_t per_block = 256 * per_thread;
   const dim3 grid((unsigned)((E + per_block - 1) / per_block), (unsigned)pl.P);
-  if (grid.x > 1) {
-    const cudaError_t err = cudaMemsetAsync(
-        counts_dev, 0, (size_t)pl.P * pl.V * 64 * (ALL ? 4 : 1) * sizeof(unsigned long long), st);
+  const bool many = grid.x > 1;
+  if (many) {
+    const int n = pl.P * pl.V * 64 * (ALL ? 4 : 1);
+    k_clear<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(counts_dev, n);
+    const cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
   }
   const bool few = per_thread <= kFew;
-#define KA_LAUNCH(V, S) k_observe<V, ALL, S><<<grid, 256, 0, st>>>(pl, counts_dev, (int)per_thread)
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = many ? 1 : 0;
+#define KA_LAUNCH(V, S) \
+  return cudaLaunchKernelEx(&cfg, k_observe<V, ALL, S>, pl, counts_dev, (int)per_thread)
   if (pl.V == 4) {
-    if (few) KA_LAUNCH(4, kFewDigits); else KA_LAUNCH(4, kDigits);
+    if (few) KA_LAUNCH(4, kFewDigits);
+    KA_LAUNCH(4, kDigits);
   } else if (pl.V == 2) {
-    if (few) KA_LAUNCH(2, kFewDigits); else KA_LAUNCH(2, kDigits);
-  } else {
-    if (few) KA_LAUNCH(1, kFewDigits); else KA_LAUNCH(1, kDigits);
+    if (few) KA_LAUNCH(2, kFewDigits);
+    KA_LAUNCH(2, kDigits);
   }
+  if (few) KA_LAUNCH(1, kFewDigits);
+  KA_LAUNCH(1, kDigits);
 #undef KA_LAUNCH
-  return cudaGetLastError();
 }
 
 }  // namespace

@@ -39,7 +39,8 @@ def test_initial_states(kw, topo):
             assert np.array_equal(sim.observe()[1], O.observe(st))
 
 
-@pytest.mark.parametrize("R,N", [(64, 1), (64, 2048 * 3 + 1), (128, 300_000), (4096, 130)])
+@pytest.mark.parametrize("R,N", [(64, 1), (64, 2048 * 3 + 1), (128, 300_000), (4096, 130),
+                                 (64, 800_001), (192, 500_001)])  # an odd number of fours a thread
 def test_counts_of_arbitrary_planes(R, N):
     """Full, empty and random words: every digit of the counters, tails of every tile."""
     import torch
