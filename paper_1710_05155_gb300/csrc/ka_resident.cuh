@@ -141,7 +141,7 @@ struct GroupEnd {
   __device__ __forceinline__ void wait(int* err) {
     const uint32_t parity = (phase >> 1) & 1u;
     uint32_t done = 0;
-    for (int i = 0; i < (1 << 22) && !done && !dead; ++i)
+    for (int i = 0; i < (1 << 20) && !done && !dead; ++i)
       asm volatile(
           "{\n.reg .pred q;\n"
           "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], %2;\n"
