@@ -745,7 +745,7 @@ def run_native(args, rank: int, world: int) -> None:
             achieved=achieved, peak=peak, peak_kind=peak_kind, traffic=traffic,
             pencil_ms=pencil_ms, pencil_iso_ms=float(iso_ms[1:3].sum() / iso_n[1:3].sum()),
             row_ms=row_ms, row_iso_ms=float(iso_ms[0] / iso_n[0]),
-            bytes_per_launch=bytes_per_launch, nq=nq, path_achieved=path_achieved,
+            bytes_per_launch=bytes_per_launch, nq=nq_run, path_achieved=path_achieved,
             cpu=extra.pop("cpu_baseline", None), e2e_value=e2e_value, h2d=h2d, d2h=d2h,
             gpu_launches=launches_per_step * args.steps, clocks=clk, extra=extra)
         print(json.dumps(line), flush=True)
