@@ -24,6 +24,9 @@
 // p is not read: the bits that swaps clear are collected in shared memory
 // (cubic: per site; graphs: per bond) and cleared in p by one atomic AND per
 // word at the end; where a lattice leaves no room for that, at each swap.
+// They are collected outside the group ends, while the others' words are
+// awaited: a graph's by the bond's own thread, a lattice's by whichever thread
+// has the site in the group, with a CTA barrier at the end of each sweep.
 #pragma once
 
 #include "ka_internal.cuh"

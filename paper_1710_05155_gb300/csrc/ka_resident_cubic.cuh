@@ -149,6 +149,9 @@ __global__ void __launch_bounds__(1024) k_resident_cubic(const __grid_constant__
   auto mark = [&](int i0, int i1, int i2, int i3, uint64_t f0, uint64_t f1, uint64_t f2, uint64_t f3) {
     if (fsmem) {
       const uint64_t e0 = f[i0], e1 = f[i1], e2 = f[i2], e3 = f[i3];
+#ifdef KA_SLOW_MARKS  // test builds: a delay here lets the other warps run ahead
+      KA_SLOW_MARKS;
+#endif
       f[i0] = e0 | f0;
       f[i1] = e1 | f1;
       f[i2] = e2 | f2;
@@ -320,6 +323,13 @@ __global__ void __launch_bounds__(1024) k_resident_cubic(const __grid_constant__
       gates(gn ? t : t + 1, gn >> 1, gn & 1);
       ge.wait(su.err);
     }
+    // Marks are made after the arrival, so a wait says nothing about other
+    // warps' marks.  Inside a sweep none meet without a barrier between: the
+    // two groups of mu = 0 have different rows, those of mu > 0 barriers of
+    // their own.  The last group's would meet the next sweep's first and the
+    // final loop's reads, so the CTA meets here (us a sweep without and with:
+    // L = 16 6.4, 6.4; L = 20 9.7, 9.8; d = 2, L = 128, 256 replicas 10.6, 10.9).
+    __syncthreads();
   }
   store_plane(su, n, N, rank, C);
   if (fsmem)
