@@ -236,11 +236,14 @@ __device__ __forceinline__ void store_plane(const Unit& su, const uint64_t* n, i
     su.n[(size_t)i * su.stride] = n[i];
 }
 
+// most: the largest smem of any launch of the kernel.  The attribute belongs to the
+// kernel, not to the launch: always the same value, so that host threads whose
+// launches want different amounts do not take it from each other.
 template <typename Kern>
 cudaError_t launch_cluster(Kern kern, const Args& a, unsigned words, int C, int threads, size_t smem,
-                           cudaStream_t st) {
+                           size_t most, cudaStream_t st) {
   const cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(words * (unsigned)C);

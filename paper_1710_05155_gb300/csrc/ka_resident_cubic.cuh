@@ -352,7 +352,7 @@ constexpr size_t kCubicSmem = kSmemMax - 512;  // beside the unit and the mbarri
 
 template <int D, int M, int C, bool B>
 cudaError_t launch_c(const Args& a, unsigned words, int threads, size_t smem, cudaStream_t st) {
-  return launch_cluster(k_resident_cubic<D, M, C, B>, a, words, C, threads, smem, st);
+  return launch_cluster(k_resident_cubic<D, M, C, B>, a, words, C, threads, smem, kCubicSmem, st);
 }
 
 template <int D, int M>

@@ -194,14 +194,18 @@ __global__ void __launch_bounds__(1024) k_resident_graph(const __grid_constant__
   cluster_wait();
 }
 
+constexpr size_t kGraphSmem = kSmemMax - 2560;  // beside the unit and the class tables
+
 template <int Z, int M>
 cudaError_t launch_m(const Args& a, unsigned words, int C, int threads, size_t smem, cudaStream_t st) {
   const bool b = a.units != nullptr;
   switch (C) {
 #define KA_C(CC)                                                                              \
   case CC:                                                                                    \
-    return b ? launch_cluster(k_resident_graph<Z, M, CC, true>, a, words, CC, threads, smem, st) \
-             : launch_cluster(k_resident_graph<Z, M, CC, false>, a, words, CC, threads, smem, st);
+    return b ? launch_cluster(k_resident_graph<Z, M, CC, true>, a, words, CC, threads, smem,   \
+                              kGraphSmem, st)                                                 \
+             : launch_cluster(k_resident_graph<Z, M, CC, false>, a, words, CC, threads, smem,  \
+                              kGraphSmem, st);
     KA_C(1)
     KA_C(4)
 #undef KA_C
@@ -240,8 +244,6 @@ size_t smem_for(int64_t N, int64_t class_max, int64_t nbonds, int C) {
   return 2 * (size_t)entries_for(class_max, C) * 8 + (size_t)(N + 2) * 8 +
          (size_t)fslots_for(nbonds, C) * 8;
 }
-
-constexpr size_t kGraphSmem = kSmemMax - 2560;  // beside the unit and the class tables
 
 }  // namespace
 

@@ -44,6 +44,7 @@ namespace {
 
 constexpr uint32_t kTagSequential = 0xFFFFFFFCu;
 constexpr int kSmemWords = 20480;  // n and p of up to 10240 sites in shared memory
+constexpr size_t kSmemMost = (size_t)227 * 1024;  // shared memory of a CTA
 constexpr int kMakers = 7;         // warps that prepare attempts
 constexpr uint32_t kMaxStamps = 2048;  // words of one of a maker's two stamp tables, at most
 
@@ -352,8 +353,9 @@ __global__ void __launch_bounds__(32 * (kMakers + 1)) k_sequential(const __grid_
 template <int Z, int M, bool SMEM>
 cudaError_t launch_k(const SeqArgs& a, unsigned words, size_t smem, cudaStream_t st) {
   auto kern = k_sequential<Z, M, SMEM>;
-  const cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the kernel's attribute, not the launch's: always the most, so that host
+  // threads on lattices of different sizes do not take it from each other
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMost);
   if (e != cudaSuccess) return e;
   kern<<<words, 32 * (kMakers + 1), smem, st>>>(a);
   return cudaGetLastError();
@@ -434,14 +436,14 @@ extern "C" ka_status ka_sweep_sequential(ka_ctx* c, int64_t nsweeps) {
   const size_t planes = smem ? (size_t)2 * c->N * sizeof(uint64_t) : 0;
   uint32_t H = kMaxStamps, log2H = 11;
   auto smem_for = [&](uint32_t words) { return planes + ring + (size_t)kMakers * 2 * words * 4; };
-  while (H > 32 && smem_for(H) > (size_t)227 * 1024) {
+  while (H > 32 && smem_for(H) > kSmemMost) {
     H >>= 1;
     --log2H;
   }
   a.hmask = H - 1;
   a.hshift = 32 - log2H;
   const size_t smem_bytes = smem_for(H);
-  if (smem_bytes > (size_t)227 * 1024) {
+  if (smem_bytes > kSmemMost) {
     if (prev >= 0) cudaSetDevice(prev);
     c->err = "sequential sweep: shared memory plan too large";
     return KA_EINVAL;
