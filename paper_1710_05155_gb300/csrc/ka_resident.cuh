@@ -37,6 +37,9 @@ namespace resident {
 constexpr size_t kSmemMax = 227 * 1024;
 constexpr int kMaxCluster = 8;  // the portable cluster size
 constexpr int64_t kMaxSweeps = 4096;  // sweeps per launch (a bound on one kernel's run time)
+#ifndef KA_WAIT_POLLS  // test builds: 0, so that every wait runs out
+#define KA_WAIT_POLLS (1 << 20)
+#endif
 
 // One word of one job: its plane base (element i of word h is n[i * stride]),
 // the sweeps to run (count of them from t_base), and for graphs the packed bonds.
@@ -124,8 +127,11 @@ __device__ __forceinline__ void bar_init(uint32_t bar, uint32_t count) {
 }
 
 // The end of a group (above).  bars: two mbarriers of this CTA, one arrival per
-// warp.  A wait that runs out marks the context's error word; the kernel then
-// runs to its end without further waits (its result is not valid).
+// warp.  A wait that runs out marks the context's error word (the result is not
+// valid) and the CTA goes on without waits to the end of the sweep, where it
+// leaves: no further, since nothing then bounds the bytes that an mbarrier has
+// yet to see (at most 2^20 - 1; a sweep's are 290 KB at most), and the others
+// then run out of their waits too.
 struct GroupEnd {
   uint32_t bars;
   uint32_t phase;  // groups done
@@ -144,7 +150,7 @@ struct GroupEnd {
   __device__ __forceinline__ void wait(int* err) {
     const uint32_t parity = (phase >> 1) & 1u;
     uint32_t done = 0;
-    for (int i = 0; i < (1 << 20) && !done && !dead; ++i)
+    for (int i = 0; i < KA_WAIT_POLLS && !done && !dead; ++i)
       asm volatile(
           "{\n.reg .pred q;\n"
           "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], %2;\n"

@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(1024) k_resident_cubic(const __grid_constant__
     // their own.  The last group's would meet the next sweep's first and the
     // final loop's reads, so the CTA meets here (us a sweep without and with:
     // L = 16 6.4, 6.4; L = 20 9.7, 9.8; d = 2, L = 128, 256 replicas 10.6, 10.9).
-    __syncthreads();
+    if (__syncthreads_or(ge.dead)) break;  // a wait ran out
   }
   store_plane(su, n, N, rank, C);
   if (fsmem)

@@ -180,6 +180,7 @@ __global__ void __launch_bounds__(1024) k_resident_graph(const __grid_constant__
         __syncthreads();
       }
     }
+    if (__syncthreads_or(ge.dead)) break;  // a wait ran out
   }
   store_plane(su, n, N, rank, C);
   for (int c = 0; c < nclass; ++c) {
