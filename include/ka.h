@@ -60,7 +60,7 @@
  *
  * Errors.  Every entry point returns a ka_status; no exception crosses the
  * ABI.  Kernel faults surface as KA_ECUDA at the next call that synchronises
- * (ka_observe, ka_get_state, ka_sync, ka_destroy).  ka_last_error gives a
+ * (ka_observe, ka_four_point, ka_get_state, ka_sync, ka_destroy).  ka_last_error gives a
  * message.  A context is not thread-safe; distinct contexts are independent.
  * All device work of a context is issued on its stream, in call order.
  */
@@ -79,7 +79,8 @@ typedef enum {
     KA_EINVAL = 1,   /* bad argument or unsupported parameter set */
     KA_ENOMEM = 2,   /* device or host allocation failed, or buffer too small */
     KA_ECUDA = 3,    /* CUDA runtime or kernel error */
-    KA_ETIMEOUT = 4, /* a bounded device wait ran out */
+    KA_ETIMEOUT = 4, /* a bounded device wait ran out: the context's state is not valid,
+                        and calls that use it return this, until ka_init or ka_set_state */
     KA_EBUSY = 5,    /* resource budget exhausted (admission refused) */
     KA_ESTATE = 6    /* call out of order (e.g. sweep before init) */
 } ka_status;

@@ -351,16 +351,15 @@ ka_status drain_profile(ka_ctx* c) {
   return KA_OK;
 }
 
-// KA_ETIMEOUT (and the word cleared) when a bounded wait ran out since the
-// last check: h is the device error word as just read.
+// KA_ETIMEOUT (and the word cleared, the state marked invalid) when a bounded
+// wait ran out since the last check: h is the device error word as just read.
 ka_status report_device_error(ka_ctx* c, int h) {
   if (!h) return KA_OK;
   cudaError_t e = cudaMemsetAsync(c->err_dev, 0, sizeof(int), c->stream);
   if (!e) e = cudaStreamSynchronize(c->stream);
   if (e) return cuda_fail(c, e, "sync");
-  return fail(c, KA_ETIMEOUT,
-              std::string("a bounded device wait ran out (code ") +
-                  std::to_string(h) + "); the state of this context is not valid");
+  c->timed_out = true;
+  return ka::valid_state(c, "");
 }
 
 // Read the device error word; synchronises the context stream.
@@ -399,6 +398,17 @@ resident::Unit resident_unit(const ka_ctx* c, int w, uint32_t t0, uint32_t count
   u.rk = c->rk;
   return u;
 }
+
+ka_status valid_state(ka_ctx* c, const char* what) {
+  if (c->timed_out)
+    return fail(c, KA_ETIMEOUT,
+                "a bounded device wait ran out; the state of this context is not valid until ka_init "
+                "or ka_set_state");
+  if (!c->initialized) return fail(c, KA_ESTATE, std::string(what) + " before init or set_state");
+  return KA_OK;
+}
+
+ka_status check_waits(ka_ctx* c) { return check_device_error(c); }
 
 ka_status create_context(const ka_params* params, void* buf, size_t bytes, bool owns, ka_ctx** out) {
   return create_common(params, buf, bytes, owns, out);
@@ -472,13 +482,14 @@ ka_status ka_init(ka_ctx* c, uint64_t seed, double rho) {
   c->K = K;
   c->sweep = 0;
   c->initialized = true;
+  c->timed_out = false;
   return KA_OK;
 }
 
 ka_status ka_sweep(ka_ctx* c, int64_t n) {
   ka::NvtxRange nvtx_range("ka_sweep");
   if (!c || n < 0) return c ? fail(c, KA_EINVAL, "n must be >= 0") : KA_EINVAL;
-  if (!c->initialized) return fail(c, KA_ESTATE, "sweep before init or set_state");
+  if (ka_status st = ka::valid_state(c, "sweep")) return st;
   if (c->sweep + n > ((int64_t)1 << 32)) return fail(c, KA_EINVAL, "sweep counter would pass 2^32");
   if (n == 0) return KA_OK;
   DeviceGuard dg(c->device);
@@ -489,6 +500,7 @@ ka_status ka_sweep(ka_ctx* c, int64_t n) {
                                  ? ka::resident::cubic_pays(c->d, c->L, c->pl.P, C, c->sms, n)
                                  : ka::resident::graph_pays(c->N, c->pl.W, C, c->sms, n));
   if (on_chip) {
+    c->waits = true;
     ka::resident::Args a{};
     a.plane_elems = c->pl.plane_elems();
     a.words_per_plane = c->pl.V;
@@ -565,7 +577,7 @@ ka_status ka_sweep(ka_ctx* c, int64_t n) {
 ka_status ka_observe_device(ka_ctx* c, int64_t* counts_device) {
   ka::NvtxRange nvtx_range("ka_observe");
   if (!c || !counts_device) return KA_EINVAL;
-  if (!c->initialized) return fail(c, KA_ESTATE, "observe before init or set_state");
+  if (ka_status st = ka::valid_state(c, "observe")) return st;
   DeviceGuard dg(c->device);
   cudaError_t e = ka::launch_observe(c->pl, (unsigned long long*)counts_device, c->stream);
   if (e) return cuda_fail(c, e, "observe");
@@ -575,7 +587,7 @@ ka_status ka_observe_device(ka_ctx* c, int64_t* counts_device) {
 ka_status ka_observe(ka_ctx* c, int64_t* sweep_out, int64_t* counts) {
   ka::NvtxRange nvtx_range("ka_observe");
   if (!c || !counts) return KA_EINVAL;
-  if (!c->initialized) return fail(c, KA_ESTATE, "observe before init or set_state");
+  if (ka_status st = ka::valid_state(c, "observe")) return st;
   DeviceGuard dg(c->device);
   cudaError_t e = ka::launch_observe(c->pl, c->counts_dev, c->stream);
   // counts and error word in one copy: each copy to pageable memory waits for
@@ -597,6 +609,7 @@ ka_status ka_observe(ka_ctx* c, int64_t* sweep_out, int64_t* counts) {
 ka_status ka_get_state(ka_ctx* c, uint64_t* n, uint64_t* n0, uint64_t* p) {
   ka::NvtxRange nvtx_range("ka_get_state");
   if (!c) return KA_EINVAL;
+  if (c->timed_out) return ka::valid_state(c, "get_state");
   DeviceGuard dg(c->device);
   const size_t bytes = (size_t)c->pl.P * c->pl.plane_elems() * sizeof(uint64_t);
   uint64_t* dst[3] = {n, n0, p};
@@ -651,6 +664,7 @@ ka_status set_state_impl(ka_ctx* c, const uint64_t* n, const uint64_t* n0, const
   c->rk = ka::round_keys(seed);
   c->K = -1;
   c->initialized = true;
+  c->timed_out = false;
   return KA_OK;
 }
 

@@ -35,6 +35,8 @@ struct ka_ctx {
   cudaEvent_t turn = nullptr;  // the fork, then the join, of a call
   ka::Topology host;  // class offsets (graphs) and tables for inspection
   bool initialized = false;
+  bool waits = false;      // sweeps of this context have run kernels with bounded waits
+  bool timed_out = false;  // a bounded wait ran out: the state is not valid until init or set_state
   int64_t sweep = 0, K = -1;
   uint64_t seed = 0;
   ka::RoundKeys rk{};
@@ -56,6 +58,12 @@ ka_status create_context(const ka_params* params, void* buf, size_t bytes, bool 
 // sweeps t0 .. t0 + count - 1.  Defined in ka_api.cu.
 int resident_cluster(const ka_ctx* c, int64_t words);
 resident::Unit resident_unit(const ka_ctx* c, int w, uint32_t t0, uint32_t count);
+// KA_OK if the context holds a valid state, else why not (also ka_last_error).
+// what: the call; defined in ka_api.cu.
+ka_status valid_state(ka_ctx* c, const char* what);
+// KA_ETIMEOUT if a bounded wait ran out (reads the device error word;
+// synchronises the context's stream); defined in ka_api.cu.
+ka_status check_waits(ka_ctx* c);
 // Device bytes a context needs; defined in ka_api.cu.
 ka_status context_bytes(const ka_params* params, size_t* bytes);
 }  // namespace ka

@@ -238,7 +238,7 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
   if (!phi || smax < 0) return four_point_fail(c, KA_EINVAL, "phi must be non-NULL, smax >= 0");
   if (c->topo != KA_CUBIC)
     return four_point_fail(c, KA_EINVAL, "four-point correlations need a cubic lattice");
-  if (!c->initialized) return four_point_fail(c, KA_ESTATE, "four-point before init or set_state");
+  if (ka_status st = valid_state(c, "four-point")) return st;
   const int d = c->d, L = c->L, half = L / 2;
   if ((int64_t)smax > (int64_t)d * half * half)
     return four_point_fail(c, KA_EINVAL, "smax above d (L/2)^2, the largest shell");
@@ -373,5 +373,5 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
   const cudaError_t es = cudaStreamSynchronize(st);
   if (!e) e = es;
   if (e) return four_point_fail(c, KA_ECUDA, std::string("four-point: ") + cudaGetErrorString(e));
-  return KA_OK;
+  return c->waits ? check_waits(c) : KA_OK;
 }

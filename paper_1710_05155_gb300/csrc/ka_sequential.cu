@@ -400,10 +400,7 @@ extern "C" ka_status ka_sweep_sequential(ka_ctx* c, int64_t nsweeps) {
   ka::NvtxRange nvtx_range("ka_sweep_sequential");
   using namespace ka;
   if (!c || nsweeps < 0) return KA_EINVAL;
-  if (!c->initialized) {
-    c->err = "sequential sweep before init or set_state";
-    return KA_ESTATE;
-  }
+  if (ka_status st = valid_state(c, "sequential sweep")) return st;
   if (c->sweep + nsweeps > ((int64_t)1 << 32)) {
     c->err = "sweep counter would pass 2^32";
     return KA_EINVAL;

@@ -49,3 +49,38 @@ with K.Simulation(**eval(sys.argv[1])) as sim:
 @pytest.mark.parametrize("params", PARAMS, ids=_name)
 def test_a_kernel_whose_wait_runs_out_leaves(library, params):
     variant.run(library, LEAVES, params)
+
+
+INVALID = """
+import torch, numpy as np, paper_1710_05155_gb300 as K
+def status(call, *args):
+    try:
+        call(*args)
+        return K.KA_OK
+    except K.KaError as e:
+        return e.status
+with K.Simulation(**eval(sys.argv[1])) as sim:
+    sim.init(17, 0.6)
+    state = sim.get_state()
+    counts = torch.empty((sim.info["replicas"], 4), dtype=torch.int64, device="cuda")
+    uses = [(sim.sweep, 1), (sim.observe,), (sim.get_state,), (sim.sweep_sequential, 1),
+            (K.ka_observe_device, sim.ctx, counts.data_ptr())]
+    if "L" in sys.argv[1]:
+        uses.append((sim.four_point, 1))
+    for valid in (lambda: sim.init(17, 0.6), lambda: sim.set_state(*state, 0, 17)):
+        sim.sweep(50)
+        assert status(K.ka_sync, sim.ctx) == K.KA_ETIMEOUT
+        for u in uses:
+            assert status(*u) == K.KA_ETIMEOUT, u
+        valid()
+        assert np.array_equal(sim.get_state()[0], state[0])
+        assert sim.observe()[0] == 0
+    if "L" in sys.argv[1]:
+        sim.sweep(50)
+        assert status(sim.four_point, 1) == K.KA_ETIMEOUT
+"""
+
+
+@pytest.mark.parametrize("params", [PARAMS[0], PARAMS[5]], ids=_name)
+def test_the_state_stays_invalid_until_it_is_set_again(library, params):
+    variant.run(library, INVALID, params)
