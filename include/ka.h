@@ -334,13 +334,17 @@ ka_status ka_job_bytes(const ka_params *params, const ka_job_spec *spec, size_t 
  * sweep count (absolute, >= the context's sweep); spec->seed and rho are not
  * used.  The context's stream is synchronised and replaced by the batch's,
  * and the first observation is recorded at the context's current sweep.
- * KA_EBUSY when over budget, KA_EINVAL for a context the batch cannot own;
+ * KA_EBUSY when over budget, KA_EINVAL for a context the batch cannot own,
+ * KA_ETIMEOUT for one whose state is not valid since a wait ran out;
  * on any error the context stays the caller's. */
 ka_status ka_batch_adopt(ka_batch *b, ka_ctx *ctx, const ka_job_spec *spec, int64_t *job_id);
 
 /* One round: advance every unfinished job by up to max_sweeps sweeps (a job
  * stops early at its next observation point or its target), then record
- * the due observations.  *sweeps_run = the round's length.  Synchronises. */
+ * the due observations.  *sweeps_run = the round's length.  Synchronises.
+ * KA_ETIMEOUT if a bounded device wait of a job ran out in the round: that job
+ * is finished (ka_batch_poll) and its state and observations are refused with
+ * KA_ETIMEOUT; the other jobs have run the round and go on with the next. */
 ka_status ka_batch_step(ka_batch *b, int64_t max_sweeps, int64_t *sweeps_run);
 
 /* Tune the live batch by timing real rounds, in two stages: (1) which cubic
@@ -366,14 +370,15 @@ ka_status ka_batch_poll(const ka_batch *b, int64_t job_id, int64_t *sweep, int32
 
 /* Observations of a job: *n_obs; if obs_sweeps / counts are non-NULL they
  * receive the sweep of each observation [n_obs] and the counts
- * [n_obs][R][4] (as ka_observe). */
+ * [n_obs][R][4] (as ka_observe).  KA_ETIMEOUT if a wait of the job ran out
+ * (ka_batch_step). */
 ka_status ka_batch_observations(const ka_batch *b, int64_t job_id, int64_t *n_obs,
                                 int64_t *obs_sweeps, int64_t *counts);
 
 /* State of a job (its current sweep: ka_batch_poll) copied to host arrays in
  * the canonical layout of ka_get_state, [R/64][N] uint64 each; any pointer
  * may be NULL.  Synchronises the batch stream.  KA_EINVAL for an unknown
- * job; the status of ka_get_state otherwise (a deferred device error of the
+ * job; KA_ETIMEOUT if a wait of the job ran out (ka_batch_step); the status of ka_get_state otherwise (a deferred device error of the
  * job's launches included). */
 ka_status ka_batch_state(ka_batch *b, int64_t job_id, uint64_t *n, uint64_t *n0, uint64_t *p);
 

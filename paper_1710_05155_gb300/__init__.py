@@ -419,11 +419,15 @@ class Batch:
         _check(load().ka_batch_poll(self.handle, job, C.byref(t), C.byref(f)), "ka_batch_poll")
         return t.value, bool(f.value)
 
-    def observations(self, job: int, replicas: int):
-        """(sweeps [n_obs], counts [n_obs, R, 4]) of a job."""
+    def observation_count(self, job: int) -> int:
         n = C.c_int64(0)
         _check(load().ka_batch_observations(self.handle, job, C.byref(n), None, None),
                "ka_batch_observations")
+        return n.value
+
+    def observations(self, job: int, replicas: int):
+        """(sweeps [n_obs], counts [n_obs, R, 4]) of a job."""
+        n = C.c_int64(self.observation_count(job))
         sw = np.zeros(n.value, np.int64)
         cnt = np.zeros((n.value, replicas, 4), np.int64)
         _check(load().ka_batch_observations(self.handle, job, C.byref(n), _ptr(sw), _ptr(cnt)),

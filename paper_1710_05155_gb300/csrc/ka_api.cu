@@ -186,6 +186,7 @@ ka_status create_common(const ka_params* params, void* buf, size_t bytes, bool o
   c->pl.P = s.P;
   c->pl.xs = s.xs;
   c->err_dev = (int*)(base + l.err);
+  c->wait_mark = c->err_dev;
   c->counts_dev = (unsigned long long*)(base + l.counts);
   c->stage = (s.V > 1 || s.xs || s.topo != KA_CUBIC) ? (uint64_t*)(base + l.stage) : nullptr;
   c->is.list = (uint32_t*)(base + l.list);
@@ -388,7 +389,7 @@ resident::Unit resident_unit(const ka_ctx* c, int w, uint32_t t0, uint32_t count
   u.rec = c->rec;
   u.bid = c->g.bid;
   u.coff = c->coff;
-  u.err = c->err_dev;
+  u.err = c->wait_mark;
   u.N = (int32_t)c->N;
   u.nclass = (int32_t)c->nclass;
   u.stride = c->pl.V;

@@ -36,6 +36,8 @@ struct Job {
   std::vector<int64_t> obs_t;
   bool finished = false;
   int64_t units = 0;    // its units in the tables
+  int* mark = nullptr;  // set by a kernel whose wait ran out (page-locked: read after a round's wait)
+  bool failed = false;  // it did: the job is finished, its state and observations are not valid
   bool batched = true;  // false: runs with its own (single-instance) launches inside each round
 };
 
@@ -113,6 +115,7 @@ struct ka_batch {
   std::vector<GraphClass> graph;
   std::vector<ResidentClass> resident;
   std::vector<void*> table_mem;  // device tables of the current job set
+  std::vector<int*> mark_mem, marks;  // page-locked blocks of the jobs' marks, those not in use
   bool own_stream = false;
   struct Side {
     cudaStream_t stream = nullptr;
@@ -160,6 +163,22 @@ cudaError_t dev_alloc(ka_batch* b, T** p, size_t count) {
   cudaError_t e = cudaMalloc((void**)p, count * sizeof(T));
   if (e == cudaSuccess) b->table_mem.push_back((void*)*p);
   return e;
+}
+
+// A job's mark, 0 (Job::mark).
+cudaError_t take_mark(ka_batch* b, int** mark) {
+  if (b->marks.empty()) {
+    constexpr int kBlock = 1024;
+    int* block = nullptr;
+    const cudaError_t e = cudaHostAlloc((void**)&block, kBlock * sizeof(int), cudaHostAllocMapped);
+    if (e) return e;
+    b->mark_mem.push_back(block);
+    for (int k = kBlock; k-- > 0;) b->marks.push_back(block + k);
+  }
+  *mark = b->marks.back();
+  **mark = 0;
+  b->marks.pop_back();
+  return cudaSuccess;
 }
 
 // Add a job's words to a class of on-chip units if its size runs there.
@@ -612,7 +631,18 @@ ka_status run_round(ka_batch* b, int64_t k_req, int64_t* ran) {
   }
   e = cudaStreamSynchronize(b->stream);
   if (e) return cuda_err(b, e, "round sync");
-  return KA_OK;
+  // a job whose wait ran out ends here; the others go on with the next round
+  ka_status st = KA_OK;
+  for (auto& kv : b->jobs) {
+    Job* j = kv.second;
+    if (j->failed || !*(volatile int*)j->mark) continue;
+    j->failed = true;
+    if (!j->finished && j->batched) b->idle_units += j->units;
+    j->finished = true;
+    b->err = "a bounded device wait of a job ran out; its state and observations are not valid";
+    st = KA_ETIMEOUT;
+  }
+  return st;
 }
 
 size_t obs_bytes(const ka_job_spec* spec, int64_t replicas) {
@@ -654,8 +684,15 @@ ka_status enrol(ka_batch* b, ka_ctx* ctx, const ka_job_spec* spec, int64_t* job_
   j->cap = spec->sweeps / spec->observe_every + 2;
   // small jobs share the batched launches (shares_launches)
   j->batched = shares_launches(b, ctx);
-  const ka_status st = observe_job(b, j);
+  ka_status st = observe_job(b, j);
+  if (!st) {
+    const cudaError_t e = take_mark(b, &j->mark);
+    void* at = nullptr;
+    if (e || cudaHostGetDevicePointer(&at, j->mark, 0)) st = KA_ENOMEM;
+    else ctx->wait_mark = (int*)at;
+  }
   if (st) {
+    if (j->mark) b->marks.push_back(j->mark);
     cudaFree(j->obs_dev);
     delete j;
     return st;
@@ -800,11 +837,13 @@ ka_status ka_batch_adopt(ka_batch* b, ka_ctx* ctx, const ka_job_spec* spec, int6
   if (!b || !ctx || !spec || spec->observe_every < 1) return KA_EINVAL;
   if (spec->sweeps < ctx->sweep || spec->sweeps >= ((int64_t)1 << 32)) return KA_EINVAL;
   if (!ctx->owns || ctx->device != b->device) return KA_EINVAL;
-  if (!ctx->initialized) return KA_ESTATE;
+  if (ka_status st = ka::valid_state(ctx, "adopt")) return st;
   if (b->used + ctx->bytes + obs_bytes(spec, ctx->R) > b->budget) return KA_EBUSY;
   DeviceScope scope(b->device);
   const cudaError_t e = cudaStreamSynchronize(ctx->stream);
   if (e) return cuda_err(b, e, "adopted context");
+  if (ctx->waits)
+    if (ka_status st = ka::check_waits(ctx)) return st;
   return enrol(b, ctx, spec, job_id);
 }
 
@@ -891,6 +930,7 @@ ka_status ka_batch_observations(const ka_batch* b, int64_t job_id, int64_t* n_ob
   auto it = b->jobs.find(job_id);
   if (it == b->jobs.end()) return KA_EINVAL;
   const Job* j = it->second;
+  if (j->failed) return KA_ETIMEOUT;
   if (n_obs) *n_obs = j->n_obs;
   if (obs_sweeps) std::memcpy(obs_sweeps, j->obs_t.data(), j->obs_t.size() * sizeof(int64_t));
   if (counts && j->n_obs > 0) {
@@ -907,6 +947,7 @@ ka_status ka_batch_state(ka_batch* b, int64_t job_id, uint64_t* n, uint64_t* n0,
   if (!b) return KA_EINVAL;
   auto it = b->jobs.find(job_id);
   if (it == b->jobs.end()) return KA_EINVAL;
+  if (it->second->failed) return KA_ETIMEOUT;
   DeviceScope scope(b->device);
   // the job's context runs on the batch stream: ka_get_state waits for it
   return ka_get_state(it->second->ctx, n, n0, p);
@@ -947,6 +988,7 @@ ka_status ka_batch_remove(ka_batch* b, int64_t job_id) {
   if (!j->finished) b->idle_units += in_tables;
   const ka_status st = ka_destroy(j->ctx);  // frees the context's buffer
   cudaFree(j->obs_dev);
+  b->marks.push_back(j->mark);
   b->used -= j->bytes;
   b->jobs.erase(it);
   delete j;
@@ -974,6 +1016,7 @@ ka_status ka_batch_destroy(ka_batch* b) {
     delete j;
   }
   free_tables(b);
+  for (int* block : b->mark_mem) cudaFreeHost(block);
   for (auto& x : b->side) {
     cudaStreamDestroy(x.stream);
     cudaEventDestroy(x.done);

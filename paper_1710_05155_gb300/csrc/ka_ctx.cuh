@@ -21,6 +21,7 @@ struct ka_ctx {
   ka::InitScratch is{};
   unsigned long long* counts_dev = nullptr;
   int* err_dev = nullptr;  // device error word of bounded device waits (0 = none), after the counts
+  int* wait_mark = nullptr;  // where kernels mark it: err_dev, or (jobs of a batch) the batch's word
   std::vector<int64_t> observed;  // host copy of the counts and that word
   uint64_t* stage = nullptr;
   ka::GraphDev g{};

@@ -49,7 +49,7 @@ struct Unit {
   const uint4* rec;      // graphs: per bond u, v and their other neighbours (16 bit each)
   const uint32_t* bid;   // graphs: canonical bond ids, class order
   const int32_t* coff;   // graphs: first bond of every class
-  int* err;              // set if a wait ran out (the context's device error word)
+  int* err;              // set if a wait ran out: device memory, or a batch's page-locked word
   int32_t N, nclass, stride;
   uint32_t t_base, count, word;
   RoundKeys rk;
@@ -160,7 +160,7 @@ struct GroupEnd {
           : "memory");
     if (!done && !dead) {
       dead = true;
-      atomicExch(err, 1);
+      *reinterpret_cast<volatile int*>(err) = 1;
     }
     ++phase;
   }

@@ -108,10 +108,32 @@ class DeviceBackend:
         return self.batch.info()["active"]
 
     def autotune(self) -> int:
-        return self.batch.autotune()
+        return self._round(self.batch.autotune)
 
     def step(self, k: int) -> int:
-        return self.batch.step(k)
+        return self._round(self.batch.step, k)
+
+    def _round(self, call, *args) -> int:
+        from . import KA_ETIMEOUT, KaError
+
+        try:
+            return call(*args)
+        except KaError as e:
+            if e.status != KA_ETIMEOUT:
+                raise
+            return 0  # a job's wait ran out: that job has ended (failure)
+
+    def failure(self, job_id: int) -> str:
+        """Why a finished job has no result ("" if it has one)."""
+        from . import KA_ETIMEOUT, KaError
+
+        try:
+            self.batch.observation_count(job_id)
+        except KaError as e:
+            if e.status != KA_ETIMEOUT:
+                raise
+            return str(e)
+        return ""
 
     def finished(self, job_id: int) -> bool:
         return self.batch.poll(job_id)[1]
@@ -215,7 +237,10 @@ class Server:
                     for jid in [j for j in running if be.finished(j)]:
                         r = running.pop(jid)
                         r.finished, r.status = now(), "done"
-                        if self.keep_results:
+                        r.error = be.failure(jid) if hasattr(be, "failure") else ""
+                        if r.error:  # its waits ran out: it fails alone
+                            r.status = "failed"
+                        elif self.keep_results:
                             r.sweeps, r.counts = be.observations(jid, r.job.params["replicas"])
                             if hasattr(be, "state"):
                                 r.state = be.state(jid, r.job)
