@@ -384,7 +384,8 @@ def run_rrg(dev: int, stream, sweeps: int) -> dict:
     ev1.record(stream)
     torch.cuda.synchronize(dev)
     packed_ms = ev0.elapsed_time(ev1)
-    packed_words, packed_planes = packed.info["plane_words"], packed.info["planes"]
+    packed_words = packed.info["plane_words"]
+    packed_sets = -(-packed.info["planes"] // packed.info["planes_per_launch"])  # launches per class
     packed.close()
     packed_value = RRG_N * 64 * len(RRG_RHOS) * sweeps / (packed_ms / 1000.0)
     launches = nclass * sweeps * len(RRG_RHOS)
@@ -395,7 +396,7 @@ def run_rrg(dev: int, stream, sweeps: int) -> dict:
     peak, peak_kind = _peaks()
     traffic = measured_traffic(PROFILE_GRAPH, SRC_GRAPH)
     # packed: one sweep moves all eight densities' words
-    p_launches = nclass * sweeps * packed_planes  # planes of this size run one by one
+    p_launches = nclass * sweeps * packed_sets
     p_achieved = bytes_per_sweep * len(RRG_RHOS) * sweeps / (packed_ms / 1000.0) / 1e9
     return {
         "metric": METRIC, "value": packed_value, "unit": UNIT,
@@ -604,11 +605,9 @@ def run_native(args, rank: int, world: int) -> None:
     counts_dev = [torch.zeros((R, 4), dtype=torch.int64, device=f"cuda:{dev}") for _ in sims]
     info = sims[0].info
     P, nq = info["planes"], info["planes_per_launch"]
-    # outside profiling the planes of a launch run as two chains of half as many
-    nq_run = max(1, nq // 2)
-    sets = -(-P // nq_run)  # launches per group and sweep
+    sets = -(-P // nq)  # launches per group and sweep
     sweep_launches_per_step = len(sims) * sets * S * GROUPS
-    launches_per_step = sweep_launches_per_step + len(sims)  # + one observation each
+    launches_per_step = sweep_launches_per_step + 2 * len(sims)  # + an observation each (and its clearing)
 
     def step():
         for sim, cd in zip(sims, counts_dev):
@@ -653,7 +652,7 @@ def run_native(args, rank: int, world: int) -> None:
     # one with events around each (ka_profile_read_dirs, by direction), give
     # each kernel's share of the region: k_rows runs the groups along x,
     # k_pencils those along y and z (two thirds of the launches).  A launch
-    # covers nq_run planes of one group: 32 bytes per site-word-sweep / 6 groups
+    # covers nq planes of one group: 32 bytes per site-word-sweep / 6 groups
     # (two chains run side by side: the average time is the region's share).
     iso_ms, iso_n = np.zeros(4), np.zeros(4, np.int64)
     for sim in sims:
@@ -666,7 +665,7 @@ def run_native(args, rank: int, world: int) -> None:
     region_launches = sweep_launches_per_step * args.steps
     pencil_launches = region_launches * 2 // 3
     row_launches = region_launches - pencil_launches
-    bytes_per_launch = BYTES_PER_SITE_WORD_SWEEP * N_SITES * nq_run / GROUPS
+    bytes_per_launch = BYTES_PER_SITE_WORD_SWEEP * N_SITES * nq / GROUPS
     pencil_ms = _apportion(local_ms, iso_ms, (1, 2), pencil_launches)
     row_ms = _apportion(local_ms, iso_ms, (0,), row_launches)
     achieved = bytes_per_launch / (pencil_ms / 1000.0) / 1e9
@@ -745,7 +744,7 @@ def run_native(args, rank: int, world: int) -> None:
             achieved=achieved, peak=peak, peak_kind=peak_kind, traffic=traffic,
             pencil_ms=pencil_ms, pencil_iso_ms=float(iso_ms[1:3].sum() / iso_n[1:3].sum()),
             row_ms=row_ms, row_iso_ms=float(iso_ms[0] / iso_n[0]),
-            bytes_per_launch=bytes_per_launch, nq=nq_run, path_achieved=path_achieved,
+            bytes_per_launch=bytes_per_launch, nq=nq, path_achieved=path_achieved,
             cpu=extra.pop("cpu_baseline", None), e2e_value=e2e_value, h2d=h2d, d2h=d2h,
             gpu_launches=launches_per_step * args.steps, clocks=clk, extra=extra)
         print(json.dumps(line), flush=True)

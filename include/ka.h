@@ -134,9 +134,12 @@ typedef struct {
     size_t device_bytes;  /* device memory the context uses */
     int32_t planes;       /* device state planes per array */
     int32_t plane_words;  /* words per site in one plane */
-    int32_t planes_per_launch; /* planes one sweep launch covers (cubic group
-                                  launches per class group and sweep:
-                                  ceil(planes / planes_per_launch)) */
+    int32_t planes_per_launch; /* planes that the launch of a group (lattices) or
+                                  class (graphs) covers, so that a sweep takes
+                                  ceil(planes / planes_per_launch) launches of each.
+                                  Profiled sweeps may put more in a launch; sweeps
+                                  that stay on chip (small topologies, by the number
+                                  of sweeps in the call) are one launch per call */
 } ka_info_t;
 
 /* Device bytes ka_create_in needs for these parameters. */

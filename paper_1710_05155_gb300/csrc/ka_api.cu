@@ -517,8 +517,11 @@ ka_status ka_sweep(ka_ctx* c, int64_t n) {
   } else if (c->pencil && ka::stream_supported(c->d, c->L)) {
     // Plane groups run chain by chain, all sweeps of a group before the
     // chain's next: the planes in flight stay resident in the L2.
-    int per = ka::stream_planes_per_launch(c->L, c->pl.P);
-    const int chains = c->side && !c->prof ? ka::stream_chains(c->L, c->pl.P, &per) : 1;
+    int per = 0, chains = ka::stream_chains(c->L, c->pl.P, &per);
+    if (c->prof) {
+      chains = 1;
+      per = ka::stream_planes_per_launch(c->L, c->pl.P);
+    }
     if (chains > 1) {
       e = cudaEventRecord(c->turn, c->stream);
       if (!e) e = cudaStreamWaitEvent(c->side, c->turn, 0);
@@ -710,9 +713,9 @@ ka_status ka_info(const ka_ctx* c, ka_info_t* out) {
   out->device_bytes = c->bytes;
   out->planes = c->pl.P;
   out->plane_words = c->pl.V;
-  out->planes_per_launch =
-      (c->pencil && ka::stream_supported(c->d, c->L)) ? ka::stream_planes_per_launch(c->L, c->pl.P)
-                                                                : 1;
+  int per = c->pencil ? 1 : graph_planes_per_launch(c);
+  if (c->pencil && ka::stream_supported(c->d, c->L)) ka::stream_chains(c->L, c->pl.P, &per);
+  out->planes_per_launch = per;
   return KA_OK;
 }
 
