@@ -202,8 +202,9 @@ ka_status ka_observe_device(ka_ctx *ctx, int64_t *counts_device);
  * phi: host int64 [R][smax + 1], required; psi: host int64 [smax + 1] or
  * NULL.  0 <= smax <= d (L/2)^2 and at most 65536 displacement vectors with
  * |delta|^2 <= smax, else KA_EINVAL; KA_EINVAL on graphs, KA_ESTATE before
- * init.  Uses stream-ordered scratch memory on the context's device,
- * released before return; synchronises the stream. */
+ * init.  Uses the context's staging plane or stream-ordered scratch memory on
+ * its device (up to 256 MB, less where that is not to be had), released before
+ * return; synchronises the stream. */
 ka_status ka_four_point(ka_ctx *ctx, int32_t smax, int64_t *phi, int64_t *psi);
 
 /* Copy the state to host arrays in canonical layout [R/64][N] uint64 each

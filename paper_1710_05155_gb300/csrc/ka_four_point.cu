@@ -42,7 +42,8 @@ constexpr int kSegment = 15;          // vectors per segment: 240 words per thre
 constexpr int kThreads = 256;
 constexpr int kMaxVectors = 1 << 16;  // displacement vectors per call
 // Scratch when the context's staging plane does not hold one word's padded
-// lattice: this much, or one word's, a slab of layers at a time.
+// lattice: this much, or one word's, a slab of layers at a time; less where the
+// device has not that much left.
 constexpr size_t kArena = (size_t)256 << 20;
 
 constexpr int64_t kMostPadded = (int64_t)1 << 29;  // elements: 32-bit byte offsets
@@ -324,10 +325,32 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
     if (layer * (zc + 2 * rad) >= kMostPadded)
       return four_point_fail(c, KA_ENOMEM, "scratch: a padded layer is too large");
     words = (int)std::max<size_t>(1, std::min<size_t>((size_t)W, kArena / q_bytes(zc)));
-    const size_t total = fixed + m_bytes(zc) + (size_t)words * q_bytes(zc);
-    const cudaError_t ea = cudaMallocAsync((void**)&own, total, st);
+    auto take = [&]() {
+      const cudaError_t ea = cudaMallocAsync((void**)&own, fixed + m_bytes(zc) + (size_t)words * q_bytes(zc), st);
+      if (ea) {
+        own = nullptr;
+        cudaGetLastError();
+      }
+      return ea;
+    };
+    cudaError_t ea = take();
+    if (ea) {
+      // a full device: the thickest slab that the staging plane holds, else
+      // ever thinner ones in less memory (down to (L + 2 rad)^(d - 1) (2 rad + 1)
+      // words, 0.7 MB at L = 64, rad = 5)
+      words = 1;
+      int64_t in_stage = std::min<int64_t>(L, zc);
+      while (in_stage && fixed + m_bytes(in_stage) + q_bytes(in_stage) > stage_bytes) --in_stage;
+      if (in_stage) {
+        zc = in_stage;
+        mem = (char*)c->stage;
+        ea = cudaSuccess;
+      } else {
+        for (ea = take(); ea && zc > 1; ea = take()) zc /= 2;
+      }
+    }
     if (ea) return four_point_fail(c, KA_ENOMEM, std::string("scratch: ") + cudaGetErrorString(ea));
-    mem = own;
+    if (own) mem = own;
   }
   unsigned long long* phi_dev = (unsigned long long*)mem;
   unsigned long long* psi_dev = (unsigned long long*)(mem + up(phi_bytes));
