@@ -688,8 +688,12 @@ ka_status enrol(ka_batch* b, ka_ctx* ctx, const ka_job_spec* spec, int64_t* job_
   if (!st) {
     const cudaError_t e = take_mark(b, &j->mark);
     void* at = nullptr;
-    if (e || cudaHostGetDevicePointer(&at, j->mark, 0)) st = KA_ENOMEM;
-    else ctx->wait_mark = (int*)at;
+    if (e || cudaHostGetDevicePointer(&at, j->mark, 0)) {
+      cudaGetLastError();
+      st = KA_ENOMEM;
+    } else {
+      ctx->wait_mark = (int*)at;
+    }
   }
   if (st) {
     if (j->mark) b->marks.push_back(j->mark);

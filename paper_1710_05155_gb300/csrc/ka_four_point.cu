@@ -339,8 +339,11 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
       // ever thinner ones in less memory (down to (L + 2 rad)^(d - 1) (2 rad + 1)
       // words, 0.7 MB at L = 64, rad = 5)
       words = 1;
-      int64_t in_stage = std::min<int64_t>(L, zc);
-      while (in_stage && fixed + m_bytes(in_stage) + q_bytes(in_stage) > stage_bytes) --in_stage;
+      int64_t in_stage = 0, above = std::min<int64_t>(L, zc) + 1;
+      while (above - in_stage > 1) {
+        const int64_t mid = (in_stage + above) / 2;
+        (fixed + m_bytes(mid) + q_bytes(mid) <= stage_bytes ? in_stage : above) = mid;
+      }
       if (in_stage) {
         zc = in_stage;
         mem = (char*)c->stage;
