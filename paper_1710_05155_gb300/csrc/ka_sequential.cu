@@ -47,6 +47,9 @@ constexpr int kSmemWords = 20480;  // n and p of up to 10240 sites in shared mem
 constexpr size_t kSmemMost = (size_t)227 * 1024;  // shared memory of a CTA
 constexpr int kMakers = 7;         // warps that prepare attempts
 constexpr uint32_t kMaxStamps = 2048;  // words of one of a maker's two stamp tables, at most
+constexpr uint32_t kSharedStamps = 512;  // at least, where more CTAs are to share an SM
+constexpr size_t kSmSmem = (size_t)228 * 1024;  // shared memory of an SM (1 KB of it per CTA)
+constexpr size_t kSmCtas = 2048 / (32 * (kMakers + 1));  // CTAs by threads
 
 struct SeqArgs {
   uint64_t* n;
@@ -431,12 +434,27 @@ extern "C" ka_status ka_sweep_sequential(ka_ctx* c, int64_t nsweeps) {
   // stamp tables in what the planes (if in shared memory) and the ring leave
   const size_t ring = (size_t)kMakers * 32 * (3 * 4 * (smem ? c->z + 1 : 2 * c->z + 1) + 2 * 8);
   const size_t planes = smem ? (size_t)2 * c->N * sizeof(uint64_t) : 0;
-  uint32_t H = kMaxStamps, log2H = 11;
-  auto smem_for = [&](uint32_t words) { return planes + ring + (size_t)kMakers * 2 * words * 4; };
-  while (H > 32 && smem_for(H) > kSmemMost) {
-    H >>= 1;
-    --log2H;
+  uint32_t H = kMaxStamps;
+  auto smem_for = [&](uint32_t stamps) { return planes + ring + (size_t)kMakers * 2 * stamps * 4; };
+  // no more stamps than sites (a power of two), nor than there is room for
+  if (smem)
+    while (H > 32 && H >= 2 * (uint64_t)c->N) H >>= 1;
+  while (H > 32 && smem_for(H) > kSmemMost) H >>= 1;
+  // Words beyond what runs at once take turns: the most stamps, but no fewer than
+  // kSharedStamps (false conflicts), of those with the fewest turns.  us a sweep
+  // with always 2048 stamps and so: 1024 words of L = 4 27.0, 8.7; of L = 8 78.0,
+  // 38.2; 800 of L = 12 166, 97 (one warp a word, many to an SM: 16.4, 53.3, 139).
+  if (smem) {
+    auto turns = [&](uint32_t stamps) {
+      const size_t per_sm = std::min<size_t>(kSmCtas, kSmSmem / (smem_for(stamps) + 1024));
+      const size_t at_once = std::max<size_t>(1, per_sm * (size_t)std::max(0, c->sms));
+      return (words + at_once - 1) / at_once;
+    };
+    for (uint32_t h = H / 2; h >= kSharedStamps; h /= 2)
+      if (turns(h) < turns(H)) H = h;
   }
+  uint32_t log2H = 0;
+  while ((1u << log2H) < H) ++log2H;
   a.hmask = H - 1;
   a.hshift = 32 - log2H;
   const size_t smem_bytes = smem_for(H);

@@ -1,0 +1,47 @@
+"""Random-sequential sweeps of more words than the device has SMs.
+
+Results at both sides of the rule for the stamp tables, against the oracle on the
+first and last words.  And the time: one warp per word (many to an SM) took as
+long at 1024 words of L = 8 as 4.6 times what 152 words take now, so no more.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+import paper_1710_05155_gb300 as K
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d,L,W", [(3, 4, 160), (3, 8, 200), (3, 12, 152), (3, 12, 160), (2, 44, 160), (2, 48, 160),
+                                   (3, 16, 160)])
+def test_words(d, L, W):
+    topo, m, sweeps = O.cubic(d, L), d, 2
+    with K.Simulation(topo=K.KA_CUBIC, d=d, L=L, m=m, replicas=64 * W) as sim:
+        sim.init(17, 0.6)
+        sim.sweep_sequential(sweeps)
+        n, _, p = sim.get_state()
+    for w in (0, W - 1):
+        st = O.init(topo.N, 64, 17, 0.6, r0=64 * w)
+        O.sequential_sweeps(topo, m, st, 17, sweeps)
+        assert np.array_equal(n[w], O.pack_words(st.n)[0]) and np.array_equal(p[w], O.pack_words(st.p)[0]), w
+
+
+def test_time():
+    import torch
+
+    def least(W):
+        with K.Simulation(topo=K.KA_CUBIC, d=3, L=8, m=3, replicas=64 * W) as sim:
+            sim.init(1, 0.7)
+            sim.sweep_sequential(20)
+            times = []
+            for _ in range(5):
+                begin, end = torch.cuda.Event(True), torch.cuda.Event(True)
+                begin.record()
+                sim.sweep_sequential(20)
+                end.record()
+                torch.cuda.synchronize()
+                times.append(begin.elapsed_time(end))
+            return min(times)
+
+    assert least(1024) < 4.6 * least(152)
