@@ -14,7 +14,7 @@
 // weight 2.  q (and M) are first written as words in site order with a margin
 // of the largest component on every side, filled periodically: site i + delta
 // is then a fixed offset from i for all sites, and neighbouring threads read
-// neighbouring words.  A thread takes eight sites and, shell by shell, adds
+// neighbouring words.  A thread takes sixteen sites and, shell by shell, adds
 // q_i & q_{i + delta} for all of them into bit-sliced counters, eight words at
 // a time (ka_count.cuh); a block sums a shell's counters in shared memory and
 // adds 64 integers to phi.  One launch covers all shells; small lattices
@@ -24,8 +24,9 @@
 // adders 5, the AND 2, the load and its address 2, the sums over lanes the
 // rest).  L = 64, 256 replicas, smax = 25 (515 vectors), the whole call: 4.56 ms
 // before, when each shell was a launch and a thread worked out periodic
-// coordinates for each vector; 0.50 ms now.
+// coordinates for each vector; 0.35 ms now.
 #include <algorithm>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -46,6 +47,12 @@ constexpr int kMaxVectors = 1 << 16;  // displacement vectors per call
 // device has not that much left.
 constexpr size_t kArena = (size_t)256 << 20;
 
+// Passes over the words in the staging plane before an allocation is made: one
+// takes 150 us, a pass over a small lattice 15 (L = 8, 4096 replicas, smax = 6:
+// 64 passes 1530 us, one 220).
+constexpr int kMostPasses = 8;
+constexpr size_t kSmallResult = (size_t)64 << 10;  // bytes that are cheaper to copy twice on the host
+
 constexpr int64_t kMostPadded = (int64_t)1 << 29;  // elements: 32-bit byte offsets
 
 // Vectors of one shell and weight: offsets [first, first + count).
@@ -62,33 +69,37 @@ struct Slab {
   int64_t sites;     // sites of the slab
 };
 
+// Sites (below 2^31) and padded elements (below kMostPadded) in 32 bits: a thread
+// divides for each of its sites (one block of k_phi took 17 us with 64).
 // storage position of the site that padded element k shows
-__device__ __forceinline__ int64_t shown(const Slab& g, int xs, int64_t k) {
-  int64_t site = 0, stride = 1;
+__device__ __forceinline__ uint32_t shown(const Slab& g, int xs, uint32_t k) {
+  uint32_t site = 0, stride = 1;
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
     if (m < g.d) {
-      const int64_t extent = m == g.d - 1 ? g.zc + 2 * g.rad : g.L + 2 * g.rad;
-      int64_t x = k % extent - g.rad + (m == g.d - 1 ? g.z0 : 0);
+      const uint32_t extent = (uint32_t)(m == g.d - 1 ? g.zc + 2 * g.rad : g.L + 2 * g.rad);
+      int64_t x = (int64_t)(k % extent) - g.rad + (m == g.d - 1 ? g.z0 : 0);
       k /= extent;
       x += x < 0 ? g.L : 0;
       x -= x >= g.L ? g.L : 0;
-      site += x * stride;
-      stride *= g.L;
+      site += (uint32_t)x * stride;
+      stride *= (uint32_t)g.L;
     }
   }
-  return dev_site(xs, site);
+  if (!xs) return site;
+  const uint32_t x = site % (uint32_t)xs;  // dev_site
+  return site - x + (x & 1u) * ((uint32_t)xs >> 1) + (x >> 1);
 }
 
 // padded element of the slab's site k
-__device__ __forceinline__ int64_t centre(const Slab& g, int64_t k) {
-  int64_t e = 0;
+__device__ __forceinline__ uint32_t centre(const Slab& g, uint32_t k) {
+  uint32_t e = 0;
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
     if (m < g.d) {
-      const int64_t x = m == g.d - 1 ? k : k % g.L;
-      if (m < g.d - 1) k /= g.L;
-      e += (x + g.rad) * g.ps[m];
+      const uint32_t q = m == g.d - 1 ? 0 : k / (uint32_t)g.L, x = k - q * (uint32_t)g.L;
+      k = q;
+      e += (x + (uint32_t)g.rad) * (uint32_t)g.ps[m];
     }
   }
   return e;
@@ -101,7 +112,7 @@ __global__ void __launch_bounds__(kThreads) k_pad(const __grid_constant__ Planes
   const int64_t k = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   if (k >= g.padded) return;
   const int w = w0 + (int)blockIdx.y;
-  const size_t e = (size_t)(w / pl.V) * pl.plane_elems() + (size_t)shown(g, pl.xs, k) * pl.V + w % pl.V;
+  const size_t e = (size_t)(w / pl.V) * pl.plane_elems() + (size_t)shown(g, pl.xs, (uint32_t)k) * pl.V + w % pl.V;
   out[(size_t)blockIdx.y * g.padded + k] = pl.n[e] & pl.n0[e];
 }
 
@@ -111,11 +122,13 @@ __global__ void __launch_bounds__(kThreads) k_pad_counts(const __grid_constant__
                                                          uint32_t* __restrict__ M) {
   const int64_t k = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   if (k >= g.padded) return;
-  const size_t at = (size_t)shown(g, pl.xs, k) * pl.V;
+  const size_t at = (size_t)shown(g, pl.xs, (uint32_t)k) * pl.V;
+  const int lv = pl.V == 4 ? 2 : pl.V == 2 ? 1 : 0;
   uint32_t m = 0;
-  for (int w = 0; w < pl.W; ++w) {
-    const size_t e = (size_t)(w / pl.V) * pl.plane_elems() + at + w % pl.V;
-    m += (uint32_t)__popcll(pl.n[e] & pl.n0[e]);
+#pragma unroll 8
+  for (int w = 0; w < pl.W; ++w) {  // eight words' loads at once
+    const size_t e = (size_t)(w >> lv) * pl.plane_elems() + at + (w & (pl.V - 1));
+    m += (uint32_t)__popcll(__ldg(pl.n + e) & __ldg(pl.n0 + e));
   }
   M[k] = m;
 }
@@ -135,7 +148,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_phi(const __grid_constant__ Sla
   for (int u = 0; u < kSites; ++u) {
     const int64_t s = s0 + u * kThreads;
     const bool in = s < g.sites;
-    at[u] = 8u * (uint32_t)centre(g, in ? s : 0);
+    at[u] = 8u * centre(g, in ? (uint32_t)s : 0u);
     own[u] = in ? *reinterpret_cast<const uint64_t*>(reinterpret_cast<const char*>(q) + at[u]) : 0ull;
   }
   const int b0 = (int)((int64_t)nseg * blockIdx.z / gridDim.z);
@@ -187,7 +200,7 @@ __global__ void __launch_bounds__(kThreads) k_psi(const __grid_constant__ Slab g
   for (int u = 0; u < kPsiSites; ++u) {
     const int64_t s = s0 + u * kThreads;
     const bool in = s < g.sites;
-    at[u] = (int32_t)centre(g, in ? s : 0);
+    at[u] = (int32_t)centre(g, in ? (uint32_t)s : 0u);
     own[u] = in ? M[at[u]] : 0u;
   }
   const int b0 = (int)((int64_t)nseg * blockIdx.z / gridDim.z);
@@ -317,9 +330,10 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
   int words = 0;  // per pass
   char* own = nullptr;
   char* mem = nullptr;
-  if (layer * (L + 2 * rad) < kMostPadded && stage_bytes >= fixed + m_bytes(L) + q_bytes(L)) {
-    mem = (char*)c->stage;
+  if (layer * (L + 2 * rad) < kMostPadded && stage_bytes >= fixed + m_bytes(L) + q_bytes(L))
     words = (int)std::min<size_t>((size_t)W, (stage_bytes - fixed - m_bytes(L)) / q_bytes(L));
+  if (words && (W + words - 1) / words <= kMostPasses) {
+    mem = (char*)c->stage;
   } else {
     if (layer * (zc + 2 * rad) > most) zc = std::max<int64_t>(1, most / layer - 2 * rad);
     if (layer * (zc + 2 * rad) >= kMostPadded)
@@ -362,8 +376,11 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
   uint32_t* M = (uint32_t*)(mem + fixed);
   uint64_t* q = (uint64_t*)(mem + fixed + m_bytes(zc));
   cudaError_t e = cudaMemsetAsync(mem, 0, up(phi_bytes) + up(psi_bytes), st);
-  if (!e) e = cudaMemcpyAsync(seg_dev, segs.data(), seg_bytes, cudaMemcpyHostToDevice, st);
-  if (!e) e = cudaMemcpyAsync(off_dev, offsets.data(), off_bytes, cudaMemcpyHostToDevice, st);
+  // both tables in one copy, and below both results: a copy takes about 8 us
+  std::vector<char> tables(up(seg_bytes) + off_bytes);
+  std::memcpy(tables.data(), segs.data(), seg_bytes);
+  std::memcpy(tables.data() + up(seg_bytes), offsets.data(), off_bytes);
+  if (!e) e = cudaMemcpyAsync(seg_dev, tables.data(), tables.size(), cudaMemcpyHostToDevice, st);
   const Planes& pl = c->pl;
   // blocks along z share out the segments until the grid has four blocks per SM
   auto split = [&](int64_t blocks) {
@@ -390,8 +407,13 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
       e = cudaGetLastError();
     }
   }
-  if (!e) e = cudaMemcpyAsync(phi, phi_dev, phi_bytes, cudaMemcpyDeviceToHost, st);
-  if (!e && psi) e = cudaMemcpyAsync(psi, psi_dev, psi_bytes, cudaMemcpyDeviceToHost, st);
+  std::vector<char> both(psi && up(phi_bytes) + psi_bytes <= kSmallResult ? up(phi_bytes) + psi_bytes : 0);
+  if (!both.empty()) {
+    if (!e) e = cudaMemcpyAsync(both.data(), mem, both.size(), cudaMemcpyDeviceToHost, st);
+  } else {
+    if (!e) e = cudaMemcpyAsync(phi, phi_dev, phi_bytes, cudaMemcpyDeviceToHost, st);
+    if (!e && psi) e = cudaMemcpyAsync(psi, psi_dev, psi_bytes, cudaMemcpyDeviceToHost, st);
+  }
   if (own) {
     const cudaError_t ef = cudaFreeAsync(own, st);
     if (!e) e = ef;
@@ -399,5 +421,9 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
   const cudaError_t es = cudaStreamSynchronize(st);
   if (!e) e = es;
   if (e) return four_point_fail(c, KA_ECUDA, std::string("four-point: ") + cudaGetErrorString(e));
+  if (!both.empty()) {
+    std::memcpy(phi, both.data(), phi_bytes);
+    std::memcpy(psi, both.data() + up(phi_bytes), psi_bytes);
+  }
   return c->waits ? check_waits(c) : KA_OK;
 }
