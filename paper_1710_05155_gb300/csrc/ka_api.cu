@@ -595,16 +595,25 @@ ka_status ka_observe(ka_ctx* c, int64_t* sweep_out, int64_t* counts) {
   DeviceGuard dg(c->device);
   cudaError_t e = ka::launch_observe(c->pl, c->counts_dev, c->stream);
   // counts and error word in one copy: each copy to pageable memory waits for
-  // the stream (10 sweeps and an observation at L = 16: 109 us with two)
+  // the stream (10 sweeps and an observation at L = 16: 109 us with two, 98
+  // with one); but many counts cost more to copy again on the host (65536
+  // replicas: 189 us with one, 84 with two)
   const size_t bytes = (size_t)c->R * 4 * sizeof(int64_t);
-  c->observed.resize((size_t)c->R * 4 + 1);
-  if (!e) e = cudaMemcpyAsync(c->observed.data(), c->counts_dev, bytes + sizeof(int32_t),
-                              cudaMemcpyDeviceToHost, c->stream);
+  int32_t timed_out = 0;
+  if (c->R <= 4096) {
+    c->observed.resize((size_t)c->R * 4 + 1);
+    if (!e) e = cudaMemcpyAsync(c->observed.data(), c->counts_dev, bytes + sizeof(timed_out),
+                                cudaMemcpyDeviceToHost, c->stream);
+  } else {
+    if (!e) e = cudaMemcpyAsync(counts, c->counts_dev, bytes, cudaMemcpyDeviceToHost, c->stream);
+    if (!e) e = cudaMemcpyAsync(&timed_out, c->err_dev, sizeof(timed_out), cudaMemcpyDeviceToHost, c->stream);
+  }
   if (!e) e = cudaStreamSynchronize(c->stream);
   if (e) return cuda_fail(c, e, "observe");
-  std::memcpy(counts, c->observed.data(), bytes);
-  int32_t timed_out = 0;
-  std::memcpy(&timed_out, c->observed.data() + (size_t)c->R * 4, sizeof(timed_out));
+  if (c->R <= 4096) {
+    std::memcpy(counts, c->observed.data(), bytes);
+    std::memcpy(&timed_out, c->observed.data() + (size_t)c->R * 4, sizeof(timed_out));
+  }
   if (ka_status st = report_device_error(c, timed_out)) return st;
   if (sweep_out) *sweep_out = c->sweep;
   return KA_OK;

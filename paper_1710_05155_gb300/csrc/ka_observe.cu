@@ -40,7 +40,7 @@ namespace {
 // binary digits of a thread's counters: up to 120 words, or (small planes) 8
 constexpr int kDigits = 7, kFewDigits = 4;
 constexpr int kPerThread = 120, kFew = 8;
-constexpr size_t kOneBlock = 8192;  // words of a plane that one block takes
+constexpr size_t kOneBlock = 2048;  // words of a plane that one block takes
 
 // ALL: the four observables; else only the particles
 template <int V, bool ALL, int S>
@@ -136,7 +136,8 @@ cudaError_t launch_counts(const Planes& pl, unsigned long long* counts_dev, cuda
   const size_t wave = (size_t)256 * 2 * (size_t)(sms > 0 ? sms : 148);
   size_t per_thread = (E * (size_t)pl.P + wave - 1) / wave;
   // a small plane is one block's, which stores its counts: no clearing launch
-  // before (1 us; 16 more words a thread take a fraction of that)
+  // before (us of ka_observe, one block and several: 1728 words 19.4, -; 4096
+  // 27.9, 22.5; 8000 28.2, 22.2)
   if (E <= kOneBlock) per_thread = std::max(per_thread, (E + 255) / 256);
   per_thread = std::min<size_t>((per_thread + 3) / 4 * 4, kPerThread);
   const size_t per_block = 256 * per_thread;
