@@ -499,7 +499,7 @@ ka_status ka_sweep(ka_ctx* c, int64_t n) {
   const int C = c->prof ? 0 : ka::resident_cluster(c, c->pl.W);
   const bool on_chip = C && (c->topo == KA_CUBIC
                                  ? ka::resident::cubic_pays(c->d, c->L, c->pl.P, C, c->sms, n)
-                                 : ka::resident::graph_pays(c->N, c->pl.W, C, c->sms, n));
+                                 : ka::resident::graph_pays(c->N, c->z, c->nclass, c->pl.W, C, c->sms, n));
   if (on_chip) {
     c->waits = true;
     ka::resident::Args a{};

@@ -87,7 +87,7 @@ cudaError_t launch_cubic(const Args& a, int d, int L, int m, unsigned words, int
 // whether a graph of N sites may run here, and its CTAs per word (0: it does not)
 bool graph_fits(int64_t N);
 int graph_cluster(int64_t N, int64_t nbonds, int64_t class_max);
-bool graph_pays(int64_t N, int64_t words, int C, int sms, int64_t n);
+bool graph_pays(int64_t N, int z, int64_t nclass, int64_t words, int C, int sms, int64_t n);
 // the packed record of every bond, from tables in storage positions
 int graph_record_bytes(int z);
 void graph_records(int64_t N, int z, const int32_t* nbr, const int32_t* bu, const int32_t* bv,

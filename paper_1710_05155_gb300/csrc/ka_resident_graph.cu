@@ -285,13 +285,21 @@ int graph_cluster(int64_t N, int64_t nbonds, int64_t class_max) {
   return 0;
 }
 
-bool graph_pays(int64_t N, int64_t words, int C, int sms, int64_t n) {
-  // us of a sweep (above): 28 with a launch per class, whatever the words up to
-  // a few hundred thousand site-words, then with them; on chip 12 + 0.0012 N for
-  // as many words as run at once, and 12 for the launch
-  const double group = 28.0 + 2.0e-5 * (double)N * (double)words;
+bool graph_pays(int64_t N, int z, int64_t nclass, int64_t words, int C, int sms, int64_t n) {
+  // us, fitted.  A launch per class 1.75 (z = 1 to 4 1.65 to 1.85), then with the
+  // site-words.  On chip, a class of b bonds: one CTA 0.5 (b = 16), 0.55 (200),
+  // 1.0 (512); four CTAs 1.4 (1024), 1.6 (1300), 2.0 (2000); a quarter more with
+  // 32-byte records; for as many words as run at once.  The launch, the planes and
+  // the records: one CTA 7 (64 sites), 13 (1000), 32 (4096), four CTAs 12 to 20.
+  // Calls of one sweep and of 20, launches / on chip: z = 1, 64 sites 4.1, 34 / 7.5,
+  // 17; z = 2, 10 000 sites 10, 168 / 22, 210; z = 4, 4096 sites 29, 590 / 48, 360.
+  const double b = 0.5 * (double)N * (double)z / (double)nclass;
+  const bool one = C == 1;
+  const double group = 1.75 * (double)nclass + 2.0e-5 * (double)N * (double)words;
+  const double chip = (double)nclass * (one ? 0.45 + 1.1e-3 * b : 0.75 + 0.62e-3 * b) * (z > 4 ? 1.25 : 1.0);
+  const double launch = one ? 7.0 + 6.0e-3 * (double)N : 10.0 + 1.0e-3 * (double)N;
   const double waves = (double)((words * C + sms - 1) / (sms > 0 ? sms : 1));
-  return group * (double)n > (12.0 + (12.0 + 1.2e-3 * (double)N) * (double)n) * waves;
+  return group * (double)n > (launch + chip * (double)n) * waves;
 }
 
 cudaError_t launch_graph(const Args& args, int64_t Nmax, int64_t bonds_max, int64_t class_max, int z,
