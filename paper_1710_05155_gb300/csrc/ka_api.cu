@@ -518,7 +518,10 @@ ka_status ka_sweep(ka_ctx* c, int64_t n) {
     // Plane groups run chain by chain, all sweeps of a group before the
     // chain's next: the planes in flight stay resident in the L2.
     int per = 0, chains = ka::stream_chains(c->L, c->pl.P, &per);
-    if (c->prof) {
+    // one chain while profiling, and where a single sweep gains less than the
+    // fork and the join cost (6 us; one sweep of L = 80, 3 planes 36 us in one
+    // chain, 42 in two; 4 planes 48, 45)
+    if (c->prof || (n == 1 && c->N * c->pl.P < 2000000)) {
       chains = 1;
       per = ka::stream_planes_per_launch(c->L, c->pl.P);
     }

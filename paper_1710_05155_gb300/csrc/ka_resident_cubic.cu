@@ -32,17 +32,20 @@ int cubic_cluster(int d, int L, int64_t words, int sms) {
 bool cubic_pays(int d, int L, int64_t planes, int C, int sms, int64_t n) {
   // us of a sweep, measured and fitted.  On chip: d = 3, L = 8 to 28 4.5, 5.2,
   // 6.4, 9.7, 14.8, 22.3; d = 2, L = 16, 64, 128 2.5, 3.6, 10.6; d = 4, L = 8, 12 10.8, 34;
-  // for as many words as run at once.  A launch per group: 10 (L <= 16) to 15 for
-  // up to four planes of a three-dimensional lattice; 12 and 18 to 22 for every
-  // plane of the others.  A launch on chip (planes in and out, the cluster) costs 12
-  // us more: single sweeps of L = 16 10.6, on chip 16.4.
+  // for as many words as run at once.  A launch per group: 10 (L <= 16; 12 for
+  // two planes and more) to 15 for up to four planes of a three-dimensional
+  // lattice; 12 and 18 to 22 for every plane of the others.  A launch on chip
+  // (planes in and out, the cluster) costs 12 us more, small lattices 8 to 10:
+  // calls of 1, 2 and 3 sweeps of L = 16, 3 planes 12.4, 25, 37 in groups, on chip
+  // 18, -, 30; L = 12 13, 25, 37, on chip -, 19, 24.
   double N = 1.0;
   for (int k = 0; k < d; ++k) N *= L;
-  const double group = d == 3 ? (L <= 16 ? 10.2 : 14.0) * (double)((planes + 3) / 4)
+  const double group = d == 3 ? (L > 16 ? 14.0 : planes > 1 ? 12.2 : 10.2) * (double)((planes + 3) / 4)
                               : (d == 2 ? 12.0 : 18.0) * (double)planes;
   const double chip = d == 3 ? 3.0 + 8.8e-4 * N : d == 2 ? 2.5 + 5.0e-4 * N : 5.0 + 1.4e-3 * N;
   const double waves = (double)((planes * C + sms - 1) / (sms > 0 ? sms : 1));
-  return group * (double)n > (12.0 + chip * (double)n) * waves;
+  const double launch = d == 3 && N < 4000.0 ? 8.0 + 1.0e-3 * N : 12.0;
+  return group * (double)n > (launch + chip * (double)n) * waves;
 }
 
 cudaError_t launch_cubic(const Args& a, int d, int L, int m, unsigned words, int C,
