@@ -25,9 +25,9 @@
 // read; attempts applied in one round touch disjoint sites.
 //
 // The chain's rounds are one warp's latency; all that does not depend on the
-// state -- the draws, the sites, who conflicts with whom -- is prepared by kMakers
+// state -- the draws, the sites, who conflicts with whom -- is prepared by seven
 // other warps of the CTA, a batch of 32 attempts each, while the chain's warp
-// applies the kMakers batches before (in turn; one warp doing both took 4500
+// applies the seven batches before (in turn; one warp doing both took 4500
 // cycles a batch, most of them for the preparation).  A maker finds the
 // conflicts by stamps: every attempt sets its lane bit in a word of a table
 // for both sites of W, then ORs the words over R.  Sites share words of a
@@ -45,11 +45,11 @@ namespace {
 constexpr uint32_t kTagSequential = 0xFFFFFFFCu;
 constexpr int kSmemWords = 20480;  // n and p of up to 10240 sites in shared memory
 constexpr size_t kSmemMost = (size_t)227 * 1024;  // shared memory of a CTA
-constexpr int kMakers = 7;         // warps that prepare attempts
+constexpr int kMakers = 7;         // warps that prepare attempts, or
+constexpr int kFewMakers = 3;      // with more words than run at once
 constexpr uint32_t kMaxStamps = 2048;  // words of one of a maker's two stamp tables, at most
-constexpr uint32_t kSharedStamps = 512;  // at least, where more CTAs are to share an SM
 constexpr size_t kSmSmem = (size_t)228 * 1024;  // shared memory of an SM (1 KB of it per CTA)
-constexpr size_t kSmCtas = 2048 / (32 * (kMakers + 1));  // CTAs by threads
+constexpr int kSmThreads = 2048;
 
 struct SeqArgs {
   uint64_t* n;
@@ -170,10 +170,11 @@ __global__ void __launch_bounds__(32 * (kMakers + 1)) k_sequential(const __grid_
     p = sm + a.N;
   }
   const int z = Z ? Z : a.z, fields = SMEM ? z + 1 : 2 * z + 1;
-  uint32_t* ring = reinterpret_cast<uint32_t*>(sm + (SMEM ? 2 * a.N : 0));  // [3][kMakers][fields][32]
-  uint64_t* swaps = reinterpret_cast<uint64_t*>(ring + 3 * kMakers * fields * 32);  // [2][kMakers][32]
-  uint32_t* stamps = reinterpret_cast<uint32_t*>(swaps + 2 * kMakers * 32);  // [kMakers][2][hmask + 1]
-  for (uint32_t b = threadIdx.x; b < 2 * kMakers * (a.hmask + 1); b += blockDim.x) stamps[b] = 0;
+  const uint32_t makers = blockDim.x / 32 - 1;
+  uint32_t* ring = reinterpret_cast<uint32_t*>(sm + (SMEM ? 2 * a.N : 0));  // [3][makers][fields][32]
+  uint64_t* swaps = reinterpret_cast<uint64_t*>(ring + 3 * makers * fields * 32);  // [2][makers][32]
+  uint32_t* stamps = reinterpret_cast<uint32_t*>(swaps + 2 * makers * 32);  // [makers][2][hmask + 1]
+  for (uint32_t b = threadIdx.x; b < 2 * makers * (a.hmask + 1); b += blockDim.x) stamps[b] = 0;
   const uint32_t per_sweep = (uint32_t)((a.N + 31) / 32), batches = per_sweep * (uint32_t)a.nsweeps;
   const uint64_t range = (uint64_t)a.N * (uint64_t)z;
   const uint32_t earlier = (1u << lane) - 1u;  // lanes of the earlier attempts
@@ -321,22 +322,22 @@ __global__ void __launch_bounds__(32 * (kMakers + 1)) k_sequential(const __grid_
     }
   };
 
-  // turn t: the makers prepare batches t kMakers .., warp 0 applies those of
+  // turn t: the makers prepare batches t makers .., warp 0 applies those of
   // turn t - 1, the makers clear p for those of turn t - 2
-  const uint32_t turns = (batches + kMakers - 1) / kMakers + 2;
+  const uint32_t turns = (batches + makers - 1) / makers + 2;
   const int batch_words = fields * 32;
   __syncthreads();
   for (uint32_t t = 0; t < turns; ++t) {
     if (warp > 0) {
-      const uint32_t m = (uint32_t)warp - 1, b = t * kMakers + m;
-      uint32_t* slot = ring + ((t % 3) * kMakers + m) * batch_words;
+      const uint32_t m = (uint32_t)warp - 1, b = t * makers + m;
+      uint32_t* slot = ring + ((t % 3) * makers + m) * batch_words;
       if (b < batches) make(b, slot, stamps + (size_t)m * 2 * (a.hmask + 1));
-      if (SMEM && t >= 2 && b - 2 * kMakers < batches)
-        clear(ring + (((t + 1) % 3) * kMakers + m) * batch_words, swaps + ((t & 1) * kMakers + m) * 32);
+      if (SMEM && t >= 2 && b - 2 * makers < batches)
+        clear(ring + (((t + 1) % 3) * makers + m) * batch_words, swaps + ((t & 1) * makers + m) * 32);
     } else if (t > 0) {
-      const uint32_t b0 = (t - 1) * kMakers, count = b0 < batches ? min(batches - b0, (uint32_t)kMakers) : 0u;
-      const uint32_t* in = ring + ((t + 2) % 3) * kMakers * batch_words;
-      uint64_t* swap_out = swaps + ((t + 1) & 1) * kMakers * 32;
+      const uint32_t b0 = (t - 1) * makers, count = b0 < batches ? min(batches - b0, makers) : 0u;
+      const uint32_t* in = ring + ((t + 2) % 3) * makers * batch_words;
+      uint64_t* swap_out = swaps + ((t + 1) & 1) * makers * 32;
       for (uint32_t m = 0; m < count; ++m) {
         take(in + m * batch_words);
         apply(swap_out + m * 32);
@@ -354,22 +355,22 @@ __global__ void __launch_bounds__(32 * (kMakers + 1)) k_sequential(const __grid_
 }
 
 template <int Z, int M, bool SMEM>
-cudaError_t launch_k(const SeqArgs& a, unsigned words, size_t smem, cudaStream_t st) {
+cudaError_t launch_k(const SeqArgs& a, unsigned words, int makers, size_t smem, cudaStream_t st) {
   auto kern = k_sequential<Z, M, SMEM>;
   // the kernel's attribute, not the launch's: always the most, so that host
   // threads on lattices of different sizes do not take it from each other
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMost);
   if (e != cudaSuccess) return e;
-  kern<<<words, 32 * (kMakers + 1), smem, st>>>(a);
+  kern<<<words, 32 * (makers + 1), smem, st>>>(a);
   return cudaGetLastError();
 }
 
 template <int Z, bool SMEM>
-cudaError_t launch_m(const SeqArgs& a, int m, unsigned words, size_t smem, cudaStream_t st) {
+cudaError_t launch_m(const SeqArgs& a, int m, unsigned words, int makers, size_t smem, cudaStream_t st) {
   switch (m < 7 ? m : 7) {
 #define KA_CASE(MM) \
   case MM:          \
-    return launch_k<Z, (Z == 0 || MM < Z ? MM : 0), SMEM>(a, words, smem, st);
+    return launch_k<Z, (Z == 0 || MM < Z ? MM : 0), SMEM>(a, words, makers, smem, st);
     KA_CASE(0)
     KA_CASE(1)
     KA_CASE(2)
@@ -385,15 +386,15 @@ cudaError_t launch_m(const SeqArgs& a, int m, unsigned words, size_t smem, cudaS
 }
 
 template <bool SMEM>
-cudaError_t launch_z(const SeqArgs& a, int m, unsigned words, size_t smem, cudaStream_t st) {
+cudaError_t launch_z(const SeqArgs& a, int m, unsigned words, int makers, size_t smem, cudaStream_t st) {
   // instances of their own where the loop over the neighbours costs time; with
   // the planes in global memory they were slower (L = 32: 1.67 ms a sweep, all
   // loads at once, against 1.15)
   if constexpr (SMEM) {
-    if (a.z == 4) return launch_m<4, SMEM>(a, m, words, smem, st);
-    if (a.z == 6) return launch_m<6, SMEM>(a, m, words, smem, st);
+    if (a.z == 4) return launch_m<4, SMEM>(a, m, words, makers, smem, st);
+    if (a.z == 6) return launch_m<6, SMEM>(a, m, words, makers, smem, st);
   }
-  return launch_m<0, SMEM>(a, m, words, smem, st);
+  return launch_m<0, SMEM>(a, m, words, makers, smem, st);
 }
 
 }  // namespace
@@ -432,32 +433,48 @@ extern "C" ka_status ka_sweep_sequential(ka_ctx* c, int64_t nsweeps) {
   const unsigned words = (unsigned)(c->R / 64);
   const bool smem = 2 * c->N <= kSmemWords;
   // stamp tables in what the planes (if in shared memory) and the ring leave
-  const size_t ring = (size_t)kMakers * 32 * (3 * 4 * (smem ? c->z + 1 : 2 * c->z + 1) + 2 * 8);
   const size_t planes = smem ? (size_t)2 * c->N * sizeof(uint64_t) : 0;
+  auto smem_for = [&](int makers, uint32_t stamps) {
+    const size_t ring = (size_t)32 * (3 * 4 * (smem ? c->z + 1 : 2 * c->z + 1) + 2 * 8);
+    return planes + (size_t)makers * (ring + 2 * (size_t)stamps * 4);
+  };
+  int makers = kMakers;
   uint32_t H = kMaxStamps;
-  auto smem_for = [&](uint32_t stamps) { return planes + ring + (size_t)kMakers * 2 * stamps * 4; };
   // no more stamps than sites (a power of two), nor than there is room for
   if (smem)
     while (H > 32 && H >= 2 * (uint64_t)c->N) H >>= 1;
-  while (H > 32 && smem_for(H) > kSmemMost) H >>= 1;
-  // Words beyond what runs at once take turns: the most stamps, but no fewer than
-  // kSharedStamps (false conflicts), of those with the fewest turns.  us a sweep
-  // with always 2048 stamps and so: 1024 words of L = 4 27.0, 8.7; of L = 8 78.0,
-  // 38.2; 800 of L = 12 166, 97 (one warp a word, many to an SM: 16.4, 53.3, 139).
+  while (H > 32 && smem_for(makers, H) > kSmemMost) H >>= 1;
+  // Words beyond what runs at once take turns: of seven makers and three, and of the
+  // stamps down to 128 to 512 by the sites an attempt reads (fewer, more false
+  // conflicts), the most with the fewest turns; but three makers where three or
+  // more CTAs would share an SM anyway, whose warps then wait for each other.
+  // us a sweep with seven makers and 2048 stamps whatever the words, and so: 1024
+  // words of L = 4 27, 6.0; of L = 8 78, 22; 800 of L = 12 166, 74; 1024 of d = 1,
+  // L = 64 8.0, 4.7 (one warp a word, many to an SM: 17, 54, 142, 4.8).
   if (smem) {
-    auto turns = [&](uint32_t stamps) {
-      const size_t per_sm = std::min<size_t>(kSmCtas, kSmSmem / (smem_for(stamps) + 1024));
-      const size_t at_once = std::max<size_t>(1, per_sm * (size_t)std::max(0, c->sms));
+    auto per_sm = [&](int mk, uint32_t stamps) {
+      return std::min<size_t>(kSmThreads / (32 * (mk + 1)), kSmSmem / (smem_for(mk, stamps) + 1024));
+    };
+    auto turns = [&](int mk, uint32_t stamps) {
+      const size_t at_once = std::max<size_t>(1, per_sm(mk, stamps) * (size_t)std::max(0, c->sms));
       return (words + at_once - 1) / at_once;
     };
-    for (uint32_t h = H / 2; h >= kSharedStamps; h /= 2)
-      if (turns(h) < turns(H)) H = h;
+    const uint32_t most = H, least = c->z <= 2 ? 128 : c->z <= 4 ? 256 : 512;
+    for (int mk : {kMakers, kFewMakers})
+      for (uint32_t h = most; h == most || h >= least; h /= 2) {
+        const size_t t = turns(mk, h), best = turns(makers, H);
+        const bool crowded = mk < makers && (int)words > 2 * c->sms && per_sm(makers, H) >= 3;
+        if (t < best || (t == best && crowded)) {
+          makers = mk;
+          H = h;
+        }
+      }
   }
   uint32_t log2H = 0;
   while ((1u << log2H) < H) ++log2H;
   a.hmask = H - 1;
   a.hshift = 32 - log2H;
-  const size_t smem_bytes = smem_for(H);
+  const size_t smem_bytes = smem_for(makers, H);
   if (smem_bytes > kSmemMost) {
     if (prev >= 0) cudaSetDevice(prev);
     c->err = "sequential sweep: shared memory plan too large";
@@ -469,8 +486,8 @@ extern "C" ka_status ka_sweep_sequential(ka_ctx* c, int64_t nsweeps) {
   for (int64_t done = 0; done < nsweeps && !e; done += chunk) {
     a.t0 = (uint32_t)(c->sweep + done);
     a.nsweeps = (int)std::min<int64_t>(chunk, nsweeps - done);
-    e = smem ? launch_z<true>(a, c->m, words, smem_bytes, c->stream)
-             : launch_z<false>(a, c->m, words, smem_bytes, c->stream);
+    e = smem ? launch_z<true>(a, c->m, words, makers, smem_bytes, c->stream)
+             : launch_z<false>(a, c->m, words, makers, smem_bytes, c->stream);
   }
   if (prev >= 0) cudaSetDevice(prev);
   if (e) {

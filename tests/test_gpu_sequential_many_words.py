@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("d,L,W", [(3, 4, 160), (3, 8, 200), (3, 12, 152), (3, 12, 160), (2, 44, 160), (2, 48, 160),
-                                   (3, 16, 160)])
+                                   (3, 16, 160), (1, 4, 1024), (1, 1024, 800), (2, 16, 800), (3, 4, 500), (4, 4, 500)])
 def test_words(d, L, W):
     topo, m, sweeps = O.cubic(d, L), d, 2
     with K.Simulation(topo=K.KA_CUBIC, d=d, L=L, m=m, replicas=64 * W) as sim:
