@@ -51,6 +51,7 @@ constexpr size_t kArena = (size_t)256 << 20;
 // takes 150 us, a pass over a small lattice 15 (L = 8, 4096 replicas, smax = 6:
 // 64 passes 1530 us, one 220).
 constexpr int kMostPasses = 8;
+constexpr size_t kSmallScratch = (size_t)8 << 20;
 constexpr size_t kSmallResult = (size_t)64 << 10;  // bytes that are cheaper to copy twice on the host
 
 constexpr int64_t kMostPadded = (int64_t)1 << 29;  // elements: 32-bit byte offsets
@@ -329,6 +330,7 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
   int64_t zc = L;
   int words = 0;  // per pass
   char* own = nullptr;
+  size_t own_bytes = 0;
   char* mem = nullptr;
   if (layer * (L + 2 * rad) < kMostPadded && stage_bytes >= fixed + m_bytes(L) + q_bytes(L))
     words = (int)std::min<size_t>((size_t)W, (stage_bytes - fixed - m_bytes(L)) / q_bytes(L));
@@ -340,7 +342,8 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
       return four_point_fail(c, KA_ENOMEM, "scratch: a padded layer is too large");
     words = (int)std::max<size_t>(1, std::min<size_t>((size_t)W, kArena / q_bytes(zc)));
     auto take = [&]() {
-      const cudaError_t ea = cudaMallocAsync((void**)&own, fixed + m_bytes(zc) + (size_t)words * q_bytes(zc), st);
+      own_bytes = fixed + m_bytes(zc) + (size_t)words * q_bytes(zc);
+      const cudaError_t ea = cudaMallocAsync((void**)&own, own_bytes, st);
       if (ea) {
         own = nullptr;
         cudaGetLastError();
@@ -414,12 +417,14 @@ extern "C" ka_status ka_four_point(ka_ctx* c, int32_t smax, int64_t* phi, int64_
     if (!e) e = cudaMemcpyAsync(phi, phi_dev, phi_bytes, cudaMemcpyDeviceToHost, st);
     if (!e && psi) e = cudaMemcpyAsync(psi, psi_dev, psi_bytes, cudaMemcpyDeviceToHost, st);
   }
-  if (own) {
-    const cudaError_t ef = cudaFreeAsync(own, st);
-    if (!e) e = ef;
-  }
+  // A free before the wait gives the memory back to the device in the wait,
+  // which takes 130 us; a small block is freed after it, so that the pool keeps
+  // it until the next wait and the next call finds it there.
+  cudaError_t ef = own && own_bytes > kSmallScratch ? cudaFreeAsync(own, st) : cudaSuccess;
   const cudaError_t es = cudaStreamSynchronize(st);
+  if (own && own_bytes <= kSmallScratch) ef = cudaFreeAsync(own, st);
   if (!e) e = es;
+  if (!e) e = ef;
   if (e) return four_point_fail(c, KA_ECUDA, std::string("four-point: ") + cudaGetErrorString(e));
   if (!both.empty()) {
     std::memcpy(phi, both.data(), phi_bytes);
