@@ -127,9 +127,12 @@ typedef struct {
     uint64_t seed;      /* dynamics seed */
     int32_t kernel;     /* 0 = cubic pencil kernels, 1 = edge-gather kernel,
                            3 = group kernels of three-dimensional lattices (d = 3,
-                           L % 4 == 0, L <= 128: reported from two planes up and,
-                           for one plane, at the sides that first had them; the
-                           other one-plane sides, reported as 0, run them too) */
+                           L % 4 == 0, L <= 128).  Fourteen sides with one plane
+                           (20, 24, 28, 36, 40, 44, 52, 56, 60, 68, 72, 76, 100,
+                           108) run the group kernels too but are reported as 0,
+                           as they were before they did.  Small topologies, whose
+                           sweeps may stay on chip, are reported by the kernels of
+                           their launches per group or class */
     int32_t rrg_attempts; /* configuration-model attempts (KA_RRG) */
     size_t device_bytes;  /* device memory the context uses */
     int32_t planes;       /* device state planes per array */
@@ -172,10 +175,10 @@ ka_status ka_sweep(ka_ctx *ctx, int64_t n);
  * key = the dynamics seed, draw = 0, 1, ... until accepted, and takes site
  * i = r / z and its neighbour in slot r mod z (on cubic lattices slot 2 mu is
  * the up and 2 mu + 1 the down neighbour along mu; on graphs the slots are
- * the neighbour row in ascending order, as ka_graph_tables returns it).  One CTA per word runs
- * the chain, 32 attempts at a time, applying together the attempts that do
- * not touch each other's sites (the result is the in-order chain's), in
- * shared memory when the lattice has at most 10240 sites.  Advances the sweep
+ * the neighbour row in ascending order, as ka_graph_tables returns it).  One
+ * CTA per word runs the chain, 32 attempts at a time, applying together the
+ * attempts that do not touch each other's sites (the result is the in-order
+ * chain's), in shared memory when the lattice has at most 10240 sites.  Advances the sweep
  * counter; no synchronisation.  KA_ESTATE before init, KA_EINVAL if
  * N z >= 2^32. */
 ka_status ka_sweep_sequential(ka_ctx *ctx, int64_t n);
@@ -291,7 +294,9 @@ ka_status ka_destroy(ka_ctx *ctx);
  * group of every three-dimensional job of the same side and m (the group
  * kernels, one table entry per job plane), or of every other small cubic
  * job of the same shape class (d, words per plane, m), and one launch runs
- * a colour class of every graph job of the same (words per plane, m).  A
+ * a colour class of every graph job of the same (words per plane, m) and of a
+ * size within a factor of two.  Jobs on small topologies stay on chip: one
+ * launch runs the whole round of all those of a shape.  A
  * cubic job whose groups have at least the batch's own-launch threshold of
  * tiles (ka_batch_tuning; ka_batch_autotune sets it) runs with its own
  * launches inside each round.  Each job's result is bit-identical to running it alone:

@@ -1,4 +1,4 @@
-// ka_cubic_stream_l64.cu -- instances of the streaming group kernel for L = 64
+// ka_cubic_stream_l64.cu -- instances of the group kernels for L = 64
 // (one translation unit per side, so that they compile in parallel).
 #define KA_STREAM_INSTANCES
 #include "ka_cubic_stream.cuh"

@@ -1,4 +1,4 @@
-// ka_cubic_stream_s1.cu -- instances of the group kernels' general form for the
+// ka_cubic_stream_s1.cu -- instances of the group kernels for the
 // sides 20, 24, 28, 36 (a few sides per translation unit, so that the
 // instances compile in parallel).
 #define KA_STREAM_INSTANCES

@@ -1,4 +1,4 @@
-// ka_cubic_stream_s6.cu -- instances of the group kernels' general form for the
+// ka_cubic_stream_s6.cu -- instances of the group kernels for the
 // sides 108, 112, 116, 120 (a few sides per translation unit, so that the
 // instances compile in parallel).
 #define KA_STREAM_INSTANCES

@@ -1,5 +1,5 @@
-// ka_cubic_stream_s7.cu -- instances of the group kernels' general form for the
-// sides 124 (a few sides per translation unit, so that the
+// ka_cubic_stream_s7.cu -- instances of the group kernels for the
+// side 124 (a few sides per translation unit, so that the
 // instances compile in parallel).
 #define KA_STREAM_INSTANCES
 #include "ka_cubic_stream.cuh"

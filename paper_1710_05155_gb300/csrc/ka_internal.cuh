@@ -2,9 +2,10 @@
 //
 // Device layout of one state plane set (n, n0, p): P = W / V planes, each
 // [N][V] uint64, W = R / 64 words per site.  Word w of site i lives in plane
-// w / V at element i * V + w % V.  Cubic lattices on the pencil kernel use
-// V = 4 (one 32-byte sector per site) when 4 divides W; otherwise V = 2 for
-// even W, else 1.
+// w / V at element i * V + w % V.  Cubic lattices of dimension 2 and more on
+// the pencil kernels, the group kernels and on chip have V = 1; graphs, d = 1
+// and the edge-gather path V = 4 (one 32-byte sector per site) when 4 divides
+// W, otherwise V = 2 for even W, else 1.
 #pragma once
 
 #include <nvtx3/nvToolsExt.h>
