@@ -829,10 +829,7 @@ ka_status ka_batch_add(ka_batch* b, const ka_params* params, const ka_job_spec* 
   }
   ka_ctx* ctx = nullptr;
   st = ka::create_context(&prm, buf, bytes, true, &ctx);
-  if (st) {
-    cudaFree(buf);
-    return st;
-  }
+  if (st) return st;  // the buffer is freed
   st = ka_init(ctx, spec->seed, spec->rho);
   if (!st) st = enrol(b, ctx, spec, job_id);
   if (st) ka_destroy(ctx);
